@@ -390,7 +390,7 @@ extern "C" int vie_tucker_cp(vie_op* op, int rank, double tol, int max_iter, uns
     set_error("tol must be >= 0 and max_iter in [1, 100000]");
     return VIE_ERR_ARG;
   }
-  if (op->oct32 == nullptr) {
+  if (op->oct32 == nullptr || !lane_fft_edge(op->P[2])) {
     set_error("Tucker+CP needs the rebuild scratch (grid edge P3 = 32 R with a four-step or "
               "register FFT)");
     return VIE_ERR_ARG;

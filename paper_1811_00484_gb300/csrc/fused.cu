@@ -147,20 +147,6 @@ __global__ void __launch_bounds__(256, 3) fused_z_kernel(const FusedArgs<T> a) {
   }
 }
 
-// Register-resident variant for P3 = 32 R: one CTA of four warps per (k1, k2)
-// mirror group, see fused_warp_group.
-// Resident CTAs per SM the register budget is sized for (up to radix 4: 96
-// registers, five CTAs of four warps; radix 5-6: 128; radix 8: 168).
-__host__ __device__ constexpr int fused_min_blocks(int R) {
-  return R <= 4 ? 5 : (R <= 6 ? 4 : (R <= 8 ? 3 : 2));
-}
-
-template <int R, bool STORED>
-__global__ void __launch_bounds__(128, fused_min_blocks(R)) fused_warp_kernel(const FusedArgs<float> a) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  fused_warp_group<R, STORED>(a, a.g0 + blockIdx.x, reinterpret_cast<float2*>(smem_raw));
-}
-
 // Rebuild of the half fibres of eq. (13) for k1 in [k1a, k1a + gridDim.y), every
 // k2 and k3 <= P3/2, into out[k1 - k1a][k2][c][k3]:
 //   W_c[k2, q]      = sum_b U2_c[k2, b] S_c[k1][b, q]          (S = slab core)
@@ -641,94 +627,30 @@ __global__ void __launch_bounds__(kTcThreads, 1) octant_cp_kernel(const OctCpArg
 
 int launch_octant_args(const vie_op* op, int k1a, cudaStream_t s, bool cp);
 
-// Four-step variant (fused_fs_group) for P3 = 8 V, V = 4 R with R even.
-__host__ __device__ constexpr int fused_fs_min_blocks(int V) { return V <= 8 ? 8 : (V <= 16 ? 5 : 4); }
-
-template <int V, bool STORED>
-__global__ void __launch_bounds__(96, fused_fs_min_blocks(V)) fused_fs_kernel(const FusedArgs<float> a) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  fused_fs_group<V, STORED>(a, a.g0 + blockIdx.x, reinterpret_cast<float2*>(smem_raw));
-}
-
-template <int R, bool STORED>
-static void launch_fused_warp_r(FusedArgs<float> a, cudaStream_t s) {
-  const size_t smem = fused_warp_smem(R, a.H3, a.r2max, a.r3max);
-  const int fam = STORED ? PF_FUSED_STORED : PF_FUSED_TUCKER;
+// FP32 z stage of a planned edge (planfft.cuh), or of length 512 with rebuilt or
+// stored half fibres (tp512.cu: 12.4 ms per eight 256^3 right-hand sides, 15.5 ms
+// for the planned 8 x 8 x 8).  False: no such kernel for this edge.
+static bool launch_fused_fast(FusedArgs<float> a, cudaStream_t s) {
+  if (!plan_exists(a.P3)) return false;
+  const int fam = a.spec != nullptr ? PF_FUSED_STORED : PF_FUSED_TUCKER;
   a.prof = prof_bytes(fam);
-  a.prof_rhs_bytes = 12ull * a.comp_stride * sizeof(float2);     // 48 B per padded voxel
-  a.prof_launch_bytes = STORED ? 6ull * a.spec_stride * sizeof(float2) : 0ull;
-  // the four-step kernel when R is even (and, on the Tucker path, the half
-  // fibres come from the rebuild scratch)
-  constexpr bool kFs = (R == 2 || R == 4 || R == 6);
-  const bool fs = kFs && (STORED || a.octant != nullptr);
-  const size_t fs_smem = fused_fs_smem(4 * R, a.H3);
-  // P3 = 512: the three-pass radix-8 kernel (tp512.cu); P3 = 128: radix 8, 4, 4 (t128.cu)
-  const bool tp = (R == 16) && fused_tp_supported(a, STORED);
-  const bool t128 = (R == 4) && fused_t128_supported(a, STORED);
-  if (STORED || a.octant == nullptr) {
+  const bool tp = fused_tp_supported(a);
+  auto launch = [&](int k1a, int nk1) {
     ProfScope ps(fam, s);
-    a.g0 = 0;
-    if (tp) {
-      launch_fused_tp(a, a.H1 * a.H2, STORED, s);
-      return;
-    }
-    if (t128) {
-      launch_fused_t128(a, a.H1 * a.H2, STORED, s);
-      return;
-    }
-    if constexpr (kFs) {
-      if (fs) {
-        launch_pdl(fused_fs_kernel<4 * R, STORED>, dim3(a.H1 * a.H2), dim3(96), fs_smem, s, a);
-        return;
-      }
-    }
-    launch_pdl(fused_warp_kernel<R, STORED>, dim3(a.H1 * a.H2), dim3(128), smem, s, a);
-    return;
-  }
+    if (!tp) return launch_plan_fused(a, k1a, nk1, s);
+    a.g0 = k1a * a.H2;
+    launch_fused_tp(a, nk1 * a.H2, s);
+    return true;
+  };
+  if (a.octant == nullptr) return launch(0, a.H1);
   // Tucker path: per chunk of k1, rebuild the half fibres (chunk 0 may already be
   // rebuilt, see matvec_run), then the groups of the chunk
-  const int chunk = a.oct_chunk;
-  for (int k1a = 0; k1a < a.H1; k1a += chunk) {
-    const int nk1 = std::min(chunk, a.H1 - k1a);
+  for (int k1a = 0; k1a < a.H1; k1a += a.oct_chunk) {
     if (k1a > 0 || !a.oct_first_ready) launch_octant_args(a.op, k1a, s, a.oct_cp);
     a.oct_k1a = k1a;
-    a.g0 = k1a * a.H2;
-    ProfScope ps(fam, s);
-    bool done = false;
-    if (tp) {
-      launch_fused_tp(a, nk1 * a.H2, STORED, s);
-      done = true;
-    }
-    if (t128) {
-      launch_fused_t128(a, nk1 * a.H2, STORED, s);
-      done = true;
-    }
-    if constexpr (kFs) {
-      if (fs && !done) {
-        launch_pdl(fused_fs_kernel<4 * R, STORED>, dim3(nk1 * a.H2), dim3(96), fs_smem, s, a);
-        done = true;
-      }
-    }
-    if (!done) launch_pdl(fused_warp_kernel<R, STORED>, dim3(nk1 * a.H2), dim3(128), smem, s, a);
+    if (!launch(k1a, std::min(a.oct_chunk, a.H1 - k1a))) return false;
   }
-}
-
-template <bool STORED>
-static bool launch_fused_warp(const FusedArgs<float>& a, cudaStream_t s) {
-  if (a.P3 % 32 != 0) return false;
-  switch (a.P3 / 32) {
-    case 1: launch_fused_warp_r<1, STORED>(a, s); return true;
-    case 2: launch_fused_warp_r<2, STORED>(a, s); return true;
-    case 3: launch_fused_warp_r<3, STORED>(a, s); return true;
-    case 4: launch_fused_warp_r<4, STORED>(a, s); return true;
-    case 5: launch_fused_warp_r<5, STORED>(a, s); return true;
-    case 6: launch_fused_warp_r<6, STORED>(a, s); return true;
-    case 8: launch_fused_warp_r<8, STORED>(a, s); return true;
-    case 10: launch_fused_warp_r<10, STORED>(a, s); return true;
-    case 12: launch_fused_warp_r<12, STORED>(a, s); return true;
-    case 16: launch_fused_warp_r<16, STORED>(a, s); return true;
-    default: return false;
-  }
+  return true;
 }
 
 template <typename T>
@@ -739,7 +661,7 @@ static size_t fused_smem(const FusedArgs<T>& a, int LR) {
 template <typename T, bool STORED>
 static int launch_fused_impl(FusedArgs<T> a, cudaStream_t s) {
   if constexpr (sizeof(T) == 4) {
-    if (launch_fused_warp<STORED>(a, s)) return VIE_OK;
+    if (launch_fused_fast(a, s)) return VIE_OK;
   }
   const size_t limit = 227 * 1024;
   int LR = 4;
@@ -804,11 +726,11 @@ vie::FusedArgs<T> make_fused_args(const vie_op* op, cx<T>* data, int B, bool sto
   a.data = data;
   if constexpr (sizeof(T) == 4) {
     a.roots = op->roots32[2];
-    a.spec = op->spec32;
+    a.spec = stored ? op->spec32 : nullptr;
     a.meta = reinterpret_cast<const CompMeta<T>*>(op->meta);
   } else {
     a.roots = op->roots64[2];
-    a.spec = op->spec64;
+    a.spec = stored ? op->spec64 : nullptr;
     a.meta = reinterpret_cast<const CompMeta<T>*>(static_cast<char*>(op->meta) +
                                                   6 * sizeof(CompMeta<float>));
   }
@@ -834,8 +756,7 @@ vie::FusedArgs<T> make_fused_args(const vie_op* op, cx<T>* data, int B, bool sto
   // padded voxel and right-hand side; the fused kernel itself moves half of
   // that (n3 of P3 z-points in and out), the zero padding never leaving chip
   a.prof_rhs_bytes = 12ull * a.comp_stride * sizeof(cx<T>);
-  a.prof_launch_bytes = stored ? 6ull * a.spec_stride * sizeof(cx<T>) : 0ull;
-  (void)stored;
+  a.prof_launch_bytes = stored ? 6ull * a.H1 * a.H2 * a.H3 * sizeof(cx<T>) : 0ull;
   return a;
 }
 
@@ -843,10 +764,15 @@ int launch_octant(const vie_op* op, int k1a, cudaStream_t s, bool cp) {
   return vie::launch_octant_args(op, k1a, s, cp);
 }
 
+bool lane_fft_edge(int P3) { return P3 % 32 == 0 && vie::warp_fft_supported(P3 / 32); }
+
 bool octant_uses_tc(const vie_op* op) { return op->u3frag != nullptr; }
 
 bool tc_rebuild_eligible(const vie_op* op) {
-  return op->oct32 != nullptr && !(op->flags & VIE_REBUILD_SIMT) &&
+  // edges other than 32 R keep FP32 FMAs: 3xTF32 raised the product's error against
+  // 64 bits there (50 x 72 x 60 at 1e-6: 4.2e-7 to 5.6e-7; 90 x 63 x 105: 4.0e-7 to
+  // 5.4e-7), and the rebuild runs beside the x and y stages either way
+  return op->oct32 != nullptr && !(op->flags & VIE_REBUILD_SIMT) && lane_fft_edge(op->P[2]) &&
          vie::tc_ks(op->rmax[2]) <= vie::kTcMaxKs;
 }
 
@@ -1072,12 +998,6 @@ int fused_init_attributes() {
   e = e != cudaSuccess ? e : cudaFuncSetAttribute(vie::fused_z_kernel<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
   e = e != cudaSuccess ? e : cudaFuncSetAttribute(vie::fused_z_kernel<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
   e = e != cudaSuccess ? e : cudaFuncSetAttribute(vie::fused_z_kernel<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-  e = e != cudaSuccess ? e : cudaFuncSetAttribute(vie::fused_fs_kernel<8, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-  e = e != cudaSuccess ? e : cudaFuncSetAttribute(vie::fused_fs_kernel<8, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-  e = e != cudaSuccess ? e : cudaFuncSetAttribute(vie::fused_fs_kernel<16, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-  e = e != cudaSuccess ? e : cudaFuncSetAttribute(vie::fused_fs_kernel<16, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-  e = e != cudaSuccess ? e : cudaFuncSetAttribute(vie::fused_fs_kernel<24, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-  e = e != cudaSuccess ? e : cudaFuncSetAttribute(vie::fused_fs_kernel<24, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
   e = e != cudaSuccess ? e : cudaFuncSetAttribute(vie::octant_tc_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
   e = e != cudaSuccess ? e : cudaFuncSetAttribute(vie::octant_tc_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
   e = e != cudaSuccess ? e : cudaFuncSetAttribute(vie::octant_tc_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);

@@ -75,120 +75,6 @@ __global__ void __launch_bounds__(256, 3) line_fft_kernel(const LineArgs<T> a) {
   }
 }
 
-// Register-resident variant for N = 32 R (columns contiguous in memory): one
-// 16-column tile per CTA, see line_warp_tile.
-// Resident CTAs per SM the register budget is sized for: up to radix 4 the
-// kernel fits 40 registers without spills (six 256-thread CTAs per SM), up to
-// radix 8 64 registers; larger radices get more registers than that.
-__host__ __device__ constexpr int line_min_blocks(int R) { return R <= 4 ? 6 : (R <= 8 ? 4 : 2); }
-
-template <int R, bool HALF>
-__global__ void __launch_bounds__(256, line_min_blocks(R)) line_warp_kernel(const LineArgs<float> a) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  line_warp_tile<R, HALF>(a, blockIdx.x * kLineTile, blockIdx.y, blockIdx.z,
-                          reinterpret_cast<float2*>(smem_raw));
-}
-
-// Register-direct variant (no shared memory): one warp per kRegCols adjacent
-// columns, see line_reg_group.  Used for radix <= 6.
-__host__ __device__ constexpr int line_reg_min_blocks(int R) { return R <= 4 ? 8 : 5; }
-
-template <int R, bool HALF>
-__global__ void __launch_bounds__(128, line_reg_min_blocks(R)) line_reg_kernel(const LineArgs<float> a,
-                                                                             int vec) {
-  const int lane = threadIdx.x & 31;
-  const long long w = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int ncg = (a.ncol + kRegCols - 1) / kRegCols;
-  if (w >= (long long)ncg * a.nother * a.nbatch) return;        // warp-uniform; no barriers
-  const int cg = (int)(w % ncg);
-  const int o = (int)((w / ncg) % a.nother);
-  const int bb = (int)(w / ((long long)ncg * a.nother));
-  line_reg_group<R, HALF>(a, cg * kRegCols, o, bb, vec != 0, lane);
-}
-
-// Four-step variant (see line_fs_group) for N = 8 V with V = 4 R, R even.
-__host__ __device__ constexpr int line_fs_min_blocks(int V) { return V <= 16 ? 8 : 4; }
-
-template <int V, bool HALF>
-__global__ void __launch_bounds__(128, line_fs_min_blocks(V)) line_fs_kernel(const LineArgs<float> a) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  float2* xs = reinterpret_cast<float2*>(smem_raw) + (size_t)warp * kRegCols * fs_col_stride(V);
-  const long long w = (long long)blockIdx.x * (blockDim.x >> 5) + warp;
-  const int ncg = (a.ncol + kRegCols - 1) / kRegCols;
-  if (w >= (long long)ncg * a.nother * a.nbatch) return;        // warp-uniform; no barriers
-  const int cg = (int)(w % ncg);
-  const int o = (int)((w / ncg) % a.nother);
-  const int bb = (int)(w / ((long long)ncg * a.nother));
-  line_fs_group<V, HALF>(a, cg * kRegCols, o, bb, lane, xs);
-}
-
-template <int V>
-static void launch_fs_v(LineArgs<float> a, cudaStream_t s) {
-  const int ncg = (a.ncol + kRegCols - 1) / kRegCols;
-  const long long warps = (long long)ncg * a.nother * a.nbatch;
-  const int threads = a.threads > 0 && a.threads <= 128 ? a.threads : 128;
-  const unsigned grid = (unsigned)((warps + threads / 32 - 1) / (threads / 32));
-  a.prof = prof_bytes(a.prof_family);
-  ProfScope ps(a.prof_family, s);
-  const bool half = a.inverse ? (2 * a.lout == a.plan.N) : (2 * a.lin == a.plan.N);
-  launch_pdl(half ? line_fs_kernel<V, true> : line_fs_kernel<V, false>, dim3(grid), dim3(threads),
-             line_fs_smem(V, threads / 32), s, a);
-}
-
-static bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
-
-template <int R>
-static void launch_reg_r(LineArgs<float> a, cudaStream_t s) {
-  const int ncg = (a.ncol + kRegCols - 1) / kRegCols;
-  const long long warps = (long long)ncg * a.nother * a.nbatch;
-  const int threads = a.threads > 0 && a.threads <= 128 ? a.threads : 128;
-  const unsigned grid = (unsigned)((warps + threads / 32 - 1) / (threads / 32));
-  // 16-byte row accesses: every row start of every group is a multiple of 16 bytes
-  const bool even = a.in_bs % 2 == 0 && a.in_os % 2 == 0 && a.in_ls % 2 == 0 &&
-                    a.out_bs % 2 == 0 && a.out_os % 2 == 0 && a.out_ls % 2 == 0;
-  const int vec = even && aligned16(a.in) && aligned16(a.out) ? 1 : 0;
-  a.chi_vec = a.chi != nullptr && aligned16(a.chi) && a.chi_os % 2 == 0 && a.chi_ls % 2 == 0;
-  a.addend_vec = a.addend != nullptr && aligned16(a.addend);
-  a.prof = prof_bytes(a.prof_family);
-  ProfScope ps(a.prof_family, s);
-  const bool half = a.inverse ? (2 * a.lout == a.plan.N) : (2 * a.lin == a.plan.N);
-  launch_pdl(half ? line_reg_kernel<R, true> : line_reg_kernel<R, false>, dim3(grid), dim3(threads), 0,
-             s, a, vec);
-}
-
-template <int R>
-static void launch_warp_r(LineArgs<float> a, cudaStream_t s) {
-  const size_t smem = line_warp_smem(R);
-  dim3 grid((a.ncol + kLineTile - 1) / kLineTile, a.nother, a.nbatch);
-  a.prof = prof_bytes(a.prof_family);
-  ProfScope ps(a.prof_family, s);
-  const int threads = a.threads > 0 ? a.threads : 256;
-  // half-length lines: forward from n = N/2 points, or inverse cropped to N/2
-  const bool half = a.inverse ? (2 * a.lout == a.plan.N) : (2 * a.lin == a.plan.N);
-  launch_pdl(half ? line_warp_kernel<R, true> : line_warp_kernel<R, false>, grid, dim3(threads), smem,
-             s, a);
-}
-
-static bool launch_warp(const LineArgs<float>& a, cudaStream_t s) {
-  const int N = a.plan.N;
-  if (N % 32 != 0 || a.in_cs != 1 || a.out_cs != 1) return false;
-  if ((a.flags & (PRO_CHI | EPI_CHI)) && a.chi_cs != 1) return false;
-  switch (N / 32) {
-    case 1: launch_reg_r<1>(a, s); return true;
-    case 2: launch_fs_v<8>(a, s); return true;
-    case 3: launch_reg_r<3>(a, s); return true;
-    case 4: launch_fs_v<16>(a, s); return true;
-    case 5: launch_reg_r<5>(a, s); return true;
-    case 6: launch_fs_v<24>(a, s); return true;
-    case 8: launch_warp_r<8>(a, s); return true;
-    case 10: launch_warp_r<10>(a, s); return true;
-    case 12: launch_warp_r<12>(a, s); return true;
-    case 16: if (!launch_line_tp(a, s)) launch_warp_r<16>(a, s); return true;
-    default: return false;
-  }
-}
-
 template <typename T, int TW>
 static void launch_tw(LineArgs<T> a, size_t smem, cudaStream_t s) {
   dim3 grid((a.ncol + TW - 1) / TW, a.nother, a.nbatch);
@@ -197,12 +83,18 @@ static void launch_tw(LineArgs<T> a, size_t smem, cudaStream_t s) {
   line_fft_kernel<T, TW><<<grid, 256, smem, s>>>(a);
 }
 
+// The general kernel below takes what the planned and length-512 kernels leave:
+// padded edges without a plan (below 16, 490, above 512), full-length transforms
+// and lines along z (the setup's 3-D FFT).
 // Widest tile (16, 8 or 4 lines; 128 bytes per row for c64 at 16) whose two
 // ping-pong buffers and root table fit in 227 KB of shared memory.
 template <typename T>
 void launch_line_fft(const LineArgs<T>& a, cudaStream_t s) {
   if constexpr (sizeof(T) == 4) {
-    if (launch_warp(a, s)) return;
+    // length 512: the persistent TMA-fed kernel (x + y + their inverses of eight
+    // 256^3 right-hand sides 12.4 ms; 32 x 16 of the planned kernel 14.8 ms)
+    if (a.plan.N == 512 && launch_line_tp(a, s)) return;
+    if (launch_plan_line(a, s)) return;
   } else {
     if (a.plan.N == 512 && launch_line_tp64(a, s)) return;
   }
@@ -238,14 +130,6 @@ int line_fft_init_attributes() {
   e = e != cudaSuccess ? e : cudaFuncSetAttribute(vie::line_fft_kernel<float, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
   e = e != cudaSuccess ? e : cudaFuncSetAttribute(vie::line_fft_kernel<double, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
   e = e != cudaSuccess ? e : cudaFuncSetAttribute(vie::line_fft_kernel<double, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-  e = e != cudaSuccess ? e : cudaFuncSetAttribute(vie::line_warp_kernel<8, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-  e = e != cudaSuccess ? e : cudaFuncSetAttribute(vie::line_warp_kernel<8, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-  e = e != cudaSuccess ? e : cudaFuncSetAttribute(vie::line_warp_kernel<10, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-  e = e != cudaSuccess ? e : cudaFuncSetAttribute(vie::line_warp_kernel<10, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-  e = e != cudaSuccess ? e : cudaFuncSetAttribute(vie::line_warp_kernel<12, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-  e = e != cudaSuccess ? e : cudaFuncSetAttribute(vie::line_warp_kernel<12, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-  e = e != cudaSuccess ? e : cudaFuncSetAttribute(vie::line_warp_kernel<16, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-  e = e != cudaSuccess ? e : cudaFuncSetAttribute(vie::line_warp_kernel<16, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
   return e == cudaSuccess ? VIE_OK : cuda_status(e, "line kernel attributes");
 }
 

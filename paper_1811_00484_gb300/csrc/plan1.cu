@@ -1,0 +1,4 @@
+// Matvec stages of the edges in VIE_PLAN_SET_1 (plan_table.h).
+#define VIE_SET 1
+#define VIE_SET_SIZES VIE_PLAN_SET_1
+#include "plan_set.cuh"

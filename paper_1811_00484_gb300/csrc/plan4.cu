@@ -1,0 +1,4 @@
+// Matvec stages of the edges in VIE_PLAN_SET_4 (plan_table.h).
+#define VIE_SET 4
+#define VIE_SET_SIZES VIE_PLAN_SET_4
+#include "plan_set.cuh"

@@ -1,0 +1,4 @@
+// Matvec stages of the edges in VIE_PLAN_SET_9 (plan_table.h).
+#define VIE_SET 9
+#define VIE_SET_SIZES VIE_PLAN_SET_9
+#include "plan_set.cuh"

@@ -1,0 +1,449 @@
+// Matvec stages for every padded edge N = 2n with a factor plan: x / y line
+// stages (zero-padded forward, cropped inverse) and the fused z stage (forward
+// transform, voxel-wise product, inverse transform), in FP32 and FP64.  All
+// lengths, strides in shared memory and radices are compile-time constants, so
+// the only index arithmetic left is one multiply-add per access.
+//
+// Line stage, N = Q1 Q2, thread (col, t): columns are adjacent in memory.
+// With n = a + Q2 b, k = c + Q1 h,
+//   X[c + Q1 h] = sum_a w_{Q2}^{a h} w_N^{a c} sum_b x[a + Q2 b] w_{Q1}^{b c}:
+//   pass 1 (thread a): DFT of length Q1 over b, twiddle, X1[c][a][col] to shared
+//   pass 2 (thread c): DFT of length Q2 over a, rows c + Q1 h to global memory.
+// One shared-memory exchange and one barrier per line.  The padding (b >= Q1/2
+// are zero; Q1 even forward) and the crop (only h < Q2/2 are kept; Q2 even
+// inverse) are pruned out of the butterflies.
+//
+// Fused stage, N = R1 R2 R3 (R3 = 1: two passes), S threads per z-line, up to
+// four mirror lines of one (k1, k2) group per CTA.  n = a + M1 b (M1 = R2 R3),
+// a = e + R3 f, k = c + R1 g + R1 R2 h:
+//   pass 1 (thread a):      DFT-R1 over b, twiddle w_N^{a c}
+//   pass 2 (thread (c, e)): DFT-R2 over f, twiddle w_{R2 R3}^{e g}
+//   pass 3 (thread (c, g)): DFT-R3 over e, frequencies c + R1 g + R1 R2 h
+// Every pass reads and writes the same addresses in the same thread, so each of
+// the three Cartesian components keeps one buffer and a barrier is needed only
+// between passes (two per right-hand side with two passes, four with three).
+// The thread ends with the three components of its frequencies in registers,
+// forms Y = D G D J there (mirror signs folded into G's off-diagonal entries)
+// and runs the passes backwards in place.
+//
+// The half fibre G[6][N/2+1] of the group is copied from the FP32 rebuild
+// scratch, read from the stored spectra (only the octant k <= P/2: the rest is
+// its mirror image, an eighth of the bytes), or rebuilt by the CTA (FP64, and
+// ranks beyond the rebuild kernels').
+#pragma once
+
+#include "regdft.cuh"
+#include "stages.cuh"
+
+namespace vie {
+namespace plan {
+
+__host__ __device__ constexpr int imax(int a, int b) { return a > b ? a : b; }
+
+// ---------------------------------------------------------------------------
+// line stage
+// ---------------------------------------------------------------------------
+// columns per CTA: 128 bytes of a row, fewer when a line needs more than 16 threads
+template <typename T> __host__ __device__ constexpr int line_cols(int S) {
+  return sizeof(T) == 4 ? (S <= 16 ? 16 : 8) : (S <= 16 ? 8 : 4);
+}
+// registers a thread may use: the larger radix's values, its DFT's temporaries
+// and the addresses
+template <typename T> __host__ __device__ constexpr int line_regs(int R) {
+  const int r = sizeof(T) == 4 ? (R <= 8 ? 40 : R <= 10 ? 48 : R <= 16 ? 72 : R <= 21 ? 96 : 128)
+                               : (R <= 8 ? 80 : R <= 10 ? 96 : R <= 16 ? 128 : 168);
+  return r;
+}
+template <typename T> __host__ __device__ constexpr int line_blocks(int Q1, int Q2) {
+  const int S = imax(Q1, Q2), th = line_cols<T>(S) * S;
+  const int b = 65536 / (line_regs<T>(S) * ((th + 31) / 32 * 32));
+  return b < 1 ? 1 : (b > 24 ? 24 : b);
+}
+
+template <typename T, int Q1, int Q2, bool INV>
+__global__ void __launch_bounds__(line_cols<T>(imax(Q1, Q2)) * imax(Q1, Q2), line_blocks<T>(Q1, Q2))
+    plan_line_kernel(const LineArgs<T> a) {
+  using C = cx<T>;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C* X = reinterpret_cast<C*>(smem_raw);               // [Q1][Q2][CW]
+  const int CW = blockDim.x, col = threadIdx.x, t = threadIdx.y;
+  const int c0 = blockIdx.x * CW + col, o = blockIdx.y, bb = blockIdx.z;
+  pdl_trigger();
+  pdl_wait();
+  if (a.active != nullptr && a.active[bb / a.batch_per_rhs] == 0) return;   // block-uniform
+  if (a.prof != nullptr && blockIdx.x == 0 && o == 0 && col == 0 && t == 0)
+    atomicAdd(a.prof, a.prof_batch_bytes);
+  const bool col_ok = c0 < a.ncol;
+  const T rs = (a.flags & (PRO_RSCALE | EPI_RSCALE))
+                   ? (T)a.rscale[(long long)(bb / a.batch_per_rhs) * a.rscale_stride]
+                   : (T)1;
+  if (t < Q2) {
+    const C* in = a.in + bb * a.in_bs + o * a.in_os + c0 + (long long)t * a.in_ls;
+    const long long step = (long long)Q2 * a.in_ls;
+    C v[Q1];
+    if constexpr (!INV) {
+      C x[Q1 / 2];
+#pragma unroll
+      for (int m = 0; m < Q1 / 2; ++m) x[m] = col_ok ? in[m * step] : czero<C>();
+      if (a.flags & (PRO_RSCALE | PRO_CONJ | PRO_CHI)) {
+        const C* chi = a.chi + o * a.chi_os + c0 + (long long)t * a.chi_ls;
+#pragma unroll
+        for (int m = 0; m < Q1 / 2; ++m) {
+          if (a.flags & PRO_RSCALE) x[m] = rs * x[m];
+          if (a.flags & PRO_CONJ) x[m] = conjg(x[m]);
+          if ((a.flags & PRO_CHI) && col_ok) x[m] = chi[(long long)m * Q2 * a.chi_ls] * x[m];
+        }
+      }
+      dft_half_in<Q1, false>(x, v);
+    } else {
+#pragma unroll
+      for (int m = 0; m < Q1; ++m) v[m] = col_ok ? in[m * step] : czero<C>();
+      dft_reg<Q1, true>(v);
+    }
+#pragma unroll
+    for (int c = 1; c < Q1; ++c) {
+      const C w = __ldg(a.roots + t * c);
+      v[c] = v[c] * (INV ? conjg(w) : w);
+    }
+#pragma unroll
+    for (int c = 0; c < Q1; ++c) X[(c * Q2 + t) * CW + col] = v[c];
+  }
+  __syncthreads();
+  if (t >= Q1 || !col_ok) return;
+  C u[Q2];
+#pragma unroll
+  for (int f = 0; f < Q2; ++f) u[f] = X[(t * Q2 + f) * CW + col];
+  const long long obase = bb * a.out_bs + o * a.out_os + c0 + (long long)t * a.out_ls;
+  const long long ostep = (long long)Q1 * a.out_ls;
+  C* out = a.out + obase;
+  if constexpr (!INV) {
+    dft_reg<Q2, false>(u);
+#pragma unroll
+    for (int h = 0; h < Q2; ++h) out[h * ostep] = u[h];
+  } else {
+    C y[Q2 / 2];
+    dft_half_out<Q2, true>(u, y);
+#pragma unroll
+    for (int h = 0; h < Q2 / 2; ++h) y[h] = a.scale * y[h];
+    if (a.flags & (EPI_CONJ | EPI_SUB | EPI_ADD)) {
+      const C* chi = a.chi + o * a.chi_os + c0 + (long long)t * a.chi_ls;
+      const C* add = a.addend + obase;
+#pragma unroll
+      for (int h = 0; h < Q2 / 2; ++h) {
+        C x = y[h];
+        if (a.flags & EPI_CONJ) x = conjg(x);
+        if (a.flags & (EPI_SUB | EPI_ADD)) {
+          if (a.flags & EPI_CHI) x = chi[(long long)h * Q1 * a.chi_ls] * x;
+          C w = add[h * ostep];
+          if (a.flags & EPI_RSCALE) w = rs * w;
+          x = (a.flags & EPI_SUB) ? (w - x) : (w + x);
+        }
+        y[h] = x;
+      }
+    }
+#pragma unroll
+    for (int h = 0; h < Q2 / 2; ++h) out[h * ostep] = y[h];
+  }
+}
+
+// Q1 is even: forward Q1 x Q2, inverse Q2 x Q1 (the even radix where the half is)
+template <typename T, int Q1, int Q2> void launch_plan_line(LineArgs<T> a, cudaStream_t s) {
+  static_assert(Q1 % 2 == 0, "the pruned radix is even");
+  constexpr int S = imax(Q1, Q2), CMAX = line_cols<T>(S);
+  // lines whose columns are adjacent across `o` too (the x stages) form one run
+  if (a.in_os == a.ncol && a.out_os == a.ncol && (a.chi == nullptr || a.chi_os == a.ncol) &&
+      (long long)a.ncol * a.nother < (1LL << 30)) {
+    a.ncol *= a.nother;
+    a.nother = 1;
+  }
+  // equal column groups: 50 columns are 4 groups of 13, not 3 of 16 and one of 2
+  const int tiles = (a.ncol + CMAX - 1) / CMAX;
+  const int cw = (a.ncol + tiles - 1) / tiles;
+  a.prof = sizeof(T) == 4 ? prof_bytes(a.prof_family) : nullptr;
+  ProfScope ps(a.prof_family, s);
+  const dim3 grid((unsigned)tiles, (unsigned)a.nother, (unsigned)a.nbatch), block((unsigned)cw, S);
+  const size_t smem = (size_t)Q1 * Q2 * cw * sizeof(cx<T>);
+  if (a.inverse) launch_pdl(plan_line_kernel<T, Q2, Q1, true>, grid, block, smem, s, a);
+  else launch_pdl(plan_line_kernel<T, Q1, Q2, false>, grid, block, smem, s, a);
+}
+
+template <typename T, int Q1, int Q2> cudaError_t prepare_plan_line() {
+  constexpr size_t smem = (size_t)Q1 * Q2 * line_cols<T>(imax(Q1, Q2)) * sizeof(cx<T>);
+  if constexpr (smem > 48 * 1024) {
+    cudaError_t e = cudaFuncSetAttribute(plan_line_kernel<T, Q1, Q2, false>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(plan_line_kernel<T, Q2, Q1, true>,
+                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    return e;
+  }
+  return cudaSuccess;
+}
+
+// ---------------------------------------------------------------------------
+// fused z stage
+// ---------------------------------------------------------------------------
+template <int R1, int R2, int R3> struct FusedPlan {
+  static constexpr int N = R1 * R2 * R3, M1 = R2 * R3, H3 = N / 2 + 1;
+  static constexpr int HL = R3 > 1 ? R3 : R2;               // frequencies per thread
+  static constexpr int TL = R3 > 1 ? R1 * R2 : R1;          // threads that hold them
+  static constexpr int S = imax(imax(M1, R1 * R3), TL);     // threads per line
+  static constexpr int PR = R3 > 1 ? (R3 | 1) : 1;          // padded run of e
+  static constexpr int LD = (R3 > 1 ? R2 * PR : R2) | 1;    // row c of a line's buffer (odd)
+  static constexpr int LS = R1 * LD;                        // one line of one component
+  static constexpr int NL = (R1 + 1) / 2;                   // inputs that can be nonzero
+  // small groups share a CTA
+  static constexpr int GP = 4 * S >= 64 ? 1 : (64 + 4 * S - 1) / (4 * S);
+  static constexpr int threads = 4 * S * GP;
+  static constexpr int GH = 6 * H3 + (6 * H3 & 1);          // half fibres, 16-byte multiple
+  static __host__ __device__ constexpr int inner(int a) {   // X1 column of a = e + R3 f
+    return R3 > 1 ? (a / R3) * PR + a % R3 : a;
+  }
+};
+template <typename T, int R1, int R2, int R3> __host__ __device__ constexpr int fused_blocks() {
+  using P = FusedPlan<R1, R2, R3>;
+  // live at the peak: three components of HL frequencies and a half fibre
+  // entry, or two components' inputs, one transform and its temporaries
+  const int live = imax(6 * P::HL + 60, 4 * P::NL + 3 * R1 + 36);
+  const int regs = sizeof(T) == 4 ? (live < 64 ? 64 : live > 168 ? 168 : live)
+                                  : (live * 2 > 255 ? 255 : live * 2);
+  const int wt = (P::threads + 31) / 32 * 32;
+  const int b = 65536 / (((regs + 7) / 8 * 8) * wt);
+  return b < 1 ? 1 : (b > 16 ? 16 : b);
+}
+
+template <typename T, int R1, int R2, int R3>
+__global__ void __launch_bounds__(FusedPlan<R1, R2, R3>::threads, fused_blocks<T, R1, R2, R3>())
+    plan_fused_kernel(const FusedArgs<T> a, int k10) {
+  using C = cx<T>;
+  using P = FusedPlan<R1, R2, R3>;
+  constexpr int N = P::N, S = P::S, H3 = P::H3, HL = P::HL, LD = P::LD, NL = P::NL, M1 = P::M1;
+  constexpr bool kEven = R1 % 2 == 0;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int gp = threadIdx.x / (4 * S), lt = threadIdx.x % (4 * S);
+  const int l = lt / S, t = lt % S;
+  C* G = reinterpret_cast<C*>(smem_raw) + gp * P::GH;                      // [6][H3]
+  C* X = reinterpret_cast<C*>(smem_raw) + P::GP * P::GH + (gp * 12 + l * 3) * P::LS;   // [3][R1][LD]
+  const int k1 = k10 + blockIdx.y, k2 = blockIdx.x * P::GP + gp;
+  const bool group = k2 < a.H2;
+  const int nx = (k1 == 0 || 2 * k1 == a.P1) ? 1 : 2;
+  const int ny = (k2 == 0 || 2 * k2 == a.P2) ? 1 : 2;
+  const bool valid = group && l < nx * ny;
+  const int ix = valid ? l / ny : 0, iy = valid ? l % ny : 0;
+  const int kx = ix ? a.P1 - k1 : k1, ky = iy ? a.P2 - k2 : k2;
+  C* line0 = a.data + ((long long)kx * a.P2 + ky) * (N / 2) + t;
+  // no rebuilt half fibres to copy (FP64; FP32 beyond the rebuild kernels' ranks):
+  // eq. (13) for this group here
+  const bool here = a.spec == nullptr && a.octant == nullptr;
+  if (here && group) {
+    // W_c = U2_c[k2, :] S_c[k1], G_c[k3] = W_c . U3_c[k3, :]
+    C* W = reinterpret_cast<C*>(smem_raw) + P::GP * (P::GH + 12 * P::LS) + gp * 6 * a.r3max;
+    for (int it = lt; it < 6 * a.r3max; it += 4 * S) {
+      const int c = it / a.r3max, q = it - c * a.r3max;
+      const CompMeta<T>& m = a.meta[c];
+      C acc = czero<C>();
+      if (q < m.r3) {
+        const C* sl = m.slab + (long long)k1 * a.r2max * a.r3max + q;
+        const C* u2 = m.U2 + (long long)k2 * m.r2;
+        for (int b = 0; b < m.r2; ++b) acc = cmadd(u2[b], sl[b * a.r3max], acc);
+      }
+      W[it] = acc;
+    }
+  }
+  if (here) {
+    __syncthreads();
+    if (group) {
+      const C* W = reinterpret_cast<C*>(smem_raw) + P::GP * (P::GH + 12 * P::LS) + gp * 6 * a.r3max;
+      for (int it = lt; it < 6 * H3; it += 4 * S) {
+        const int c = it / H3, kk = it - c * H3;
+        const int r3 = a.meta[c].r3;
+        const C* u3 = a.meta[c].U3 + (long long)kk * r3;
+        C acc = czero<C>();
+        for (int q = 0; q < r3; ++q) acc = cmadd(W[c * a.r3max + q], u3[q], acc);
+        G[it] = acc;
+      }
+    }
+  }
+  pdl_trigger();
+  pdl_wait();
+  if (a.prof != nullptr && blockIdx.x == 0 && k1 == 0 && threadIdx.x == 0) {
+    unsigned long long nb = 0;
+    for (int b = 0; b < a.B; ++b) nb += (a.active == nullptr || a.active[b]) ? 1 : 0;
+    atomicAdd(a.prof, nb * a.prof_rhs_bytes + a.prof_launch_bytes);
+  }
+  auto next_active = [&](int b) {
+    if (a.active != nullptr)
+      while (b < a.B && a.active[b] == 0) ++b;
+    return b;
+  };
+  // the three components' inputs in flight together
+  C x[3][NL];
+  auto load = [&](int b) {
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      const C* src = line0 + (long long)(b * 3 + q) * a.comp_stride;
+#pragma unroll
+      for (int m = 0; m < NL; ++m)
+        x[q][m] = (valid && t < M1 && (kEven || t + M1 * m < N / 2)) ? src[M1 * m] : czero<C>();
+    }
+  };
+  int b = next_active(0);
+  if (b < a.B) load(b);
+  if (group) {
+    if (a.spec != nullptr) {
+      const C* src = a.spec + ((long long)k1 * a.P2 + k2) * N;
+      for (int it = lt; it < 6 * H3; it += 4 * S) {
+        const int c = it / H3, kk = it - c * H3;
+        G[it] = src[c * a.spec_stride + kk];
+      }
+    } else if (!here) {
+      const float4* src = reinterpret_cast<const float4*>(
+          a.octant + ((long long)(k1 - a.oct_k1a) * a.H2 + k2) * 6 * H3);
+      float4* dst = reinterpret_cast<float4*>(G);
+      for (int it = lt; it < 6 * H3 * (int)sizeof(C) / 16; it += 4 * S) dst[it] = src[it];
+    }
+  }
+  const T sx = ix ? (T)-1 : (T)1, sy = iy ? (T)-1 : (T)1;
+  const int c2 = t % R1, e2 = t / R1;                  // slots (c, e) and (c, g)
+  for (bool first = true; b < a.B; b = next_active(b + 1), first = false) {   // block-uniform
+    if (!first) load(b);
+    if (t < M1) {
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        C v[R1];
+        if constexpr (kEven) {
+          dft_half_in<R1, false>(x[q], v);
+        } else {
+#pragma unroll
+          for (int m = 0; m < R1; ++m) v[m] = m < NL ? x[q][m < NL ? m : 0] : czero<C>();
+          dft_reg<R1, false>(v);
+        }
+        C* row = X + q * P::LS + P::inner(t);
+        row[0] = v[0];
+#pragma unroll
+        for (int c = 1; c < R1; ++c) row[c * LD] = v[c] * __ldg(a.roots + t * c);
+      }
+    }
+    __syncthreads();
+    if constexpr (R3 > 1) {
+      if (t < R1 * R3) {
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          C u[R2];
+          C* p = X + q * P::LS + c2 * LD + e2;
+#pragma unroll
+          for (int f = 0; f < R2; ++f) u[f] = p[f * P::PR];
+          dft_reg<R2, false>(u);
+          p[0] = u[0];
+#pragma unroll
+          for (int g = 1; g < R2; ++g) p[g * P::PR] = u[g] * __ldg(a.roots + R1 * e2 * g);
+        }
+      }
+      __syncthreads();
+    }
+    if (t < P::TL) {
+      C s[3][HL];
+      C* own = X + c2 * LD + (R3 > 1 ? e2 * P::PR : 0);     // this thread's points of a component
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+#pragma unroll
+        for (int e = 0; e < HL; ++e) s[q][e] = own[q * P::LS + e];
+        dft_reg<HL, false>(s[q]);
+      }
+      // Y = D G D J at f = t + TL h
+#pragma unroll
+      for (int h = 0; h < HL; ++h) {
+        const int f = t + P::TL * h;
+        const bool zm = 2 * f > N;
+        const C* gp_ = G + (zm ? N - f : f);
+        const T sz = zm ? (T)-1 : (T)1;
+        const C gxx = gp_[0], gyy = gp_[3 * H3], gzz = gp_[5 * H3];
+        const C gxy = (sx * sy) * gp_[H3], gxz = (sx * sz) * gp_[2 * H3], gyz = (sy * sz) * gp_[4 * H3];
+        const C jx = s[0][h], jy = s[1][h], jz = s[2][h];
+        s[0][h] = cmadd(gxx, jx, cmadd(gxy, jy, gxz * jz));
+        s[1][h] = cmadd(gxy, jx, cmadd(gyy, jy, gyz * jz));
+        s[2][h] = cmadd(gxz, jx, cmadd(gyz, jy, gzz * jz));
+      }
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        dft_reg<HL, true>(s[q]);
+        own[q * P::LS] = s[q][0];                      // e = 0, or a = 0
+        if constexpr (R3 > 1) {
+#pragma unroll
+          for (int e = 1; e < HL; ++e)
+            own[q * P::LS + e] = s[q][e] * conjg(__ldg(a.roots + R1 * e * e2));
+        } else {
+#pragma unroll
+          for (int e = 1; e < HL; ++e) own[q * P::LS + e] = s[q][e] * conjg(__ldg(a.roots + e * c2));
+        }
+      }
+    }
+    __syncthreads();
+    if constexpr (R3 > 1) {
+      if (t < R1 * R3) {
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          C u[R2];
+          C* p = X + q * P::LS + c2 * LD + e2;
+#pragma unroll
+          for (int g = 0; g < R2; ++g) u[g] = p[g * P::PR];
+          dft_reg<R2, true>(u);
+#pragma unroll
+          for (int f = 0; f < R2; ++f) p[f * P::PR] = u[f] * conjg(__ldg(a.roots + (e2 + R3 * f) * c2));
+        }
+      }
+      __syncthreads();
+    }
+    if (t < M1) {
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        C v[R1];
+        const C* row = X + q * P::LS + P::inner(t);
+#pragma unroll
+        for (int c = 0; c < R1; ++c) v[c] = row[c * LD];
+        C* dst = line0 + (long long)(b * 3 + q) * a.comp_stride;
+        if constexpr (kEven) {
+          C y[R1 / 2];
+          dft_half_out<R1, true>(v, y);
+          if (valid) {
+#pragma unroll
+            for (int m = 0; m < R1 / 2; ++m) dst[M1 * m] = y[m];
+          }
+        } else {
+          dft_reg<R1, true>(v);
+          if (valid) {
+#pragma unroll
+            for (int m = 0; m < NL; ++m)
+              if (t + M1 * m < N / 2) dst[M1 * m] = v[m];
+          }
+        }
+      }
+    }
+  }
+}
+
+template <typename T, int R1, int R2, int R3>
+constexpr size_t fused_smem_fixed() {
+  using P = FusedPlan<R1, R2, R3>;
+  return (size_t)P::GP * (P::GH + 12 * P::LS) * sizeof(cx<T>);
+}
+
+// groups k1 in [k10, k10 + nk1), every k2
+template <typename T, int R1, int R2, int R3>
+void launch_plan_fused(const FusedArgs<T>& a, int k10, int nk1, cudaStream_t s) {
+  using P = FusedPlan<R1, R2, R3>;
+  size_t smem = fused_smem_fixed<T, R1, R2, R3>();
+  if (a.spec == nullptr && a.octant == nullptr) smem += (size_t)P::GP * 6 * a.r3max * sizeof(cx<T>);
+  launch_pdl(plan_fused_kernel<T, R1, R2, R3>, dim3((unsigned)((a.H2 + P::GP - 1) / P::GP), (unsigned)nk1),
+             dim3(P::threads), smem, s, a, k10);
+}
+
+constexpr size_t kFusedSmemMax = 200 * 1024;
+
+template <typename T, int R1, int R2, int R3> cudaError_t prepare_plan_fused() {
+  return cudaFuncSetAttribute(plan_fused_kernel<T, R1, R2, R3>,
+                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFusedSmemMax);
+}
+
+}  // namespace plan
+}  // namespace vie

@@ -29,7 +29,7 @@
 #include <vector>
 
 #include "vie_internal.cuh"
-#include "warpfft.cuh"
+#include "stages.cuh"
 
 namespace {
 
@@ -467,6 +467,7 @@ static int init_tables(vie_op* op) {
     VIE_TRY(dalloc(&op->roots32[q], N * sizeof(float2)));
     VIE_CUDA(cudaMemcpy(op->roots64[q], r64.data(), N * sizeof(double2), cudaMemcpyHostToDevice));
     VIE_CUDA(cudaMemcpy(op->roots32[q], r32.data(), N * sizeof(float2), cudaMemcpyHostToDevice));
+    VIE_TRY(plan_prepare(N));
   }
   return VIE_OK;
 }
@@ -727,10 +728,9 @@ static int finish_operator(vie_op* op) {
   // for the operator, so formed once here rather than at every matvec
   VIE_TRY(launch_slab_cores<float>(op, 0));
   VIE_TRY(launch_slab_cores<double>(op, 0));
-  // FP32 scratch for the per-matvec rebuild of the half fibres (register-path
-  // fused kernel): whole k1 planes of [H2][6][H3], as many as fit in kOctBudget
-  if (op->P[2] % 32 == 0 && vie::warp_fft_supported(op->P[2] / 32) &&
-      octant_smem_bytes(op->rmax[1], op->rmax[2]) <= kOctantSmemMax) {
+  // FP32 scratch for the per-matvec rebuild of the half fibres (planned z edges):
+  // whole k1 planes of [H2][6][H3], as many as fit in kOctBudget
+  if (vie::plan_exists(op->P[2]) && octant_smem_bytes(op->rmax[1], op->rmax[2]) <= kOctantSmemMax) {
     constexpr size_t kOctBudget = 64u << 20;
     const size_t plane = (size_t)op->H[1] * 6 * op->H[2] * sizeof(float2);
     op->oct_k1 = (int)std::max<size_t>(1, std::min<size_t>(op->H[0], kOctBudget / plane));
@@ -738,7 +738,8 @@ static int finish_operator(vie_op* op) {
     VIE_CUDA(cudaStreamCreateWithFlags(&op->rb_stream, cudaStreamNonBlocking));
     VIE_CUDA(cudaEventCreateWithFlags(&op->rb_fork, cudaEventDisableTiming));
     VIE_CUDA(cudaEventCreateWithFlags(&op->rb_join, cudaEventDisableTiming));
-    if ((op->flags & VIE_REBUILD_TCGEN05) && !(op->flags & VIE_REBUILD_SIMT) && umma_rebuild_eligible(op)) {
+    if ((op->flags & VIE_REBUILD_TCGEN05) && !(op->flags & VIE_REBUILD_SIMT) && lane_fft_edge(op->P[2]) &&
+        umma_rebuild_eligible(op)) {
       op->umma = true;
     } else if (tc_rebuild_eligible(op)) {
       tc_layout(op->rmax[2], op->H[2], &op->tc_ks, &op->tc_nsplit, &op->tc_ntc);

@@ -725,10 +725,11 @@ __device__ __forceinline__ void fused_fs_group(const FusedArgs<float>& a, int g,
 // Length-512 kernels (tp512.cu): x / y line stages and the fused z stage
 bool launch_line_tp(LineArgs<float> a, cudaStream_t s);
 bool launch_line_tp64(LineArgs<double> a, cudaStream_t s);
-bool fused_tp_supported(const FusedArgs<float>& a, bool stored);
-void launch_fused_tp(const FusedArgs<float>& a, int groups, bool stored, cudaStream_t s);
-// P3 = 128 (64-voxel z edges): 16 threads per line, radix 8, 4, 4 (t128.cu)
-bool fused_t128_supported(const FusedArgs<float>& a, bool stored);
-void launch_fused_t128(const FusedArgs<float>& a, int groups, bool stored, cudaStream_t s);
+bool fused_tp_supported(const FusedArgs<float>& a);
+void launch_fused_tp(const FusedArgs<float>& a, int groups, cudaStream_t s);
+// every edge with a factor plan (plan.cu): false when the launch is not one of theirs
+bool plan_exists(int N);
+bool launch_plan_line(const LineArgs<float>& a, cudaStream_t s);
+bool launch_plan_fused(const FusedArgs<float>& a, int k10, int nk1, cudaStream_t s);
 
 }  // namespace vie

@@ -550,16 +550,15 @@ __global__ void __launch_bounds__(256, 3) line_tp64_kernel(const LineArgs<double
 // thread carries the three Cartesian components of its line through the
 // forward passes (one after another, sharing the line's exchange buffers),
 // holds their spectra at the eight frequencies c + 8g + 64h in registers,
-// forms Y = D G D J there (G the rebuilt half fibre with mirror signs D, or
-// the stored spectra), and runs the inverse passes.  The line's 256 outputs
+// forms Y = D G D J there (G the rebuilt or stored half fibre with mirror signs
+// D), and runs the inverse passes.  The line's 256 outputs
 // overwrite its 256 inputs.
 // ---------------------------------------------------------------------------
 constexpr int kGS = 256 + 32 + 1;     // ghalf_slot(256) + 1
 constexpr int kLA = 72;               // X1 row stride of the fused layout
 constexpr size_t kFusedSmem = (size_t)(6 * kGS + 4 * kX2 + 4 * kX2 + kTwRows * kM) * sizeof(float2);
 
-template <bool STORED>
-__global__ void __launch_bounds__(256, STORED ? 2 : 3) fused_tp_kernel(const FusedArgs<float> a) {
+__global__ void __launch_bounds__(256, 3) fused_tp_kernel(const FusedArgs<float> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2* ghalf = reinterpret_cast<float2*>(smem_raw);   // [6][kGS]
   const int tid = threadIdx.x, l = tid >> 6, t = tid & 63;
@@ -583,14 +582,20 @@ __global__ void __launch_bounds__(256, STORED ? 2 : 3) fused_tp_kernel(const Fus
     for (int b = 0; b < a.B; ++b) nb += (a.active == nullptr || a.active[b]) ? 1 : 0;
     atomicAdd(a.prof, nb * a.prof_rhs_bytes + a.prof_launch_bytes);
   }
-  if (!STORED) {
-    const float2* src = a.octant + ((long long)(k1 - a.oct_k1a) * a.H2 + k2) * 6 * a.H3;
-    for (int it = tid; it < 6 * a.H3; it += 256) {
-      const int cc = it / a.H3, kk = it - cc * a.H3;
-      ghalf[cc * kGS + ghalf_slot(kk)] = src[it];
+  {
+    // the group's half fibre: rebuilt for this matvec into the scratch, or the
+    // octant k <= P/2 of the stored spectra (the rest is its mirror image)
+    constexpr int H3 = kN / 2 + 1;
+    const bool stored = a.spec != nullptr;
+    const float2* src = stored ? a.spec + ((long long)k1 * a.P2 + k2) * kN
+                               : a.octant + ((long long)(k1 - a.oct_k1a) * a.H2 + k2) * 6 * H3;
+    const long long cs = stored ? a.spec_stride : H3;
+    for (int it = tid; it < 6 * H3; it += 256) {
+      const int cc = it / H3, kk = it - cc * H3;
+      ghalf[cc * kGS + ghalf_slot(kk)] = src[cc * cs + kk];
     }
   }
-  const float sx = (STORED || !ix) ? 1.f : -1.f, sy = (STORED || !iy) ? 1.f : -1.f;
+  const float sx = ix ? -1.f : 1.f, sy = iy ? -1.f : 1.f;
   const int c = t >> 3, g = t & 7;
   __syncthreads();
   for (int b = 0; b < a.B; ++b) {
@@ -621,19 +626,12 @@ __global__ void __launch_bounds__(256, STORED ? 2 : 3) fused_tp_kernel(const Fus
     for (int h = 0; h < 8; ++h) {
       const int f = c + 8 * g + kM * h;
       float2 G[6];
-      float sz = 1.f;
-      if (STORED) {
-        const long long off = ((long long)kx * a.P2 + ky) * kN + f;
+      const bool zm = 2 * f > kN;
+      const int fold = zm ? kN - f : f;
+      const float sz = zm ? -1.f : 1.f;
+      const float2* gp = ghalf + ghalf_slot(fold);
 #pragma unroll
-        for (int q = 0; q < 6; ++q) G[q] = __ldg(a.spec + q * a.spec_stride + off);
-      } else {
-        const bool zm = 2 * f > kN;
-        const int fold = zm ? kN - f : f;
-        sz = zm ? -1.f : 1.f;
-        const float2* gp = ghalf + ghalf_slot(fold);
-#pragma unroll
-        for (int q = 0; q < 6; ++q) G[q] = gp[q * kGS];
-      }
+      for (int q = 0; q < 6; ++q) G[q] = gp[q * kGS];
       // D G D with the mirror signs folded into the off-diagonal entries
       const float sxy = sx * sy, sxz = sx * sz, syz = sy * sz;
       const float2 gxy = sxy * G[1], gxz = sxz * G[2], gyz = syz * G[4];
@@ -753,15 +751,12 @@ bool launch_line_tp64(LineArgs<double> a, cudaStream_t s) {
 }
 
 // fused z stage over the mirror groups [a.g0, a.g0 + groups) (P3 = 512, n3 <= 256)
-bool fused_tp_supported(const FusedArgs<float>& a, bool stored) {
-  return a.P3 == tp::kN && 2 * a.n3 <= tp::kN && (stored || a.octant != nullptr);
+bool fused_tp_supported(const FusedArgs<float>& a) {
+  return a.P3 == tp::kN && 2 * a.n3 <= tp::kN && (a.spec != nullptr || a.octant != nullptr);
 }
 
-void launch_fused_tp(const FusedArgs<float>& a, int groups, bool stored, cudaStream_t s) {
-  if (stored)
-    launch_pdl(tp::fused_tp_kernel<true>, dim3(groups), dim3(256), tp::kFusedSmem, s, a);
-  else
-    launch_pdl(tp::fused_tp_kernel<false>, dim3(groups), dim3(256), tp::kFusedSmem, s, a);
+void launch_fused_tp(const FusedArgs<float>& a, int groups, cudaStream_t s) {
+  launch_pdl(tp::fused_tp_kernel, dim3(groups), dim3(256), tp::kFusedSmem, s, a);
 }
 
 }  // namespace vie
@@ -781,8 +776,7 @@ int tp_init_attributes() {
   VIE_TPP_ATTR(true, false, false); VIE_TPP_ATTR(true, false, true);
   VIE_TPP_ATTR(true, true, false); VIE_TPP_ATTR(true, true, true);
 #undef VIE_TPP_ATTR
-  e = e != cudaSuccess ? e : cudaFuncSetAttribute(vie::tp::fused_tp_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, fs);
-  e = e != cudaSuccess ? e : cudaFuncSetAttribute(vie::tp::fused_tp_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, fs);
+  e = e != cudaSuccess ? e : cudaFuncSetAttribute(vie::tp::fused_tp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, fs);
   return e == cudaSuccess ? VIE_OK : cuda_status(e, "length-512 kernel attributes");
 }
 

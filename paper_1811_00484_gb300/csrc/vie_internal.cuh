@@ -351,6 +351,9 @@ void free_cp(vie_op* op);
 int build_operator(const vie_grid* grid, double tol, int rank_rule, int flags, cudaStream_t s,
                    vie_op** out);
 int assemble_spectrum(const vie_op* op, int c, double2* out, cudaStream_t s);
+// padded z edges 32 R that the tcgen05 rebuild and the Tucker+CP model accept
+bool lane_fft_edge(int P3);
+int plan_prepare(int N);     // kernel attributes of padded edge N (plan.cu)
 int op_tables(vie_op* op);   // FFT plans and root tables of op->P
 int line_fft_init_attributes();
 // persistent grid size for `kernel` with `threads` threads and `smem` bytes of

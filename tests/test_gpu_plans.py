@@ -1,0 +1,62 @@
+"""The planned matvec stages (factor plans of the padded edges, plan_table.h) against
+the oracle's FFT matvec: every radix pair class, odd and even edges, columns that are
+no multiple of a tile, batches, masks of the mirror groups at thin edges."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import embed, kernel, matvec
+
+vie = pytest.importorskip("paper_1811_00484_gb300")
+pytestmark = pytest.mark.gpu
+
+H, F = 5e-3, 298e6
+TOL_SVD = 1e-7
+
+
+def _field(n, B, seed, dtype):
+    rng = np.random.default_rng(seed)
+    a = rng.standard_normal((B, 3) + n) + 1j * rng.standard_normal((B, 3) + n)
+    return torch.from_numpy(a.astype(dtype)).cuda()
+
+
+def _rel(y, ref):
+    y = y.cpu().numpy().astype(np.complex128)
+    return np.linalg.norm(y - ref) / np.linalg.norm(ref)
+
+
+# (n1, n2, n3): every planned edge up to 128 once along some axis, a few beyond, and
+# edges without a plan (below 8) beside planned ones
+GRIDS = [(8, 9, 10), (12, 14, 15), (16, 18, 20), (21, 24, 25), (27, 28, 30), (32, 7, 35), (36, 40, 4),
+         (42, 3, 45), (48, 2, 49), (5, 50, 54), (56, 2, 60), (2, 63, 64), (70, 3, 72), (75, 2, 80),
+         (3, 81, 84), (90, 2, 96), (98, 2, 100), (2, 105, 108), (112, 2, 120), (2, 125, 126),
+         (128, 2, 12), (9, 2, 128), (135, 2, 8), (2, 8, 140), (2, 150, 9), (8, 2, 160)]
+
+
+@pytest.mark.parametrize("n", GRIDS)
+def test_planned_edges_match_the_oracle(n):
+    op = vie.Operator(n, H, F, TOL_SVD, store_uncompressed=True)
+    G = embed.green_spectra(kernel.toeplitz_tensor(*n, H, kernel.wavenumber(F)), *n)
+    J = _field(n, 3, 7, np.complex64)
+    Jh = J.cpu().numpy().astype(np.complex128)
+    ref = matvec.matvec_fft(G, Jh)
+    adj = matvec.matvec_fft(G, Jh.conj()).conj()              # G is complex symmetric
+    # FP32 rounding (1e-5, as for the other FP32 products) plus the truncation 4 tol
+    for path, tol in (("tucker", 1e-5 + 4 * TOL_SVD), ("uncompressed", 1e-5)):
+        assert _rel(op.matvec(J, path=path), ref) <= tol, path
+        assert _rel(op.matvec_adjoint(J, path=path), adj) <= tol, path
+    # a row of the batch equals the same current alone, bit for bit
+    assert torch.equal(op.matvec(J)[1:2], op.matvec(J[1:2].contiguous()))
+    op.close()
+
+
+@pytest.mark.parametrize("n", [(12, 10, 15), (20, 9, 7)])
+def test_ranks_beyond_the_rebuild_kernels(n):
+    """A tolerance that keeps every singular vector: the z stage rebuilds in the CTA
+    where the rebuild kernels' shared memory does not hold the ranks, and the product
+    still meets the FP32 bound."""
+    op = vie.Operator(n, H, F, 1e-14)
+    G = embed.green_spectra(kernel.toeplitz_tensor(*n, H, kernel.wavenumber(F)), *n)
+    J = _field(n, 2, 3, np.complex64)
+    assert _rel(op.matvec(J), matvec.matvec_fft(G, J.cpu().numpy().astype(np.complex128))) <= 1e-5
+    op.close()
