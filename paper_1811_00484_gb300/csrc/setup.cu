@@ -28,6 +28,8 @@
 #include <numeric>
 #include <vector>
 
+#include <cooperative_groups.h>
+
 #include "vie_internal.cuh"
 #include "stages.cuh"
 
@@ -35,52 +37,55 @@ namespace {
 
 constexpr double kPi = 3.14159265358979323846;
 
-__device__ __forceinline__ int circulant_offset(int i, int n, int P, bool* zero) {
-  if (i < n) return i;
-  if (i == n) { *zero = true; return 0; }
-  return i - P;
+// One component of h^3 (k0^2 delta_ab + d_a d_b) g at the voxel-centre offset
+// (o1, o2, o3) h, or the equivalent-sphere self term at zero offset.
+__device__ double2 dyadic_entry(int ca, int cb, int o1, int o2, int o3, double h, double k0, double2 self) {
+  if (o1 == 0 && o2 == 0 && o3 == 0) return ca == cb ? self : make_double2(0.0, 0.0);
+  const double R[3] = {o1 * h, o2 * h, o3 * h};
+  const double r = sqrt(R[0] * R[0] + R[1] * R[1] + R[2] * R[2]);
+  double sn, cs;
+  sincos(k0 * r, &sn, &cs);
+  const double inv4pir = 1.0 / (4.0 * kPi * r);
+  const double2 g = make_double2(cs * inv4pir, -sn * inv4pir);   // exp(-i k0 r)/(4 pi r)
+  const double ir = 1.0 / r;
+  const double2 diag = make_double2(k0 * k0 - ir * ir, -k0 * ir);
+  const double2 dyad = make_double2(-k0 * k0 + 3.0 * ir * ir, 3.0 * k0 * ir);
+  const double Ra = ca == 0 ? R[0] : (ca == 1 ? R[1] : R[2]), Rb = cb == 0 ? R[0] : (cb == 1 ? R[1] : R[2]);
+  const double rr = (Ra * ir) * (Rb * ir);
+  double2 f = make_double2(dyad.x * rr, dyad.y * rr);
+  if (ca == cb) f = f + diag;
+  return (h * h * h) * (g * f);
 }
 
-// One component of h^3 (k0^2 delta_ab + d_a d_b) g at the voxel-centre offset,
-// or the equivalent-sphere self term at zero offset, at every circulant index.
+// One component at every circulant index.  Each entry is evaluated once, at its
+// non-negative offsets, and written to its up to eight mirror images (an odd
+// coordinate flips the sign, exactly); index n of an axis holds zeros.  The
+// evaluation is bound by FP64 arithmetic (a sincos, a square root and two
+// divisions), so an eighth of the evaluations is an eighth of the time.
 __global__ void assemble_kernel(double2* out, int ca, int cb, int n1, int n2, int n3, int P1,
                                 int P2, int P3, double h, double k0, double2 self) {
-  const long long total = (long long)P1 * P2 * P3;
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
-       idx += (long long)gridDim.x * blockDim.x) {
-    const int i3 = (int)(idx % P3);
-    const int i2 = (int)((idx / P3) % P2);
-    const int i1 = (int)(idx / ((long long)P2 * P3));
-    bool zero = false;
-    const int o1 = circulant_offset(i1, n1, P1, &zero);
-    const int o2 = circulant_offset(i2, n2, P2, &zero);
-    const int o3 = circulant_offset(i3, n3, P3, &zero);
+  const unsigned total = (unsigned)(n1 + 1) * (n2 + 1) * (n3 + 1);
+  const double s1 = ((ca == 0) != (cb == 0)) ? -1.0 : 1.0, s2 = ((ca == 1) != (cb == 1)) ? -1.0 : 1.0,
+               s3 = ((ca == 2) != (cb == 2)) ? -1.0 : 1.0;
+  for (unsigned idx = blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += gridDim.x * blockDim.x) {
+    const int o3 = (int)(idx % (unsigned)(n3 + 1)), q = (int)(idx / (unsigned)(n3 + 1));
+    const int o2 = q % (n2 + 1), o1 = q / (n2 + 1);
     double2 v = make_double2(0.0, 0.0);
-    if (!zero) {
-      if (o1 == 0 && o2 == 0 && o3 == 0) {
-        if (ca == cb) v = self;
-      } else {
-        const double R[3] = {o1 * h, o2 * h, o3 * h};
-        const double r = sqrt(R[0] * R[0] + R[1] * R[1] + R[2] * R[2]);
-        double sn, cs;
-        sincos(k0 * r, &sn, &cs);
-        const double inv4pir = 1.0 / (4.0 * kPi * r);
-        const double2 g = make_double2(cs * inv4pir, -sn * inv4pir);   // exp(-i k0 r)/(4 pi r)
-        const double ir = 1.0 / r;
-        const double2 diag = make_double2(k0 * k0 - ir * ir, -k0 * ir);
-        const double2 dyad = make_double2(-k0 * k0 + 3.0 * ir * ir, 3.0 * k0 * ir);
-        const double rr = (R[ca] * ir) * (R[cb] * ir);
-        double2 f = make_double2(dyad.x * rr, dyad.y * rr);
-        if (ca == cb) f = f + diag;
-        v = (h * h * h) * (g * f);
-      }
-    }
-    out[idx] = v;
+    if (o1 < n1 && o2 < n2 && o3 < n3) v = dyadic_entry(ca, cb, o1, o2, o3, h, k0, self);
+    const int m1 = (o1 == 0 || o1 == n1) ? 1 : 2, m2 = (o2 == 0 || o2 == n2) ? 1 : 2,
+              m3 = (o3 == 0 || o3 == n3) ? 1 : 2;
+    for (int a = 0; a < m1; ++a)
+      for (int b = 0; b < m2; ++b)
+        for (int c = 0; c < m3; ++c) {
+          const int i1 = a ? P1 - o1 : o1, i2 = b ? P2 - o2 : o2, i3 = c ? P3 - o3 : o3;
+          const double sg = (a ? s1 : 1.0) * (b ? s2 : 1.0) * (c ? s3 : 1.0);
+          out[((long long)i1 * P2 + i2) * P3 + i3] = sg * v;
+        }
   }
 }
 
-// max |A[mirror] - s A| and max |A| over the tensor (non-negative doubles
-// compare like their bit patterns).
+// max |A[mirror] - s A|^2 and max |A|^2 over the tensor (non-negative doubles
+// compare like their bit patterns; no square root per entry).
 __global__ void parity_check_kernel(const double2* A, int P1, int P2, int P3, int s1, int s2, int s3,
                                     unsigned long long* out) {
   const long long total = (long long)P1 * P2 * P3;
@@ -94,13 +99,13 @@ __global__ void parity_check_kernel(const double2* A, int P1, int P2, int P3, in
     const double s = (double)(s1 * s2 * s3);
     const int m1 = (P1 - i1) % P1, m2 = (P2 - i2) % P2, m3 = (P3 - i3) % P3;
     const double2 b = A[((long long)m1 * P2 + m2) * P3 + m3];
-    dev = fmax(dev, sqrt(abs2(b - s * a)));
-    mx = fmax(mx, sqrt(abs2(a)));
+    dev = fmax(dev, abs2(b - s * a));
+    mx = fmax(mx, abs2(a));
     // single-axis mirrors
     const double2 bx = A[((long long)m1 * P2 + i2) * P3 + i3];
-    dev = fmax(dev, sqrt(abs2(bx - (double)s1 * a)));
+    dev = fmax(dev, abs2(bx - (double)s1 * a));
     const double2 by = A[((long long)i1 * P2 + m2) * P3 + i3];
-    dev = fmax(dev, sqrt(abs2(by - (double)s2 * a)));
+    dev = fmax(dev, abs2(by - (double)s2 * a));
   }
   for (int o = 16; o > 0; o >>= 1) {
     dev = fmax(dev, __shfl_down_sync(0xffffffffu, dev, o));
@@ -142,24 +147,7 @@ __global__ void toeplitz_octant_kernel(double2* out, int ca, int cb, int n1, int
     const int o3 = (int)(idx % n3);
     const int o2 = (int)((idx / n3) % n2);
     const int o1 = (int)(idx / ((long long)n2 * n3));
-    double2 v = make_double2(0.0, 0.0);
-    if (o1 == 0 && o2 == 0 && o3 == 0) {
-      if (ca == cb) v = self;
-    } else {
-      const double R[3] = {o1 * h, o2 * h, o3 * h};
-      const double r = sqrt(R[0] * R[0] + R[1] * R[1] + R[2] * R[2]);
-      double sn, cs;
-      sincos(k0 * r, &sn, &cs);
-      const double inv4pir = 1.0 / (4.0 * kPi * r);
-      const double2 g = make_double2(cs * inv4pir, -sn * inv4pir);
-      const double ir = 1.0 / r;
-      const double2 diag = make_double2(k0 * k0 - ir * ir, -k0 * ir);
-      const double2 dyad = make_double2(-k0 * k0 + 3.0 * ir * ir, 3.0 * k0 * ir);
-      const double rr = (R[ca] * ir) * (R[cb] * ir);
-      double2 f = make_double2(dyad.x * rr, dyad.y * rr);
-      if (ca == cb) f = f + diag;
-      v = (h * h * h) * (g * f);
-    }
+    const double2 v = dyadic_entry(ca, cb, o1, o2, o3, h, k0, self);
     double w = 1.0;
     if (o1 != 0) w *= r2;
     if (o2 != 0) w *= r2;
@@ -194,32 +182,67 @@ __global__ void to_c64_kernel(const double2* a, float2* b, long long n) {
     b[i] = make_float2((float)a[i].x, (float)a[i].y);
 }
 
-// element (i, m) of the mode-q unfolding of a D0 x D1 x D2 tensor
-__device__ __forceinline__ long long unfold_index(int q, int i, long long m, int D1, int D2) {
-  if (q == 0) return (long long)i * D1 * D2 + m;
-  if (q == 1) return (m / D2) * (long long)D1 * D2 + (long long)i * D2 + (m % D2);
+// element (i, m) of the mode-q unfolding of a D0 x D1 x D2 tensor (at most 513^3
+// entries: 32-bit indices)
+__device__ __forceinline__ unsigned unfold_index(int q, unsigned i, unsigned m, unsigned D1, unsigned D2) {
+  if (q == 0) return i * D1 * D2 + m;
+  if (q == 1) return (m / D2) * D1 * D2 + i * D2 + m % D2;
   return m * D2 + i;
 }
 
-// G = X X^* for the mode-q unfolding X (Dq x M), one 16 x 16 tile per CTA.
-__global__ void __launch_bounds__(256) gram_kernel(const double2* X, double2* G, int q, int D0, int D1,
-                                                   int D2) {
+// Partial Gram matrices part[z] = X_z X_z^* of the mode-q unfolding X (Dq x M),
+// X_z its z-th range of columns: one 16 x 16 tile of the upper triangle per CTA
+// and range.  FP64 arithmetic bounds it (2 fused multiply-adds per clock and SM),
+// so the column ranges are there to occupy every SM: with one CTA per tile and no
+// ranges, 25 CTAs of a 65^3 octant took 1.9 ms per mode.
+__global__ void __launch_bounds__(256) gram_kernel(const double2* __restrict__ X, double2* part, int q, int D0,
+                                                   int D1, int D2, int ntile, unsigned chunk) {
   __shared__ double2 Ai[16][17], Aj[16][17];
-  const int Dq = q == 0 ? D0 : (q == 1 ? D1 : D2);
-  const long long M = ((long long)D0 * D1 * D2) / Dq;
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int i0 = blockIdx.y * 16, j0 = blockIdx.x * 16;
+  const unsigned Dq = q == 0 ? D0 : (q == 1 ? D1 : D2);
+  const unsigned M = (unsigned)D0 * D1 * D2 / Dq;
+  int ti = 0, tj = blockIdx.x;                          // tile row ti <= tj
+  while (tj >= ntile - ti) {
+    tj -= ntile - ti;
+    ++ti;
+  }
+  tj += ti;
+  const unsigned tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  const unsigned i0 = ti * 16, j0 = tj * 16;
+  const unsigned mlo = blockIdx.y * chunk, mhi = min(M, mlo + chunk);
+  // consecutive threads read consecutive addresses: along m, or along i for mode 3
+  const unsigned li = q == 2 ? tx : ty, lm = q == 2 ? ty : tx;
   double2 acc = make_double2(0.0, 0.0);
-  for (long long m0 = 0; m0 < M; m0 += 16) {
-    const long long m = m0 + tx;
-    Ai[ty][tx] = (i0 + ty < Dq && m < M) ? X[unfold_index(q, i0 + ty, m, D1, D2)] : make_double2(0, 0);
-    Aj[ty][tx] = (j0 + ty < Dq && m < M) ? X[unfold_index(q, j0 + ty, m, D1, D2)] : make_double2(0, 0);
+  for (unsigned m0 = mlo; m0 < mhi; m0 += 16) {
+    const unsigned m = m0 + lm;
+    Ai[li][lm] = (i0 + li < Dq && m < mhi) ? X[unfold_index(q, i0 + li, m, D1, D2)] : make_double2(0, 0);
+    Aj[li][lm] = (j0 + li < Dq && m < mhi) ? X[unfold_index(q, j0 + li, m, D1, D2)] : make_double2(0, 0);
     __syncthreads();
 #pragma unroll
-    for (int k = 0; k < 16; ++k) acc = acc + Ai[ty][k] * conjg(Aj[tx][k]);
+    for (int k = 0; k < 16; ++k) {
+      const double2 u = Ai[ty][k], v = Aj[tx][k];       // acc += u conj(v)
+      acc.x = fma(u.x, v.x, fma(u.y, v.y, acc.x));
+      acc.y = fma(u.y, v.x, fma(-u.x, v.y, acc.y));
+    }
     __syncthreads();
   }
-  if (i0 + ty < Dq && j0 + tx < Dq) G[(long long)(i0 + ty) * Dq + j0 + tx] = acc;
+  if (i0 + ty < Dq && j0 + tx < Dq)
+    part[((size_t)blockIdx.y * Dq + i0 + ty) * Dq + j0 + tx] = acc;
+}
+
+// G = sum of the partial Gram matrices, in order; the lower triangle is the
+// conjugate of the upper one, the diagonal real
+__global__ void gram_sum_kernel(const double2* part, double2* G, int D, int nz) {
+  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < D * D; idx += gridDim.x * blockDim.x) {
+    const int i = idx / D, j = idx % D;
+    const bool up = i <= j;
+    const int src = up ? idx : j * D + i;
+    // tiles hold their whole 16 x 16 square, so (i, j) with i > j inside a diagonal
+    // tile exists too; the upper entry is used for both
+    double2 s = make_double2(0.0, 0.0);
+    for (int z = 0; z < nz; ++z) s = s + part[(size_t)z * D * D + src];
+    if (i == j) s.y = 0.0;
+    G[idx] = up ? s : conjg(s);
+  }
 }
 
 // out = in x_q M with M(i, t) = Mat[t * ld + i] (conjugated if cj):
@@ -249,103 +272,144 @@ struct JacobiJob {
   int m;
 };
 
-#define JACOBI_MAX_PAIRS 257
+// One rotation of a Jacobi step: columns p < q (q < 0: the index left over when m
+// is odd), new p' = c p - conj(s) q, q' = s p + c q; np, nq the rotated diagonal.
+struct JacobiRot {
+  double c, np, nq;
+  double2 s;
+  int p, q;
+};
 
-// Parallel cyclic Jacobi (round-robin pairing, all disjoint rotations of a
-// step applied at once), one CTA per matrix.  A pair (p, q) is rotated when
-// |a_pq| > tol sqrt(|a_pp a_qq|); the sweep loop stops after a sweep without
-// rotations or after max_sweeps (status -1).
-__global__ void __launch_bounds__(1024) jacobi_kernel(const JacobiJob* jobs, int max_sweeps,
-                                                      double tol, int* status) {
-  const JacobiJob job = jobs[blockIdx.x];
-  const int m = job.m;
-  const int mm = m + (m & 1);
-  const int M = mm - 1;
-  const int npair = mm / 2;
+constexpr int kJacobiCtas = 8;        // CTAs (one cluster) per matrix
+constexpr int kJacobiThreads = 256;
+constexpr int kJacobiMaxPairs = 257;
+
+// Parallel cyclic Jacobi (round-robin pairing, all disjoint rotations of a step
+// applied at once), one cluster of eight CTAs per matrix, every matrix of the
+// operator in one launch.  A pair (p, q) is rotated when |a_pq| > tol
+// sqrt(|a_pp a_qq|); the sweep loop stops after a sweep without rotations or
+// after max_sweeps (status -1).
+//
+// A step is bound by FP64 arithmetic (2 fused multiply-adds per clock and SM), so
+// it is spread over SMs and the Hermitian half is not computed: the rotations are
+// formed by the CTAs in turn and written into every CTA's shared memory
+// (distributed shared memory), then each 2 x 2 block (pair i, pair j >= i) of A is
+// rotated from both sides by one thread, which also writes its mirror image, and
+// each row of V by pairs.  Two cluster barriers a step.  A and V change hands
+// between SMs through L2.
+__global__ void __launch_bounds__(kJacobiThreads) jacobi_kernel(const JacobiJob* jobs, int max_sweeps,
+                                                                double tol, int* rotated, int* status) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int rank = (int)cluster.block_rank();
+  const int jobid = blockIdx.x / kJacobiCtas;
+  const JacobiJob job = jobs[jobid];
+  const int m = job.m, mm = m + (m & 1), M = mm - 1, npair = mm / 2;
   double2* A = job.A;
   double2* V = job.V;
-  __shared__ double cs[JACOBI_MAX_PAIRS];
-  __shared__ double2 se[JACOBI_MAX_PAIRS];
-  __shared__ int pp[JACOBI_MAX_PAIRS], qq[JACOBI_MAX_PAIRS];
-  __shared__ double dpp[JACOBI_MAX_PAIRS], dqq[JACOBI_MAX_PAIRS];
-  __shared__ int rotated;
-  const int tid = threadIdx.x, nth = blockDim.x;
-  for (long long e = tid; e < (long long)m * m; e += nth)
-    V[e] = make_double2((e / m) == (e % m) ? 1.0 : 0.0, 0.0);
-  __syncthreads();
+  __shared__ JacobiRot rot[kJacobiMaxPairs];
+  const int gt = rank * kJacobiThreads + threadIdx.x, gn = kJacobiCtas * kJacobiThreads;
+  for (int e = gt; e < m * m; e += gn) V[e] = make_double2((e / m) == (e % m) ? 1.0 : 0.0, 0.0);
+  cluster.sync();
   int sweep = 0;
   bool done = (m <= 1);
   for (; sweep < max_sweeps && !done; ++sweep) {
-    if (tid == 0) rotated = 0;
-    __syncthreads();
+    int* flag = rotated + jobid * max_sweeps + sweep;
     for (int step = 0; step < M; ++step) {
-      for (int i = tid; i < npair; i += nth) {
+      // this CTA's pairs: rank, rank + 8, ...
+      const int i = rank + kJacobiCtas * (int)threadIdx.x;
+      if (i < npair) {
         int p, q;
         if (i == 0) { p = 0; q = 1 + step; }
         else { p = 1 + (step + i) % M; q = 1 + (step - i + M) % M; }
         if (p > q) { int t = p; p = q; q = t; }
-        double c = 1.0;
-        double2 sv = make_double2(0.0, 0.0);
-        double np_ = 0.0, nq_ = 0.0;
+        JacobiRot r;
+        r.c = 1.0;
+        r.np = r.nq = 0.0;
+        r.s = make_double2(0.0, 0.0);
+        r.p = p;
+        r.q = q < m ? q : -1;
         if (q < m) {
-          const double app = A[(long long)p * m + p].x, aqq = A[(long long)q * m + q].x;
-          const double2 apq = A[(long long)p * m + q];
+          const double app = __ldcg(&A[p * m + p]).x, aqq = __ldcg(&A[q * m + q]).x;
+          const double2 apq = __ldcg(&A[p * m + q]);
           const double mag = sqrt(abs2(apq));
           if (mag > tol * sqrt(fabs(app * aqq)) && mag > 0.0) {
             const double th = (aqq - app) / (2.0 * mag);
             const double t = (th >= 0.0 ? 1.0 : -1.0) / (fabs(th) + sqrt(th * th + 1.0));
-            c = 1.0 / sqrt(t * t + 1.0);
-            const double s = t * c;
-            sv = make_double2(s * apq.x / mag, s * apq.y / mag);   // s e^{i phi}
-            np_ = app - t * mag;                                    // rotated diagonal
-            nq_ = aqq + t * mag;
-            rotated = 1;
+            r.c = 1.0 / sqrt(t * t + 1.0);
+            const double sm = t * r.c / mag;
+            r.s = make_double2(sm * apq.x, sm * apq.y);          // s e^{i phi}
+            r.np = app - t * mag;                                 // rotated diagonal
+            r.nq = aqq + t * mag;
+            *flag = 1;
           }
         }
-        cs[i] = c; se[i] = sv; pp[i] = p; qq[i] = q < m ? q : -1;
-        dpp[i] = np_; dqq[i] = nq_;
+        for (int k = 0; k < kJacobiCtas; ++k) cluster.map_shared_rank(rot, k)[i] = r;
       }
-      __syncthreads();
-      // A <- J^* A (rows p, q)
-      for (long long it = tid; it < (long long)npair * m; it += nth) {
-        const int i = (int)(it / m), k = (int)(it % m);
-        if (qq[i] < 0 || (se[i].x == 0.0 && se[i].y == 0.0)) continue;
-        const long long ip = (long long)pp[i] * m + k, iq = (long long)qq[i] * m + k;
-        const double2 ap = A[ip], aq = A[iq];
-        A[ip] = cs[i] * ap - se[i] * aq;
-        A[iq] = conjg(se[i]) * ap + cs[i] * aq;
+      cluster.sync();
+      // A <- J^* A J, the blocks (i, j >= i) and their mirror images
+      for (int it = gt; it < npair * npair; it += gn) {
+        const int bi = it / npair, bj = it - bi * npair;
+        if (bj < bi) continue;
+        const JacobiRot& ri = rot[bi];
+        const JacobiRot& rj = rot[bj];
+        const bool zi = ri.s.x == 0.0 && ri.s.y == 0.0, zj = rj.s.x == 0.0 && rj.s.y == 0.0;
+        if (zi && zj) continue;
+        if (bi == bj) {
+          // the rotation annihilates a_pq exactly and moves t|a_pq| between a_pp and
+          // a_qq; writing those values (instead of the rounded updates) lets the
+          // relative stopping test be met on graded matrices
+          A[ri.p * m + ri.p] = make_double2(ri.np, 0.0);
+          A[ri.q * m + ri.q] = make_double2(ri.nq, 0.0);
+          A[ri.p * m + ri.q] = make_double2(0.0, 0.0);
+          A[ri.q * m + ri.p] = make_double2(0.0, 0.0);
+          continue;
+        }
+        const double2 z = make_double2(0.0, 0.0);
+        const bool hi = ri.q >= 0, hj = rj.q >= 0;
+        double2 pp = __ldcg(&A[ri.p * m + rj.p]), pq = hj ? __ldcg(&A[ri.p * m + rj.q]) : z;
+        double2 qp = hi ? __ldcg(&A[ri.q * m + rj.p]) : z, qq = hi && hj ? __ldcg(&A[ri.q * m + rj.q]) : z;
+        if (!zi) {                                      // rows: p' = c p - s q, q' = conj(s) p + c q
+          const double2 ns = make_double2(-ri.s.x, -ri.s.y);
+          const double2 u = cmadd(ns, qp, ri.c * pp), v = conj_madd(ri.s, pp, ri.c * qp);
+          const double2 u2 = cmadd(ns, qq, ri.c * pq), v2 = conj_madd(ri.s, pq, ri.c * qq);
+          pp = u; qp = v; pq = u2; qq = v2;
+        }
+        if (!zj) {                                      // columns: p' = c p - conj(s) q, q' = s p + c q
+          const double2 ns = make_double2(-rj.s.x, -rj.s.y);
+          const double2 u = conj_madd(ns, pq, rj.c * pp), v = cmadd(rj.s, pp, rj.c * pq);
+          const double2 u2 = conj_madd(ns, qq, rj.c * qp), v2 = cmadd(rj.s, qp, rj.c * qq);
+          pp = u; pq = v; qp = u2; qq = v2;
+        }
+        A[ri.p * m + rj.p] = pp;
+        A[rj.p * m + ri.p] = conjg(pp);
+        if (hj) {
+          A[ri.p * m + rj.q] = pq;
+          A[rj.q * m + ri.p] = conjg(pq);
+        }
+        if (hi) {
+          A[ri.q * m + rj.p] = qp;
+          A[rj.p * m + ri.q] = conjg(qp);
+        }
+        if (hi && hj) {
+          A[ri.q * m + rj.q] = qq;
+          A[rj.q * m + ri.q] = conjg(qq);
+        }
       }
-      __syncthreads();
-      // A <- A J, V <- V J (columns p, q)
-      for (long long it = tid; it < (long long)npair * m; it += nth) {
-        const int i = (int)(it / m), k = (int)(it % m);
-        if (qq[i] < 0 || (se[i].x == 0.0 && se[i].y == 0.0)) continue;
-        const long long ip = (long long)k * m + pp[i], iq = (long long)k * m + qq[i];
-        const double2 ap = A[ip], aq = A[iq];
-        A[ip] = cs[i] * ap - conjg(se[i]) * aq;
-        A[iq] = se[i] * ap + cs[i] * aq;
-        const double2 vp = V[ip], vq = V[iq];
-        V[ip] = cs[i] * vp - conjg(se[i]) * vq;
-        V[iq] = se[i] * vp + cs[i] * vq;
+      // V <- V J
+      for (int it = gt; it < npair * m; it += gn) {
+        const int k = it / npair, bj = it - k * npair;
+        const JacobiRot& rj = rot[bj];
+        if (rj.q < 0 || (rj.s.x == 0.0 && rj.s.y == 0.0)) continue;
+        const double2 vp = __ldcg(&V[k * m + rj.p]), vq = __ldcg(&V[k * m + rj.q]);
+        V[k * m + rj.p] = conj_madd(make_double2(-rj.s.x, -rj.s.y), vq, rj.c * vp);
+        V[k * m + rj.q] = cmadd(rj.s, vp, rj.c * vq);
       }
-      __syncthreads();
-      // the rotation annihilates a_pq exactly and moves t|a_pq| between a_pp and a_qq;
-      // writing those values (instead of the rounded updates) lets the relative
-      // stopping test be met on graded matrices
-      for (int i = tid; i < npair; i += nth) {
-        if (qq[i] < 0 || (se[i].x == 0.0 && se[i].y == 0.0)) continue;
-        const long long p = pp[i], q = qq[i];
-        A[p * m + q] = make_double2(0.0, 0.0);
-        A[q * m + p] = make_double2(0.0, 0.0);
-        A[p * m + p] = make_double2(dpp[i], 0.0);
-        A[q * m + q] = make_double2(dqq[i], 0.0);
-      }
-      __syncthreads();
+      cluster.sync();
     }
-    done = (rotated == 0);
-    __syncthreads();
+    done = __ldcg(flag) == 0;            // the same for every CTA: set before the last barrier
   }
-  if (tid == 0) status[blockIdx.x] = done ? sweep : -1;
+  if (rank == 0 && threadIdx.x == 0) status[jobid] = done ? sweep : -1;
 }
 
 int grid_for(long long n) {
@@ -376,22 +440,40 @@ template <typename P> int dalloc(P** p, size_t bytes) {
 }
 
 struct DeviceBuffers {
-  double2* full = nullptr;    // P1 P2 P3
-  double2* aw = nullptr;      // H1 H2 H3
-  double2* tmp = nullptr;     // H1 H2 H3
-  double2* gram[3] = {};      // Hq x Hq
-  double2* vec[3] = {};       // Hq x Hq
-  double2* vec2[3] = {};      // Hq x Hq
-  double2* ytr = nullptr;     // truncated Y, max Hq x Hq
-  JacobiJob* jobs = nullptr;
-  int* jstatus = nullptr;
-  unsigned long long* red = nullptr;
+  double2* full = nullptr;       // P1 P2 P3
+  double2* aw[6] = {};           // H1 H2 H3: every component's weighted octant
+  double2* tmp = nullptr;        // H1 H2 H3
+  double2* gram[6][3] = {};      // Hq x Hq
+  double2* vec[6][3] = {};       // Hq x Hq
+  double2* vec2[6][3] = {};      // Hq x Hq
+  double2* ytr = nullptr;        // truncated Y, max Hq x Hq
+  double2* part = nullptr;       // partial Gram matrices
+  size_t part_entries = 0;
+  JacobiJob* jobs = nullptr;     // [18]
+  int* jstatus = nullptr;        // [18], then the sweeps' rotation flags [18][kJacobiSweeps]
+  unsigned long long* red = nullptr;   // [6][2]
   ~DeviceBuffers() {
-    cudaFree(full); cudaFree(aw); cudaFree(tmp);
-    for (int q = 0; q < 3; ++q) { cudaFree(gram[q]); cudaFree(vec[q]); cudaFree(vec2[q]); }
-    cudaFree(ytr); cudaFree(jobs); cudaFree(jstatus); cudaFree(red);
+    cudaFree(full); cudaFree(tmp); cudaFree(ytr); cudaFree(part);
+    for (int c = 0; c < 6; ++c) {
+      cudaFree(aw[c]);
+      for (int q = 0; q < 3; ++q) { cudaFree(gram[c][q]); cudaFree(vec[c][q]); cudaFree(vec2[c][q]); }
+    }
+    cudaFree(jobs); cudaFree(jstatus); cudaFree(red);
   }
 };
+
+constexpr int kJacobiSweeps = 60;
+
+// upper-triangle 16 x 16 tiles of a D x D Gram matrix, and its column ranges: enough
+// CTAs for about four per SM
+int gram_tiles(int D) {
+  const int n = (D + 15) / 16;
+  return n * (n + 1) / 2;
+}
+int gram_ranges(int D, long long M) {
+  const long long want = (4LL * device_sms() + gram_tiles(D) - 1) / gram_tiles(D);
+  return (int)std::max<long long>(1, std::min<long long>(want, (M + 255) / 256));
+}
 
 }  // namespace
 
@@ -472,19 +554,43 @@ static int init_tables(vie_op* op) {
   return VIE_OK;
 }
 
-static int run_jacobi(DeviceBuffers& d, double2* const* A, double2* const* V, const int* m, int njobs,
-                      cudaStream_t s) {
-  JacobiJob jobs[3];
-  for (int j = 0; j < njobs; ++j) jobs[j] = JacobiJob{A[j], V[j], m[j]};
-  VIE_CUDA(cudaMemcpyAsync(d.jobs, jobs, njobs * sizeof(JacobiJob), cudaMemcpyHostToDevice, s));
-  jacobi_kernel<<<njobs, 1024, 0, s>>>(d.jobs, 60, 1e-15, d.jstatus);
-  VIE_CUDA(cudaGetLastError());
-  int st[3];
-  VIE_CUDA(cudaMemcpyAsync(st, d.jstatus, njobs * sizeof(int), cudaMemcpyDeviceToHost, s));
+// Gram matrix of the mode-q unfolding of an H[0] x H[1] x H[2] tensor
+static void launch_gram(DeviceBuffers& d, const double2* X, double2* G, int q, const int* H, cudaStream_t s) {
+  const int D = H[q], n = (D + 15) / 16;
+  const long long M = (long long)H[0] * H[1] * H[2] / D;
+  const int nz = gram_ranges(D, M);
+  const unsigned chunk = (unsigned)(((M + nz - 1) / nz + 15) / 16 * 16);
+  gram_kernel<<<dim3(gram_tiles(D), nz), 256, 0, s>>>(X, d.part, q, H[0], H[1], H[2], n, chunk);
+  gram_sum_kernel<<<grid_for((long long)D * D), 256, 0, s>>>(d.part, G, D, nz);
+}
+
+// Diagonalise the 18 Gram matrices (6 components x 3 modes) in one launch.
+static int run_jacobi(DeviceBuffers& d, double2* (&V)[6][3], const int* H, cudaStream_t s) {
+  constexpr int kJobs = 18;
+  JacobiJob jobs[kJobs];
+  for (int j = 0; j < kJobs; ++j) jobs[j] = JacobiJob{d.gram[j / 3][j % 3], V[j / 3][j % 3], H[j % 3]};
+  int* flags = d.jstatus + kJobs;
+  VIE_CUDA(cudaMemcpyAsync(d.jobs, jobs, sizeof(jobs), cudaMemcpyHostToDevice, s));
+  VIE_CUDA(cudaMemsetAsync(flags, 0, kJobs * kJacobiSweeps * sizeof(int), s));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kJobs * kJacobiCtas);
+  cfg.blockDim = dim3(kJacobiThreads);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = kJacobiCtas;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  VIE_CUDA(cudaLaunchKernelEx(&cfg, jacobi_kernel, (const JacobiJob*)d.jobs, (int)kJacobiSweeps, 1e-15, flags,
+                              d.jstatus));
+  int st[kJobs];
+  VIE_CUDA(cudaMemcpyAsync(st, d.jstatus, sizeof(st), cudaMemcpyDeviceToHost, s));
   VIE_CUDA(cudaStreamSynchronize(s));
-  for (int j = 0; j < njobs; ++j) {
+  for (int j = 0; j < kJobs; ++j) {
     if (st[j] < 0) {
-      set_error("Jacobi eigen-solver did not converge (matrix %d, size %d)", j, m[j]);
+      set_error("Jacobi eigen-solver did not converge (component %d, matrix %d, size %d)", j / 3, j % 3,
+                H[j % 3]);
       return VIE_ERR_NUMERIC;
     }
   }
@@ -509,95 +615,121 @@ static size_t rank_from_sigma2(const std::vector<double>& s2, double tol, int ru
   return H;
 }
 
-// Compress one component; fills op->comp[c].  Spectrum route: Algorithm 1 on
+// Compression of the six components (op->comp).  Spectrum route: Algorithm 1 on
 // the weighted octant of the FFT'd circulant component.  Factor-wise route
 // (VIE_SETUP_FACTORWISE, Section V.A): Algorithm 1 on the weighted octant of
 // the Toeplitz defining tensor, then the embedding and DFT of each factor
 // column; F_q E_q / sqrt(P_q) is an isometry, so both routes give the same
 // ranks and the same truncated model (core scaled by sqrt(P1 P2 P3)).
-static int compress_component(vie_op* op, int c, double tol, int rule, DeviceBuffers& d,
-                              cudaStream_t s, bool factorwise) {
+// The components go through each stage together, so that the eigen-solver, a
+// long chain on few SMs per matrix, runs once per pass on all 18 matrices.
+
+// dimensions of the weighted octant the HOSVD runs on
+static void octant_dims(const vie_op* op, bool factorwise, int* H) {
+  for (int q = 0; q < 3; ++q) H[q] = factorwise ? op->n[q] : op->H[q];
+}
+
+// weighted octant of component c into d.aw[c]; its parity check into d.red[2 c]
+static int component_octant(vie_op* op, int c, DeviceBuffers& d, cudaStream_t s, bool factorwise) {
   const int P1 = op->P[0], P2 = op->P[1], P3 = op->P[2];
-  // dimensions of the weighted octant the HOSVD runs on
-  const int H[3] = {factorwise ? op->n[0] : op->H[0], factorwise ? op->n[1] : op->H[1],
-                    factorwise ? op->n[2] : op->H[2]};
+  int H[3];
+  octant_dims(op, factorwise, H);
   const long long full = (long long)P1 * P2 * P3;
   const long long oct = (long long)H[0] * H[1] * H[2];
   TuckerComp& tc = op->comp[c];
   for (int q = 0; q < 3; ++q) tc.s[q] = component_parity(c, q);
-  const bool need_spectrum = !factorwise || op->spec64 != nullptr;
-
-  if (need_spectrum) {
+  if (!factorwise || op->spec64 != nullptr) {
     VIE_TRY(assemble_spectrum(op, c, d.full, s));
-
     // the symmetry every later step relies on
-    VIE_CUDA(cudaMemsetAsync(d.red, 0, 2 * sizeof(unsigned long long), s));
     parity_check_kernel<<<grid_for(full), 256, 0, s>>>(d.full, P1, P2, P3, tc.s[0], tc.s[1], tc.s[2],
-                                                        d.red);
-    unsigned long long red[2];
-    VIE_CUDA(cudaMemcpyAsync(red, d.red, sizeof(red), cudaMemcpyDeviceToHost, s));
-    VIE_CUDA(cudaStreamSynchronize(s));
-    double dev, mx;
-    std::memcpy(&dev, &red[0], 8);
-    std::memcpy(&mx, &red[1], 8);
-    if (!(dev <= 1e-9 * mx + 1e-300) || !std::isfinite(mx)) {
-      set_error("component %d spectrum breaks its mirror symmetry (%.3e of %.3e)", c, dev, mx);
-      return VIE_ERR_NUMERIC;
-    }
-
+                                                        d.red + 2 * c);
     if (op->spec64) {
       VIE_CUDA(cudaMemcpyAsync(op->spec64 + c * full, d.full, full * sizeof(double2),
                                cudaMemcpyDeviceToDevice, s));
       to_c64_kernel<<<grid_for(full), 256, 0, s>>>(d.full, op->spec32 + c * full, full);
     }
   }
-
   if (!factorwise) {
-    octant_kernel<<<grid_for(oct), 256, 0, s>>>(d.full, d.aw, P1, P2, P3, H[0], H[1], H[2]);
+    octant_kernel<<<grid_for(oct), 256, 0, s>>>(d.full, d.aw[c], P1, P2, P3, H[0], H[1], H[2]);
   } else {
     int ca, cb;
     component_axes(c, &ca, &cb);
-    toeplitz_octant_kernel<<<grid_for(oct), 256, 0, s>>>(d.aw, ca, cb, H[0], H[1], H[2], op->grid.h,
+    toeplitz_octant_kernel<<<grid_for(oct), 256, 0, s>>>(d.aw[c], ca, cb, H[0], H[1], H[2], op->grid.h,
                                                           op->k0, self_term_value(op));
   }
+  VIE_CUDA(cudaGetLastError());
+  return VIE_OK;
+}
 
+// Both eigen-solver passes of every component: d.vec and d.vec2 hold the
+// eigenvectors Y and V2, the diagonals of d.gram the squared singular values.
+static int component_eigenvectors(vie_op* op, DeviceBuffers& d, cudaStream_t s, bool factorwise) {
+  int H[3];
+  octant_dims(op, factorwise, H);
+  const long long oct = (long long)H[0] * H[1] * H[2];
+  VIE_CUDA(cudaMemsetAsync(d.red, 0, 12 * sizeof(unsigned long long), s));
   // pass 1: Gram matrices of the three unfoldings and their eigenvectors Y
-  for (int q = 0; q < 3; ++q) {
-    dim3 g((H[q] + 15) / 16, (H[q] + 15) / 16);
-    gram_kernel<<<g, 256, 0, s>>>(d.aw, d.gram[q], q, H[0], H[1], H[2]);
+  for (int c = 0; c < 6; ++c) {
+    VIE_TRY(component_octant(op, c, d, s, factorwise));
+    for (int q = 0; q < 3; ++q) launch_gram(d, d.aw[c], d.gram[c][q], q, H, s);
   }
   VIE_CUDA(cudaGetLastError());
-  VIE_TRY(run_jacobi(d, d.gram, d.vec, H, 3, s));
-
+  if (!factorwise || op->spec64 != nullptr) {
+    unsigned long long red[12];
+    VIE_CUDA(cudaMemcpyAsync(red, d.red, sizeof(red), cudaMemcpyDeviceToHost, s));
+    VIE_CUDA(cudaStreamSynchronize(s));
+    for (int c = 0; c < 6; ++c) {
+      double dev, mx;
+      std::memcpy(&dev, &red[2 * c], 8);
+      std::memcpy(&mx, &red[2 * c + 1], 8);
+      dev = std::sqrt(dev);
+      mx = std::sqrt(mx);
+      if (!(dev <= 1e-9 * mx + 1e-300) || !std::isfinite(mx)) {
+        set_error("component %d spectrum breaks its mirror symmetry (%.3e of %.3e)", c, dev, mx);
+        return VIE_ERR_NUMERIC;
+      }
+    }
+  }
+  VIE_TRY(run_jacobi(d, d.vec, H, s));
   // pass 2: Gram of Y^* A_w^(q), eigenvectors V2; final vectors Y V2
-  for (int q = 0; q < 3; ++q) {
-    const long long Dpre = q == 0 ? 1 : (q == 1 ? H[0] : (long long)H[0] * H[1]);
-    const long long Dpost = q == 0 ? (long long)H[1] * H[2] : (q == 1 ? H[2] : 1);
-    mode_product_kernel<<<grid_for(oct), 256, 0, s>>>(d.aw, d.tmp, d.vec[q], H[q], 1, Dpre, H[q],
-                                                      Dpost, H[q]);
-    dim3 g((H[q] + 15) / 16, (H[q] + 15) / 16);
-    gram_kernel<<<g, 256, 0, s>>>(d.tmp, d.gram[q], q, H[0], H[1], H[2]);
+  for (int c = 0; c < 6; ++c) {
+    for (int q = 0; q < 3; ++q) {
+      const long long Dpre = q == 0 ? 1 : (q == 1 ? H[0] : (long long)H[0] * H[1]);
+      const long long Dpost = q == 0 ? (long long)H[1] * H[2] : (q == 1 ? H[2] : 1);
+      mode_product_kernel<<<grid_for(oct), 256, 0, s>>>(d.aw[c], d.tmp, d.vec[c][q], H[q], 1, Dpre, H[q],
+                                                        Dpost, H[q]);
+      launch_gram(d, d.tmp, d.gram[c][q], q, H, s);
+    }
   }
   VIE_CUDA(cudaGetLastError());
-  VIE_TRY(run_jacobi(d, d.gram, d.vec2, H, 3, s));
+  return run_jacobi(d, d.vec2, H, s);
+}
+
+// Ranks, core and stored factors of component c from its eigenvectors.
+static int compress_component(vie_op* op, int c, double tol, int rule, DeviceBuffers& d,
+                              cudaStream_t s, bool factorwise) {
+  const int P1 = op->P[0], P2 = op->P[1], P3 = op->P[2];
+  int H[3];
+  octant_dims(op, factorwise, H);
+  TuckerComp& tc = op->comp[c];
 
   // sort pass-2 eigenvalues, pick ranks, form Y V2 restricted to the kept columns
   double norm2 = 0.0;
   std::vector<double2> Ytr[3];
   for (int q = 0; q < 3; ++q) {
     const int h = H[q];
-    std::vector<double2> G2((size_t)h * h), YV((size_t)h * h);
-    VIE_CUDA(cudaMemcpyAsync(G2.data(), d.gram[q], G2.size() * sizeof(double2),
-                             cudaMemcpyDeviceToHost, s));
+    std::vector<double2> G2(h), YV((size_t)h * h);             // G2: the diagonal
+    VIE_CUDA(cudaMemcpy2DAsync(G2.data(), sizeof(double2), d.gram[c][q], (h + 1) * sizeof(double2),
+                               sizeof(double2), h, cudaMemcpyDeviceToHost, s));
     // Y V2: view Y as [h][h][1] and contract its second index with V2
-    mode_product_kernel<<<grid_for((long long)h * h), 256, 0, s>>>(d.vec[q], d.ytr, d.vec2[q], h,
+    mode_product_kernel<<<grid_for((long long)h * h), 256, 0, s>>>(d.vec[c][q], d.ytr, d.vec2[c][q], h,
                                                                    0, h, h, 1, h);
     VIE_CUDA(cudaGetLastError());
     VIE_CUDA(cudaMemcpyAsync(YV.data(), d.ytr, YV.size() * sizeof(double2), cudaMemcpyDeviceToHost,
                              s));
     VIE_CUDA(cudaStreamSynchronize(s));
     std::vector<double> lam(h);
-    for (int j = 0; j < h; ++j) lam[j] = std::max(G2[(size_t)j * h + j].x, 0.0);
+    for (int j = 0; j < h; ++j) lam[j] = std::max(G2[j].x, 0.0);
     std::vector<int> order(h);
     std::iota(order.begin(), order.end(), 0);
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return lam[a] > lam[b]; });
@@ -626,14 +758,14 @@ static int compress_component(vie_op* op, int c, double tol, int rule, DeviceBuf
   // core = A_w x1 Y1^* x2 Y2^* x3 Y3^*  (the truncated Y's go to d.vec2)
   const int r1 = tc.r[0], r2 = tc.r[1], r3 = tc.r[2];
   for (int q = 0; q < 3; ++q)
-    VIE_CUDA(cudaMemcpy(d.vec2[q], Ytr[q].data(), Ytr[q].size() * sizeof(double2),
+    VIE_CUDA(cudaMemcpy(d.vec2[c][q], Ytr[q].data(), Ytr[q].size() * sizeof(double2),
                         cudaMemcpyHostToDevice));
   mode_product_kernel<<<grid_for((long long)r1 * H[1] * H[2]), 256, 0, s>>>(
-      d.aw, d.tmp, d.vec2[0], r1, 1, 1, H[0], (long long)H[1] * H[2], r1);
+      d.aw[c], d.tmp, d.vec2[c][0], r1, 1, 1, H[0], (long long)H[1] * H[2], r1);
   mode_product_kernel<<<grid_for((long long)r1 * r2 * H[2]), 256, 0, s>>>(
-      d.tmp, d.aw, d.vec2[1], r2, 1, r1, H[1], H[2], r2);
+      d.tmp, d.aw[c], d.vec2[c][1], r2, 1, r1, H[1], H[2], r2);
   mode_product_kernel<<<grid_for((long long)r1 * r2 * r3), 256, 0, s>>>(
-      d.aw, d.tmp, d.vec2[2], r3, 1, (long long)r1 * r2, H[2], 1, r3);
+      d.aw[c], d.tmp, d.vec2[c][2], r3, 1, (long long)r1 * r2, H[2], 1, r3);
   VIE_CUDA(cudaGetLastError());
   const size_t ncore = (size_t)r1 * r2 * r3;
   VIE_TRY(dalloc(&tc.core64, ncore * sizeof(double2)));
@@ -788,26 +920,35 @@ int build_operator(const vie_grid* grid, double tol, int rank_rule, int flags, c
     const bool factorwise = (flags & VIE_SETUP_FACTORWISE) != 0;
     // the P1 P2 P3 spectrum is formed only on the spectrum route or to be stored
     const bool need_full = !factorwise || (flags & VIE_STORE_UNCOMPRESSED);
+    int H[3];
+    octant_dims(op, factorwise, H);
+    const long long aw = (long long)H[0] * H[1] * H[2];
+    for (int q = 0; q < 3; ++q)
+      d.part_entries = std::max(d.part_entries, (size_t)gram_ranges(H[q], aw / H[q]) * H[q] * H[q]);
+    const size_t tmp = (size_t)std::max(oct, (long long)hmax * hmax);
+    op->setup_scratch_bytes = ((need_full ? (size_t)full : 0) + 6 * (size_t)aw + tmp + (size_t)hmax * hmax +
+                               d.part_entries) * sizeof(double2);
     if ((need_full && (st = dalloc(&d.full, full * sizeof(double2))) != VIE_OK) ||
-        (st = dalloc(&d.aw, oct * sizeof(double2))) != VIE_OK ||
-        (st = dalloc(&d.tmp, std::max(oct, (long long)hmax * hmax) * sizeof(double2))) != VIE_OK ||
+        (st = dalloc(&d.tmp, tmp * sizeof(double2))) != VIE_OK ||
         (st = dalloc(&d.ytr, (size_t)hmax * hmax * sizeof(double2))) != VIE_OK ||
-        (st = dalloc(&d.jobs, 3 * sizeof(JacobiJob))) != VIE_OK ||
-        (st = dalloc(&d.jstatus, 3 * sizeof(int))) != VIE_OK ||
-        (st = dalloc(&d.red, 2 * sizeof(unsigned long long))) != VIE_OK) {
+        (st = dalloc(&d.part, d.part_entries * sizeof(double2))) != VIE_OK ||
+        (st = dalloc(&d.jobs, 18 * sizeof(JacobiJob))) != VIE_OK ||
+        (st = dalloc(&d.jstatus, 18 * (1 + kJacobiSweeps) * sizeof(int))) != VIE_OK ||
+        (st = dalloc(&d.red, 12 * sizeof(unsigned long long))) != VIE_OK) {
       vie_destroy(op);
       return st;
     }
-    op->setup_scratch_bytes =
-        (need_full ? full * sizeof(double2) : 0) + oct * sizeof(double2) +
-        std::max(oct, (long long)hmax * hmax) * sizeof(double2) + (size_t)hmax * hmax * sizeof(double2);
-    for (int q = 0; q < 3; ++q) op->setup_scratch_bytes += 3 * (size_t)op->H[q] * op->H[q] * sizeof(double2);
-    for (int q = 0; q < 3 && st == VIE_OK; ++q) {
-      const size_t hh = (size_t)op->H[q] * op->H[q] * sizeof(double2);
-      if ((st = dalloc(&d.gram[q], hh)) != VIE_OK || (st = dalloc(&d.vec[q], hh)) != VIE_OK ||
-          (st = dalloc(&d.vec2[q], hh)) != VIE_OK)
-        break;
+    for (int c = 0; c < 6 && st == VIE_OK; ++c) {
+      st = dalloc(&d.aw[c], aw * sizeof(double2));
+      for (int q = 0; q < 3 && st == VIE_OK; ++q) {
+        const size_t hh = (size_t)H[q] * H[q] * sizeof(double2);
+        if ((st = dalloc(&d.gram[c][q], hh)) != VIE_OK || (st = dalloc(&d.vec[c][q], hh)) != VIE_OK ||
+            (st = dalloc(&d.vec2[c][q], hh)) != VIE_OK)
+          break;
+        op->setup_scratch_bytes += 3 * hh;
+      }
     }
+    if (st == VIE_OK) st = component_eigenvectors(op, d, s, factorwise);
     for (int c = 0; c < 6 && st == VIE_OK; ++c)
       st = compress_component(op, c, tol, rank_rule, d, s, factorwise);
     if (st == VIE_OK) {
