@@ -662,6 +662,10 @@ template <typename T, bool STORED>
 static int launch_fused_impl(FusedArgs<T> a, cudaStream_t s) {
   if constexpr (sizeof(T) == 4) {
     if (launch_fused_fast(a, s)) return VIE_OK;
+  } else {
+    ProfScope ps(PF_MATVEC64, s);
+    a.prof = nullptr;
+    if (launch_plan_fused(a, 0, a.H1, s)) return VIE_OK;
   }
   const size_t limit = 227 * 1024;
   int LR = 4;

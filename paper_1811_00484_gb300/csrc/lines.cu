@@ -94,10 +94,10 @@ void launch_line_fft(const LineArgs<T>& a, cudaStream_t s) {
     // length 512: the persistent TMA-fed kernel (x + y + their inverses of eight
     // 256^3 right-hand sides 12.4 ms; 32 x 16 of the planned kernel 14.8 ms)
     if (a.plan.N == 512 && launch_line_tp(a, s)) return;
-    if (launch_plan_line(a, s)) return;
   } else {
     if (a.plan.N == 512 && launch_line_tp64(a, s)) return;
   }
+  if (launch_plan_line(a, s)) return;
   const int N = a.plan.N;
   auto bytes = [&](int tw) { return (size_t)(2 * N * tw + N) * sizeof(cx<T>); };
   const size_t limit = 227 * 1024;

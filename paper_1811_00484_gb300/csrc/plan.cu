@@ -5,13 +5,20 @@
 namespace vie {
 namespace plan {
 
+// defined in the sets' own translation units
+template <typename T, int K> bool line_set(const LineArgs<T>& a, cudaStream_t s);
+template <typename T, int K> bool fused_set(const FusedArgs<T>& a, int k10, int nk1, cudaStream_t s);
+template <typename T, int K> cudaError_t prepare_set(int N);
+
 #define VIE_SETS(X) X(0) X(1) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9)
-#define VIE_DECL(K)                                                                  \
-  bool line_set##K(const LineArgs<float>& a, cudaStream_t s);                        \
-  bool fused_set##K(const FusedArgs<float>& a, int k10, int nk1, cudaStream_t s);    \
-  bool prepare_set##K(int N, cudaError_t* e);
+#define VIE_DECL_T(T, K)                                                              \
+  template <> bool line_set<T, K>(const LineArgs<T>&, cudaStream_t);                  \
+  template <> bool fused_set<T, K>(const FusedArgs<T>&, int, int, cudaStream_t);      \
+  template <> cudaError_t prepare_set<T, K>(int);
+#define VIE_DECL(K) VIE_DECL_T(float, K) VIE_DECL_T(double, K)
 VIE_SETS(VIE_DECL)
 #undef VIE_DECL
+#undef VIE_DECL_T
 
 static int set_of(int N) {
   switch (N) {
@@ -38,15 +45,18 @@ bool plan_exists(int N) { return plan::set_of(N) >= 0; }
 // Line stage of a planned length: the matvec's half-length transforms (forward
 // from N / 2 points, inverse cropped to N / 2) of adjacent columns.  Everything
 // else is left to the general kernel.
-bool launch_plan_line(const LineArgs<float>& a, cudaStream_t s) {
+template <typename T> bool launch_plan_line(const LineArgs<T>& a, cudaStream_t s) {
   const int N = a.plan.N;
   if (a.in_cs != 1 || a.out_cs != 1) return false;
   if ((a.flags & (PRO_CHI | EPI_CHI)) && a.chi_cs != 1) return false;
   if (a.inverse ? (a.lin != N || 2 * a.lout != N) : (2 * a.lin != N || a.lout != N)) return false;
   if (a.nother > 65535 || a.nbatch > 65535) return false;
+  // 32-bit element offsets inside one batch entry
+  const long long lim = 1LL << 31;
+  if (a.in_bs >= lim || a.out_bs >= lim) return false;
   switch (plan::set_of(N)) {
 #define VIE_CASE(K) \
-  case K: return plan::line_set##K(a, s);
+  case K: return plan::line_set<T, K>(a, s);
     VIE_SETS(VIE_CASE)
 #undef VIE_CASE
     default: return false;
@@ -54,16 +64,21 @@ bool launch_plan_line(const LineArgs<float>& a, cudaStream_t s) {
 }
 
 // Fused z stage of the groups k1 in [k10, k10 + nk1), every k2
-bool launch_plan_fused(const FusedArgs<float>& a, int k10, int nk1, cudaStream_t s) {
+template <typename T> bool launch_plan_fused(const FusedArgs<T>& a, int k10, int nk1, cudaStream_t s) {
   if (2 * a.n3 != a.P3 || nk1 > 65535) return false;
   switch (plan::set_of(a.P3)) {
 #define VIE_CASE(K) \
-  case K: return plan::fused_set##K(a, k10, nk1, s);
+  case K: return plan::fused_set<T, K>(a, k10, nk1, s);
     VIE_SETS(VIE_CASE)
 #undef VIE_CASE
     default: return false;
   }
 }
+
+template bool launch_plan_line<float>(const LineArgs<float>&, cudaStream_t);
+template bool launch_plan_line<double>(const LineArgs<double>&, cudaStream_t);
+template bool launch_plan_fused<float>(const FusedArgs<float>&, int, int, cudaStream_t);
+template bool launch_plan_fused<double>(const FusedArgs<double>&, int, int, cudaStream_t);
 
 }  // namespace vie
 
@@ -73,7 +88,10 @@ int plan_prepare(int N) {
   cudaError_t e = cudaSuccess;
   switch (vie::plan::set_of(N)) {
 #define VIE_CASE(K) \
-  case K: vie::plan::prepare_set##K(N, &e); break;
+  case K:                                                  \
+    e = vie::plan::prepare_set<float, K>(N);               \
+    if (e == cudaSuccess) e = vie::plan::prepare_set<double, K>(N); \
+    break;
     VIE_SETS(VIE_CASE)
 #undef VIE_CASE
     default: break;

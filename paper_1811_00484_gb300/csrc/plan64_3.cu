@@ -1,0 +1,5 @@
+// Matvec stages of the edges in VIE_PLAN_SET_3 (plan_table.h), FP64.
+#define VIE_SET 3
+#define VIE_SET_T double
+#define VIE_SET_SIZES VIE_PLAN_SET_3
+#include "plan_set.cuh"

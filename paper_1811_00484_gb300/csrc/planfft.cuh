@@ -38,118 +38,141 @@
 namespace vie {
 namespace plan {
 
+// one set of plan_table.h (plan_set.cuh); false when the edge is not in it
+template <typename T, int K> bool line_set(const LineArgs<T>& a, cudaStream_t s);
+template <typename T, int K> bool fused_set(const FusedArgs<T>& a, int k10, int nk1, cudaStream_t s);
+template <typename T, int K> cudaError_t prepare_set(int N);
+
 __host__ __device__ constexpr int imax(int a, int b) { return a > b ? a : b; }
 
 // ---------------------------------------------------------------------------
 // line stage
 // ---------------------------------------------------------------------------
+// Threads per column: the smaller radix when it divides the larger (every thread
+// then has the same work in both passes; with 16 threads for 16 x 8 half of them
+// waited at the barrier through pass 1), else the larger.
+__host__ __device__ constexpr int line_slots(int Q1, int Q2) {
+  return imax(Q1, Q2) % (Q1 + Q2 - imax(Q1, Q2)) == 0 ? Q1 + Q2 - imax(Q1, Q2) : imax(Q1, Q2);
+}
 // columns per CTA: 128 bytes of a row, fewer when a line needs more than 16 threads
 template <typename T> __host__ __device__ constexpr int line_cols(int S) {
   return sizeof(T) == 4 ? (S <= 16 ? 16 : 8) : (S <= 16 ? 8 : 4);
 }
 // registers a thread may use: the larger radix's values, its DFT's temporaries
-// and the addresses
-template <typename T> __host__ __device__ constexpr int line_regs(int R) {
-  const int r = sizeof(T) == 4 ? (R <= 8 ? 40 : R <= 10 ? 48 : R <= 16 ? 72 : R <= 21 ? 96 : 128)
-                               : (R <= 8 ? 80 : R <= 10 ? 96 : R <= 16 ? 128 : 168);
-  return r;
+// and the addresses.  Radices 12 to 16 with 12 to 16 threads per line run at 64
+// (four CTAs of 256 threads; 192 x 96 x 96 lines, 16 right-hand sides: 395 us at
+// 80 registers, 373 us at 64); with 8 threads doing two butterflies they spill there.
+template <typename T> __host__ __device__ constexpr int line_regs(int R, int S) {
+  return sizeof(T) == 4 ? (R <= 8 ? 48 : R <= 10 ? 56 : R <= 16 ? (S >= 12 ? 64 : 80) : R <= 21 ? 96 : 128)
+                        : (R <= 8 ? 80 : R <= 10 ? 96 : R <= 16 ? 128 : 168);
 }
 template <typename T> __host__ __device__ constexpr int line_blocks(int Q1, int Q2) {
-  const int S = imax(Q1, Q2), th = line_cols<T>(S) * S;
-  const int b = 65536 / (line_regs<T>(S) * ((th + 31) / 32 * 32));
+  const int S = line_slots(Q1, Q2), th = line_cols<T>(S) * S;
+  const int b = 65536 / (line_regs<T>(imax(Q1, Q2), S) * ((th + 31) / 32 * 32));
   return b < 1 ? 1 : (b > 24 ? 24 : b);
 }
 
 template <typename T, int Q1, int Q2, bool INV>
-__global__ void __launch_bounds__(line_cols<T>(imax(Q1, Q2)) * imax(Q1, Q2), line_blocks<T>(Q1, Q2))
+__global__ void __launch_bounds__(line_cols<T>(line_slots(Q1, Q2)) * line_slots(Q1, Q2), line_blocks<T>(Q1, Q2))
     plan_line_kernel(const LineArgs<T> a) {
   using C = cx<T>;
+  constexpr int S = line_slots(Q1, Q2);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* X = reinterpret_cast<C*>(smem_raw);               // [Q1][Q2][CW]
-  const int CW = blockDim.x, col = threadIdx.x, t = threadIdx.y;
+  const int CW = blockDim.x, col = threadIdx.x, t0 = threadIdx.y;
   const int c0 = blockIdx.x * CW + col, o = blockIdx.y, bb = blockIdx.z;
   pdl_trigger();
   pdl_wait();
   if (a.active != nullptr && a.active[bb / a.batch_per_rhs] == 0) return;   // block-uniform
-  if (a.prof != nullptr && blockIdx.x == 0 && o == 0 && col == 0 && t == 0)
+  if (a.prof != nullptr && blockIdx.x == 0 && o == 0 && col == 0 && t0 == 0)
     atomicAdd(a.prof, a.prof_batch_bytes);
   const bool col_ok = c0 < a.ncol;
   const T rs = (a.flags & (PRO_RSCALE | EPI_RSCALE))
                    ? (T)a.rscale[(long long)(bb / a.batch_per_rhs) * a.rscale_stride]
                    : (T)1;
-  if (t < Q2) {
-    const C* in = a.in + bb * a.in_bs + o * a.in_os + c0 + (long long)t * a.in_ls;
-    const long long step = (long long)Q2 * a.in_ls;
-    C v[Q1];
-    if constexpr (!INV) {
-      C x[Q1 / 2];
+  // offsets inside one batch entry fit 32 bits (checked at launch)
+  const unsigned ils = (unsigned)a.in_ls, ols = (unsigned)a.out_ls, hls = (unsigned)a.chi_ls;
+  const unsigned hoff = (unsigned)(o * a.chi_os) + (unsigned)c0;
+  {
+    const C* in = a.in + bb * a.in_bs;
+    const unsigned ioff = (unsigned)(o * a.in_os) + (unsigned)c0;
 #pragma unroll
-      for (int m = 0; m < Q1 / 2; ++m) x[m] = col_ok ? in[m * step] : czero<C>();
-      if (a.flags & (PRO_RSCALE | PRO_CONJ | PRO_CHI)) {
-        const C* chi = a.chi + o * a.chi_os + c0 + (long long)t * a.chi_ls;
+    for (int i = 0; i < (Q2 + S - 1) / S; ++i) {
+      const int t = t0 + i * S;
+      if (Q2 % S != 0 && t >= Q2) break;
+      C v[Q1];
+      if constexpr (!INV) {
+        C x[Q1 / 2];
 #pragma unroll
-        for (int m = 0; m < Q1 / 2; ++m) {
-          if (a.flags & PRO_RSCALE) x[m] = rs * x[m];
-          if (a.flags & PRO_CONJ) x[m] = conjg(x[m]);
-          if ((a.flags & PRO_CHI) && col_ok) x[m] = chi[(long long)m * Q2 * a.chi_ls] * x[m];
+        for (int m = 0; m < Q1 / 2; ++m) x[m] = col_ok ? in[ioff + (t + Q2 * m) * ils] : czero<C>();
+        if (a.flags & (PRO_RSCALE | PRO_CONJ | PRO_CHI)) {
+#pragma unroll
+          for (int m = 0; m < Q1 / 2; ++m) {
+            if (a.flags & PRO_RSCALE) x[m] = rs * x[m];
+            if (a.flags & PRO_CONJ) x[m] = conjg(x[m]);
+            if ((a.flags & PRO_CHI) && col_ok) x[m] = a.chi[hoff + (t + Q2 * m) * hls] * x[m];
+          }
         }
+        dft_half_in<Q1, false>(x, v);
+      } else {
+#pragma unroll
+        for (int m = 0; m < Q1; ++m) v[m] = col_ok ? in[ioff + (t + Q2 * m) * ils] : czero<C>();
+        dft_reg<Q1, true>(v);
       }
-      dft_half_in<Q1, false>(x, v);
-    } else {
 #pragma unroll
-      for (int m = 0; m < Q1; ++m) v[m] = col_ok ? in[m * step] : czero<C>();
-      dft_reg<Q1, true>(v);
+      for (int c = 1; c < Q1; ++c) {
+        const C w = __ldg(a.roots + t * c);
+        v[c] = v[c] * (INV ? conjg(w) : w);
+      }
+#pragma unroll
+      for (int c = 0; c < Q1; ++c) X[(c * Q2 + t) * CW + col] = v[c];
     }
-#pragma unroll
-    for (int c = 1; c < Q1; ++c) {
-      const C w = __ldg(a.roots + t * c);
-      v[c] = v[c] * (INV ? conjg(w) : w);
-    }
-#pragma unroll
-    for (int c = 0; c < Q1; ++c) X[(c * Q2 + t) * CW + col] = v[c];
   }
   __syncthreads();
-  if (t >= Q1 || !col_ok) return;
-  C u[Q2];
+  if (!col_ok) return;
+  C* out = a.out + bb * a.out_bs;
+  const unsigned ooff = (unsigned)(o * a.out_os) + (unsigned)c0;
 #pragma unroll
-  for (int f = 0; f < Q2; ++f) u[f] = X[(t * Q2 + f) * CW + col];
-  const long long obase = bb * a.out_bs + o * a.out_os + c0 + (long long)t * a.out_ls;
-  const long long ostep = (long long)Q1 * a.out_ls;
-  C* out = a.out + obase;
-  if constexpr (!INV) {
-    dft_reg<Q2, false>(u);
+  for (int i = 0; i < (Q1 + S - 1) / S; ++i) {
+    const int t = t0 + i * S;
+    if (Q1 % S != 0 && t >= Q1) break;
+    C u[Q2];
 #pragma unroll
-    for (int h = 0; h < Q2; ++h) out[h * ostep] = u[h];
-  } else {
-    C y[Q2 / 2];
-    dft_half_out<Q2, true>(u, y);
+    for (int f = 0; f < Q2; ++f) u[f] = X[(t * Q2 + f) * CW + col];
+    if constexpr (!INV) {
+      dft_reg<Q2, false>(u);
 #pragma unroll
-    for (int h = 0; h < Q2 / 2; ++h) y[h] = a.scale * y[h];
-    if (a.flags & (EPI_CONJ | EPI_SUB | EPI_ADD)) {
-      const C* chi = a.chi + o * a.chi_os + c0 + (long long)t * a.chi_ls;
-      const C* add = a.addend + obase;
+      for (int h = 0; h < Q2; ++h) out[ooff + (t + Q1 * h) * ols] = u[h];
+    } else {
+      C y[Q2 / 2];
+      dft_half_out<Q2, true>(u, y);
 #pragma unroll
-      for (int h = 0; h < Q2 / 2; ++h) {
-        C x = y[h];
-        if (a.flags & EPI_CONJ) x = conjg(x);
-        if (a.flags & (EPI_SUB | EPI_ADD)) {
-          if (a.flags & EPI_CHI) x = chi[(long long)h * Q1 * a.chi_ls] * x;
-          C w = add[h * ostep];
-          if (a.flags & EPI_RSCALE) w = rs * w;
-          x = (a.flags & EPI_SUB) ? (w - x) : (w + x);
+      for (int h = 0; h < Q2 / 2; ++h) y[h] = a.scale * y[h];
+      if (a.flags & (EPI_CONJ | EPI_SUB | EPI_ADD)) {
+        const C* add = a.addend + bb * a.out_bs;
+#pragma unroll
+        for (int h = 0; h < Q2 / 2; ++h) {
+          C x = y[h];
+          if (a.flags & EPI_CONJ) x = conjg(x);
+          if (a.flags & (EPI_SUB | EPI_ADD)) {
+            if (a.flags & EPI_CHI) x = a.chi[hoff + (t + Q1 * h) * hls] * x;
+            C w = add[ooff + (t + Q1 * h) * ols];
+            if (a.flags & EPI_RSCALE) w = rs * w;
+            x = (a.flags & EPI_SUB) ? (w - x) : (w + x);
+          }
+          y[h] = x;
         }
-        y[h] = x;
       }
-    }
 #pragma unroll
-    for (int h = 0; h < Q2 / 2; ++h) out[h * ostep] = y[h];
+      for (int h = 0; h < Q2 / 2; ++h) out[ooff + (t + Q1 * h) * ols] = y[h];
+    }
   }
 }
 
 // Q1 is even: forward Q1 x Q2, inverse Q2 x Q1 (the even radix where the half is)
 template <typename T, int Q1, int Q2> void launch_plan_line(LineArgs<T> a, cudaStream_t s) {
   static_assert(Q1 % 2 == 0, "the pruned radix is even");
-  constexpr int S = imax(Q1, Q2), CMAX = line_cols<T>(S);
+  constexpr int S = line_slots(Q1, Q2), CMAX = line_cols<T>(S);
   // lines whose columns are adjacent across `o` too (the x stages) form one run
   if (a.in_os == a.ncol && a.out_os == a.ncol && (a.chi == nullptr || a.chi_os == a.ncol) &&
       (long long)a.ncol * a.nother < (1LL << 30)) {
@@ -168,7 +191,7 @@ template <typename T, int Q1, int Q2> void launch_plan_line(LineArgs<T> a, cudaS
 }
 
 template <typename T, int Q1, int Q2> cudaError_t prepare_plan_line() {
-  constexpr size_t smem = (size_t)Q1 * Q2 * line_cols<T>(imax(Q1, Q2)) * sizeof(cx<T>);
+  constexpr size_t smem = (size_t)Q1 * Q2 * line_cols<T>(line_slots(Q1, Q2)) * sizeof(cx<T>);
   if constexpr (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(plan_line_kernel<T, Q1, Q2, false>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -183,19 +206,39 @@ template <typename T, int Q1, int Q2> cudaError_t prepare_plan_line() {
 // ---------------------------------------------------------------------------
 // fused z stage
 // ---------------------------------------------------------------------------
+// Threads per line: one per slot of the widest pass, or, where that makes a group
+// one warp (8 lines' butterflies: barriers become warp barriers) or the first
+// radix is so large that registers limit the threads anyway, only the M1
+// butterflies of the first pass, later passes looping over their slots (N = 128
+// with 8 right-hand sides: 16 threads 171 us, 8 threads 165 us; N = 112: 37 and
+// 30 us; N = 216: 357 and 295 us; but N = 160: 97 and 122 us, N = 40: 9.7 and
+// 13.2 us).
+__host__ __device__ constexpr int fused_slots(int R1, int R2, int R3) {
+  const int M1 = R2 * R3, wide = imax(imax(M1, R1 * R3), R3 > 1 ? R1 * R2 : R1);
+  return R3 == 1 && (M1 == 8 || R1 >= 18) ? M1 : wide;
+}
+
 template <int R1, int R2, int R3> struct FusedPlan {
   static constexpr int N = R1 * R2 * R3, M1 = R2 * R3, H3 = N / 2 + 1;
-  static constexpr int HL = R3 > 1 ? R3 : R2;               // frequencies per thread
-  static constexpr int TL = R3 > 1 ? R1 * R2 : R1;          // threads that hold them
-  static constexpr int S = imax(imax(M1, R1 * R3), TL);     // threads per line
+  static constexpr int HL = R3 > 1 ? R3 : R2;               // frequencies per slot of the last pass
+  static constexpr int TL = R3 > 1 ? R1 * R2 : R1;          // slots of the last pass
+  static constexpr int S = fused_slots(R1, R2, R3);         // threads per line
   static constexpr int PR = R3 > 1 ? (R3 | 1) : 1;          // padded run of e
   static constexpr int LD = (R3 > 1 ? R2 * PR : R2) | 1;    // row c of a line's buffer (odd)
   static constexpr int LS = R1 * LD;                        // one line of one component
+  // lines S (mod 16) entries apart: consecutive threads of neighbouring lines
+  // fall in different 8-byte banks, in the rows of pass 1 and (LD odd) the
+  // columns of pass 2
+  static constexpr int LSTR = 3 * LS + ((S - 3 * LS) % 16 + 16) % 16;
   static constexpr int NL = (R1 + 1) / 2;                   // inputs that can be nonzero
-  // small groups share a CTA
+  // small groups share a CTA (and its twiddle tables)
   static constexpr int GP = 4 * S >= 64 ? 1 : (64 + 4 * S - 1) / (4 * S);
   static constexpr int threads = 4 * S * GP;
+  static constexpr bool kWarp = 4 * S == 32;                // a group is one warp
   static constexpr int GH = 6 * H3 + (6 * H3 & 1);          // half fibres, 16-byte multiple
+  static constexpr int T1 = R1 * M1, T2 = R3 > 1 ? R2 * R3 : 0;   // twiddles [c][a], [g][e]
+  static constexpr int XS = 4 * LSTR;
+  static constexpr int fixed = GP * (GH + XS) + T1 + T2;    // shared entries
   static __host__ __device__ constexpr int inner(int a) {   // X1 column of a = e + R3 f
     return R3 > 1 ? (a / R3) * PR + a % R3 : a;
   }
@@ -208,7 +251,9 @@ template <typename T, int R1, int R2, int R3> __host__ __device__ constexpr int 
   const int regs = sizeof(T) == 4 ? (live < 64 ? 64 : live > 168 ? 168 : live)
                                   : (live * 2 > 255 ? 255 : live * 2);
   const int wt = (P::threads + 31) / 32 * 32;
-  const int b = 65536 / (((regs + 7) / 8 * 8) * wt);
+  const int by_regs = 65536 / (((regs + 7) / 8 * 8) * wt);
+  const int by_smem = (int)((size_t)227 * 1024 / (P::fixed * sizeof(cx<T>) + 1024));
+  const int b = by_regs < by_smem ? by_regs : by_smem;
   return b < 1 ? 1 : (b > 16 ? 16 : b);
 }
 
@@ -220,10 +265,13 @@ __global__ void __launch_bounds__(FusedPlan<R1, R2, R3>::threads, fused_blocks<T
   constexpr int N = P::N, S = P::S, H3 = P::H3, HL = P::HL, LD = P::LD, NL = P::NL, M1 = P::M1;
   constexpr bool kEven = R1 % 2 == 0;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  C* sm = reinterpret_cast<C*>(smem_raw);
   const int gp = threadIdx.x / (4 * S), lt = threadIdx.x % (4 * S);
   const int l = lt / S, t = lt % S;
-  C* G = reinterpret_cast<C*>(smem_raw) + gp * P::GH;                      // [6][H3]
-  C* X = reinterpret_cast<C*>(smem_raw) + P::GP * P::GH + (gp * 12 + l * 3) * P::LS;   // [3][R1][LD]
+  C* G = sm + gp * P::GH;                                          // [6][H3]
+  C* X = sm + P::GP * P::GH + gp * P::XS + l * P::LSTR;            // [3][R1][LD]
+  C* tw1 = sm + P::GP * (P::GH + P::XS);                           // w_N^{a c} at [c][a]
+  C* tw2 = tw1 + P::T1;                                            // w_{R2 R3}^{e g} at [g][e]
   const int k1 = k10 + blockIdx.y, k2 = blockIdx.x * P::GP + gp;
   const bool group = k2 < a.H2;
   const int nx = (k1 == 0 || 2 * k1 == a.P1) ? 1 : 2;
@@ -232,28 +280,29 @@ __global__ void __launch_bounds__(FusedPlan<R1, R2, R3>::threads, fused_blocks<T
   const int ix = valid ? l / ny : 0, iy = valid ? l % ny : 0;
   const int kx = ix ? a.P1 - k1 : k1, ky = iy ? a.P2 - k2 : k2;
   C* line0 = a.data + ((long long)kx * a.P2 + ky) * (N / 2) + t;
+  auto sync = [&]() {
+    if constexpr (P::kWarp) __syncwarp(); else __syncthreads();
+  };
   // no rebuilt half fibres to copy (FP64; FP32 beyond the rebuild kernels' ranks):
-  // eq. (13) for this group here
+  // eq. (13) for this group here, W_c = U2_c[k2, :] S_c[k1], G_c[k3] = W_c . U3_c[k3, :]
   const bool here = a.spec == nullptr && a.octant == nullptr;
-  if (here && group) {
-    // W_c = U2_c[k2, :] S_c[k1], G_c[k3] = W_c . U3_c[k3, :]
-    C* W = reinterpret_cast<C*>(smem_raw) + P::GP * (P::GH + 12 * P::LS) + gp * 6 * a.r3max;
-    for (int it = lt; it < 6 * a.r3max; it += 4 * S) {
-      const int c = it / a.r3max, q = it - c * a.r3max;
-      const CompMeta<T>& m = a.meta[c];
-      C acc = czero<C>();
-      if (q < m.r3) {
-        const C* sl = m.slab + (long long)k1 * a.r2max * a.r3max + q;
-        const C* u2 = m.U2 + (long long)k2 * m.r2;
-        for (int b = 0; b < m.r2; ++b) acc = cmadd(u2[b], sl[b * a.r3max], acc);
-      }
-      W[it] = acc;
-    }
-  }
   if (here) {
+    C* W = sm + P::fixed + gp * 6 * a.r3max;
+    if (group) {
+      for (int it = lt; it < 6 * a.r3max; it += 4 * S) {
+        const int c = it / a.r3max, q = it - c * a.r3max;
+        const CompMeta<T>& m = a.meta[c];
+        C acc = czero<C>();
+        if (q < m.r3) {
+          const C* sl = m.slab + (long long)k1 * a.r2max * a.r3max + q;
+          const C* u2 = m.U2 + (long long)k2 * m.r2;
+          for (int b = 0; b < m.r2; ++b) acc = cmadd(u2[b], sl[b * a.r3max], acc);
+        }
+        W[it] = acc;
+      }
+    }
     __syncthreads();
     if (group) {
-      const C* W = reinterpret_cast<C*>(smem_raw) + P::GP * (P::GH + 12 * P::LS) + gp * 6 * a.r3max;
       for (int it = lt; it < 6 * H3; it += 4 * S) {
         const int c = it / H3, kk = it - c * H3;
         const int r3 = a.meta[c].r3;
@@ -284,11 +333,15 @@ __global__ void __launch_bounds__(FusedPlan<R1, R2, R3>::threads, fused_blocks<T
       const C* src = line0 + (long long)(b * 3 + q) * a.comp_stride;
 #pragma unroll
       for (int m = 0; m < NL; ++m)
-        x[q][m] = (valid && t < M1 && (kEven || t + M1 * m < N / 2)) ? src[M1 * m] : czero<C>();
+        x[q][m] = (valid && (S == M1 || t < M1) && (kEven || t + M1 * m < N / 2)) ? src[M1 * m] : czero<C>();
     }
   };
   int b = next_active(0);
   if (b < a.B) load(b);
+  // tables and half fibres while those are under way
+  for (int i = threadIdx.x; i < P::T1; i += P::threads) tw1[i] = a.roots[(i / M1) * (i % M1)];
+  if constexpr (R3 > 1)
+    for (int i = threadIdx.x; i < P::T2; i += P::threads) tw2[i] = a.roots[R1 * (i / R3) * (i % R3)];
   if (group) {
     if (a.spec != nullptr) {
       const C* src = a.spec + ((long long)k1 * a.P2 + k2) * N;
@@ -304,10 +357,10 @@ __global__ void __launch_bounds__(FusedPlan<R1, R2, R3>::threads, fused_blocks<T
     }
   }
   const T sx = ix ? (T)-1 : (T)1, sy = iy ? (T)-1 : (T)1;
-  const int c2 = t % R1, e2 = t / R1;                  // slots (c, e) and (c, g)
+  __syncthreads();                                     // tables and half fibres
   for (bool first = true; b < a.B; b = next_active(b + 1), first = false) {   // block-uniform
     if (!first) load(b);
-    if (t < M1) {
+    if (S == M1 || t < M1) {
 #pragma unroll
       for (int q = 0; q < 3; ++q) {
         C v[R1];
@@ -321,44 +374,46 @@ __global__ void __launch_bounds__(FusedPlan<R1, R2, R3>::threads, fused_blocks<T
         C* row = X + q * P::LS + P::inner(t);
         row[0] = v[0];
 #pragma unroll
-        for (int c = 1; c < R1; ++c) row[c * LD] = v[c] * __ldg(a.roots + t * c);
+        for (int c = 1; c < R1; ++c) row[c * LD] = v[c] * tw1[c * M1 + t];
       }
     }
-    __syncthreads();
+    sync();
     if constexpr (R3 > 1) {
-      if (t < R1 * R3) {
+#pragma unroll 1
+      for (int sl = t; sl < R1 * R3; sl += S) {          // slot (c, e)
+        C* p = X + (sl % R1) * LD + sl / R1;
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
           C u[R2];
-          C* p = X + q * P::LS + c2 * LD + e2;
 #pragma unroll
-          for (int f = 0; f < R2; ++f) u[f] = p[f * P::PR];
+          for (int f = 0; f < R2; ++f) u[f] = p[q * P::LS + f * P::PR];
           dft_reg<R2, false>(u);
-          p[0] = u[0];
+          p[q * P::LS] = u[0];
 #pragma unroll
-          for (int g = 1; g < R2; ++g) p[g * P::PR] = u[g] * __ldg(a.roots + R1 * e2 * g);
+          for (int g = 1; g < R2; ++g) p[q * P::LS + g * P::PR] = u[g] * tw2[g * R3 + sl / R1];
         }
       }
-      __syncthreads();
+      sync();
     }
-    if (t < P::TL) {
+#pragma unroll 1
+    for (int sl = t; sl < P::TL; sl += S) {              // slot (c, g)
       C s[3][HL];
-      C* own = X + c2 * LD + (R3 > 1 ? e2 * P::PR : 0);     // this thread's points of a component
+      C* own = X + (sl % R1) * LD + (R3 > 1 ? (sl / R1) * P::PR : 0);
 #pragma unroll
       for (int q = 0; q < 3; ++q) {
 #pragma unroll
         for (int e = 0; e < HL; ++e) s[q][e] = own[q * P::LS + e];
         dft_reg<HL, false>(s[q]);
       }
-      // Y = D G D J at f = t + TL h
+      // Y = D G D J at f = sl + TL h
 #pragma unroll
       for (int h = 0; h < HL; ++h) {
-        const int f = t + P::TL * h;
+        const int f = sl + P::TL * h;
         const bool zm = 2 * f > N;
-        const C* gp_ = G + (zm ? N - f : f);
+        const C* gf = G + (zm ? N - f : f);
         const T sz = zm ? (T)-1 : (T)1;
-        const C gxx = gp_[0], gyy = gp_[3 * H3], gzz = gp_[5 * H3];
-        const C gxy = (sx * sy) * gp_[H3], gxz = (sx * sz) * gp_[2 * H3], gyz = (sy * sz) * gp_[4 * H3];
+        const C gxx = gf[0], gyy = gf[3 * H3], gzz = gf[5 * H3];
+        const C gxy = (sx * sy) * gf[H3], gxz = (sx * sz) * gf[2 * H3], gyz = (sy * sz) * gf[4 * H3];
         const C jx = s[0][h], jy = s[1][h], jz = s[2][h];
         s[0][h] = cmadd(gxx, jx, cmadd(gxy, jy, gxz * jz));
         s[1][h] = cmadd(gxy, jx, cmadd(gyy, jy, gyz * jz));
@@ -367,40 +422,36 @@ __global__ void __launch_bounds__(FusedPlan<R1, R2, R3>::threads, fused_blocks<T
 #pragma unroll
       for (int q = 0; q < 3; ++q) {
         dft_reg<HL, true>(s[q]);
-        own[q * P::LS] = s[q][0];                      // e = 0, or a = 0
-        if constexpr (R3 > 1) {
 #pragma unroll
-          for (int e = 1; e < HL; ++e)
-            own[q * P::LS + e] = s[q][e] * conjg(__ldg(a.roots + R1 * e * e2));
-        } else {
-#pragma unroll
-          for (int e = 1; e < HL; ++e) own[q * P::LS + e] = s[q][e] * conjg(__ldg(a.roots + e * c2));
-        }
+        for (int e = 0; e < HL; ++e) own[q * P::LS + e] = s[q][e];
       }
     }
-    __syncthreads();
+    sync();
     if constexpr (R3 > 1) {
-      if (t < R1 * R3) {
+#pragma unroll 1
+      for (int sl = t; sl < R1 * R3; sl += S) {
+        C* p = X + (sl % R1) * LD + sl / R1;
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
           C u[R2];
-          C* p = X + q * P::LS + c2 * LD + e2;
+          u[0] = p[q * P::LS];
 #pragma unroll
-          for (int g = 0; g < R2; ++g) u[g] = p[g * P::PR];
+          for (int g = 1; g < R2; ++g) u[g] = p[q * P::LS + g * P::PR] * conjg(tw2[g * R3 + sl / R1]);
           dft_reg<R2, true>(u);
 #pragma unroll
-          for (int f = 0; f < R2; ++f) p[f * P::PR] = u[f] * conjg(__ldg(a.roots + (e2 + R3 * f) * c2));
+          for (int f = 0; f < R2; ++f) p[q * P::LS + f * P::PR] = u[f];
         }
       }
-      __syncthreads();
+      sync();
     }
-    if (t < M1) {
+    if (S == M1 || t < M1) {
 #pragma unroll
       for (int q = 0; q < 3; ++q) {
         C v[R1];
         const C* row = X + q * P::LS + P::inner(t);
+        v[0] = row[0];
 #pragma unroll
-        for (int c = 0; c < R1; ++c) v[c] = row[c * LD];
+        for (int c = 1; c < R1; ++c) v[c] = row[c * LD] * conjg(tw1[c * M1 + t]);
         C* dst = line0 + (long long)(b * 3 + q) * a.comp_stride;
         if constexpr (kEven) {
           C y[R1 / 2];
@@ -424,8 +475,7 @@ __global__ void __launch_bounds__(FusedPlan<R1, R2, R3>::threads, fused_blocks<T
 
 template <typename T, int R1, int R2, int R3>
 constexpr size_t fused_smem_fixed() {
-  using P = FusedPlan<R1, R2, R3>;
-  return (size_t)P::GP * (P::GH + 12 * P::LS) * sizeof(cx<T>);
+  return (size_t)FusedPlan<R1, R2, R3>::fixed * sizeof(cx<T>);
 }
 
 // groups k1 in [k10, k10 + nk1), every k2

@@ -729,7 +729,7 @@ bool fused_tp_supported(const FusedArgs<float>& a);
 void launch_fused_tp(const FusedArgs<float>& a, int groups, cudaStream_t s);
 // every edge with a factor plan (plan.cu): false when the launch is not one of theirs
 bool plan_exists(int N);
-bool launch_plan_line(const LineArgs<float>& a, cudaStream_t s);
-bool launch_plan_fused(const FusedArgs<float>& a, int k10, int nk1, cudaStream_t s);
+template <typename T> bool launch_plan_line(const LineArgs<T>& a, cudaStream_t s);
+template <typename T> bool launch_plan_fused(const FusedArgs<T>& a, int k10, int nk1, cudaStream_t s);
 
 }  // namespace vie
