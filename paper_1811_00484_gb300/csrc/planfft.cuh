@@ -1,6 +1,6 @@
 // Matvec stages for every padded edge N = 2n with a factor plan: x / y line
 // stages (zero-padded forward, cropped inverse) and the fused z stage (forward
-// transform, voxel-wise product, inverse transform), in FP32 and FP64.  All
+// transform, voxel-wise product, inverse transform), in FP32 (planfft64.cuh: FP64).  All
 // lengths, strides in shared memory and radices are compile-time constants, so
 // the only index arithmetic left is one multiply-add per access.
 //
@@ -28,8 +28,8 @@
 //
 // The half fibre G[6][N/2+1] of the group is copied from the FP32 rebuild
 // scratch, read from the stored spectra (only the octant k <= P/2: the rest is
-// its mirror image, an eighth of the bytes), or rebuilt by the CTA (FP64, and
-// ranks beyond the rebuild kernels').
+// its mirror image, an eighth of the bytes), or rebuilt by the CTA (ranks beyond
+// the rebuild kernels').
 #pragma once
 
 #include "regdft.cuh"
@@ -44,6 +44,7 @@ template <typename T, int K> bool fused_set(const FusedArgs<T>& a, int k10, int 
 template <typename T, int K> cudaError_t prepare_set(int N);
 
 __host__ __device__ constexpr int imax(int a, int b) { return a > b ? a : b; }
+__host__ __device__ constexpr int imin(int a, int b) { return a < b ? a : b; }
 
 // ---------------------------------------------------------------------------
 // line stage
@@ -55,27 +56,24 @@ __host__ __device__ constexpr int line_slots(int Q1, int Q2) {
   return imax(Q1, Q2) % (Q1 + Q2 - imax(Q1, Q2)) == 0 ? Q1 + Q2 - imax(Q1, Q2) : imax(Q1, Q2);
 }
 // columns per CTA: 128 bytes of a row, fewer when a line needs more than 16 threads
-template <typename T> __host__ __device__ constexpr int line_cols(int S) {
-  return sizeof(T) == 4 ? (S <= 16 ? 16 : 8) : (S <= 16 ? 8 : 4);
-}
+__host__ __device__ constexpr int line_cols(int S) { return S <= 16 ? 16 : 8; }
 // registers a thread may use: the larger radix's values, its DFT's temporaries
 // and the addresses.  Radices 12 to 16 with 12 to 16 threads per line run at 64
 // (four CTAs of 256 threads; 192 x 96 x 96 lines, 16 right-hand sides: 395 us at
 // 80 registers, 373 us at 64); with 8 threads doing two butterflies they spill there.
-template <typename T> __host__ __device__ constexpr int line_regs(int R, int S) {
-  return sizeof(T) == 4 ? (R <= 8 ? 48 : R <= 10 ? 56 : R <= 16 ? (S >= 12 ? 64 : 80) : R <= 21 ? 96 : 128)
-                        : (R <= 8 ? 80 : R <= 10 ? 96 : R <= 16 ? 128 : 168);
+__host__ __device__ constexpr int line_regs(int R, int S) {
+  return R <= 8 ? 48 : R <= 10 ? 56 : R <= 16 ? (S >= 12 ? 64 : 80) : R <= 21 ? 96 : 128;
 }
-template <typename T> __host__ __device__ constexpr int line_blocks(int Q1, int Q2) {
-  const int S = line_slots(Q1, Q2), th = line_cols<T>(S) * S;
-  const int b = 65536 / (line_regs<T>(imax(Q1, Q2), S) * ((th + 31) / 32 * 32));
+__host__ __device__ constexpr int line_blocks(int Q1, int Q2) {
+  const int S = line_slots(Q1, Q2), th = line_cols(S) * S;
+  const int b = 65536 / (line_regs(imax(Q1, Q2), S) * ((th + 31) / 32 * 32));
   return b < 1 ? 1 : (b > 24 ? 24 : b);
 }
 
-template <typename T, int Q1, int Q2, bool INV>
-__global__ void __launch_bounds__(line_cols<T>(line_slots(Q1, Q2)) * line_slots(Q1, Q2), line_blocks<T>(Q1, Q2))
-    plan_line_kernel(const LineArgs<T> a) {
-  using C = cx<T>;
+template <int Q1, int Q2, bool INV>
+__global__ void __launch_bounds__(line_cols(line_slots(Q1, Q2)) * line_slots(Q1, Q2), line_blocks(Q1, Q2))
+    plan_line_kernel(const LineArgs<float> a) {
+  using C = float2;
   constexpr int S = line_slots(Q1, Q2);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* X = reinterpret_cast<C*>(smem_raw);               // [Q1][Q2][CW]
@@ -87,9 +85,9 @@ __global__ void __launch_bounds__(line_cols<T>(line_slots(Q1, Q2)) * line_slots(
   if (a.prof != nullptr && blockIdx.x == 0 && o == 0 && col == 0 && t0 == 0)
     atomicAdd(a.prof, a.prof_batch_bytes);
   const bool col_ok = c0 < a.ncol;
-  const T rs = (a.flags & (PRO_RSCALE | EPI_RSCALE))
-                   ? (T)a.rscale[(long long)(bb / a.batch_per_rhs) * a.rscale_stride]
-                   : (T)1;
+  const float rs = (a.flags & (PRO_RSCALE | EPI_RSCALE))
+                   ? (float)a.rscale[(long long)(bb / a.batch_per_rhs) * a.rscale_stride]
+                   : 1.f;
   // offsets inside one batch entry fit 32 bits (checked at launch)
   const unsigned ils = (unsigned)a.in_ls, ols = (unsigned)a.out_ls, hls = (unsigned)a.chi_ls;
   const unsigned hoff = (unsigned)(o * a.chi_os) + (unsigned)c0;
@@ -170,9 +168,9 @@ __global__ void __launch_bounds__(line_cols<T>(line_slots(Q1, Q2)) * line_slots(
 }
 
 // Q1 is even: forward Q1 x Q2, inverse Q2 x Q1 (the even radix where the half is)
-template <typename T, int Q1, int Q2> void launch_plan_line(LineArgs<T> a, cudaStream_t s) {
+template <int Q1, int Q2> void launch_plan_line(LineArgs<float> a, cudaStream_t s) {
   static_assert(Q1 % 2 == 0, "the pruned radix is even");
-  constexpr int S = line_slots(Q1, Q2), CMAX = line_cols<T>(S);
+  constexpr int S = line_slots(Q1, Q2), CMAX = line_cols(S);
   // lines whose columns are adjacent across `o` too (the x stages) form one run
   if (a.in_os == a.ncol && a.out_os == a.ncol && (a.chi == nullptr || a.chi_os == a.ncol) &&
       (long long)a.ncol * a.nother < (1LL << 30)) {
@@ -182,21 +180,21 @@ template <typename T, int Q1, int Q2> void launch_plan_line(LineArgs<T> a, cudaS
   // equal column groups: 50 columns are 4 groups of 13, not 3 of 16 and one of 2
   const int tiles = (a.ncol + CMAX - 1) / CMAX;
   const int cw = (a.ncol + tiles - 1) / tiles;
-  a.prof = sizeof(T) == 4 ? prof_bytes(a.prof_family) : nullptr;
+  a.prof = prof_bytes(a.prof_family);
   ProfScope ps(a.prof_family, s);
   const dim3 grid((unsigned)tiles, (unsigned)a.nother, (unsigned)a.nbatch), block((unsigned)cw, S);
-  const size_t smem = (size_t)Q1 * Q2 * cw * sizeof(cx<T>);
-  if (a.inverse) launch_pdl(plan_line_kernel<T, Q2, Q1, true>, grid, block, smem, s, a);
-  else launch_pdl(plan_line_kernel<T, Q1, Q2, false>, grid, block, smem, s, a);
+  const size_t smem = (size_t)Q1 * Q2 * cw * sizeof(float2);
+  if (a.inverse) launch_pdl(plan_line_kernel<Q2, Q1, true>, grid, block, smem, s, a);
+  else launch_pdl(plan_line_kernel<Q1, Q2, false>, grid, block, smem, s, a);
 }
 
-template <typename T, int Q1, int Q2> cudaError_t prepare_plan_line() {
-  constexpr size_t smem = (size_t)Q1 * Q2 * line_cols<T>(line_slots(Q1, Q2)) * sizeof(cx<T>);
+template <int Q1, int Q2> cudaError_t prepare_plan_line(float) {
+  constexpr size_t smem = (size_t)Q1 * Q2 * line_cols(line_slots(Q1, Q2)) * sizeof(float2);
   if constexpr (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(plan_line_kernel<T, Q1, Q2, false>,
+    cudaError_t e = cudaFuncSetAttribute(plan_line_kernel<Q1, Q2, false>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(plan_line_kernel<T, Q2, Q1, true>,
+      e = cudaFuncSetAttribute(plan_line_kernel<Q2, Q1, true>,
                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     return e;
   }
@@ -207,7 +205,7 @@ template <typename T, int Q1, int Q2> cudaError_t prepare_plan_line() {
 // fused z stage
 // ---------------------------------------------------------------------------
 // Threads per line: one per slot of the widest pass, or, where that makes a group
-// one warp (8 lines' butterflies: barriers become warp barriers) or the first
+// one warp (eight butterflies a line) or the first
 // radix is so large that registers limit the threads anyway, only the M1
 // butterflies of the first pass, later passes looping over their slots (N = 128
 // with 8 right-hand sides: 16 threads 171 us, 8 threads 165 us; N = 112: 37 and
@@ -234,7 +232,6 @@ template <int R1, int R2, int R3> struct FusedPlan {
   // small groups share a CTA (and its twiddle tables)
   static constexpr int GP = 4 * S >= 64 ? 1 : (64 + 4 * S - 1) / (4 * S);
   static constexpr int threads = 4 * S * GP;
-  static constexpr bool kWarp = 4 * S == 32;                // a group is one warp
   static constexpr int GH = 6 * H3 + (6 * H3 & 1);          // half fibres, 16-byte multiple
   static constexpr int T1 = R1 * M1, T2 = R3 > 1 ? R2 * R3 : 0;   // twiddles [c][a], [g][e]
   static constexpr int XS = 4 * LSTR;
@@ -243,24 +240,23 @@ template <int R1, int R2, int R3> struct FusedPlan {
     return R3 > 1 ? (a / R3) * PR + a % R3 : a;
   }
 };
-template <typename T, int R1, int R2, int R3> __host__ __device__ constexpr int fused_blocks() {
+template <int R1, int R2, int R3> __host__ __device__ constexpr int fused_blocks() {
   using P = FusedPlan<R1, R2, R3>;
   // live at the peak: three components of HL frequencies and a half fibre
   // entry, or two components' inputs, one transform and its temporaries
   const int live = imax(6 * P::HL + 60, 4 * P::NL + 3 * R1 + 36);
-  const int regs = sizeof(T) == 4 ? (live < 64 ? 64 : live > 168 ? 168 : live)
-                                  : (live * 2 > 255 ? 255 : live * 2);
+  const int regs = live < 64 ? 64 : live > 168 ? 168 : live;
   const int wt = (P::threads + 31) / 32 * 32;
   const int by_regs = 65536 / (((regs + 7) / 8 * 8) * wt);
-  const int by_smem = (int)((size_t)227 * 1024 / (P::fixed * sizeof(cx<T>) + 1024));
+  const int by_smem = (int)((size_t)227 * 1024 / (P::fixed * sizeof(float2) + 1024));
   const int b = by_regs < by_smem ? by_regs : by_smem;
   return b < 1 ? 1 : (b > 16 ? 16 : b);
 }
 
-template <typename T, int R1, int R2, int R3>
-__global__ void __launch_bounds__(FusedPlan<R1, R2, R3>::threads, fused_blocks<T, R1, R2, R3>())
-    plan_fused_kernel(const FusedArgs<T> a, int k10) {
-  using C = cx<T>;
+template <int R1, int R2, int R3>
+__global__ void __launch_bounds__(FusedPlan<R1, R2, R3>::threads, fused_blocks<R1, R2, R3>())
+    plan_fused_kernel(const FusedArgs<float> a, int k10) {
+  using C = float2;
   using P = FusedPlan<R1, R2, R3>;
   constexpr int N = P::N, S = P::S, H3 = P::H3, HL = P::HL, LD = P::LD, NL = P::NL, M1 = P::M1;
   constexpr bool kEven = R1 % 2 == 0;
@@ -280,10 +276,18 @@ __global__ void __launch_bounds__(FusedPlan<R1, R2, R3>::threads, fused_blocks<T
   const int ix = valid ? l / ny : 0, iy = valid ? l % ny : 0;
   const int kx = ix ? a.P1 - k1 : k1, ky = iy ? a.P2 - k2 : k2;
   C* line0 = a.data + ((long long)kx * a.P2 + ky) * (N / 2) + t;
+  // lines exchange nothing with one another: a line inside one warp, or of whole
+  // warps, needs no barrier of the CTA
   auto sync = [&]() {
-    if constexpr (P::kWarp) __syncwarp(); else __syncthreads();
+    if constexpr (32 % S == 0) {
+      __syncwarp();
+    } else if constexpr (S % 32 == 0) {
+      asm volatile("bar.sync %0, %1;" ::"r"(1 + gp * 4 + l), "n"(S) : "memory");
+    } else {
+      __syncthreads();
+    }
   };
-  // no rebuilt half fibres to copy (FP64; FP32 beyond the rebuild kernels' ranks):
+  // no rebuilt half fibres to copy (ranks beyond the rebuild kernels'):
   // eq. (13) for this group here, W_c = U2_c[k2, :] S_c[k1], G_c[k3] = W_c . U3_c[k3, :]
   const bool here = a.spec == nullptr && a.octant == nullptr;
   if (here) {
@@ -291,7 +295,7 @@ __global__ void __launch_bounds__(FusedPlan<R1, R2, R3>::threads, fused_blocks<T
     if (group) {
       for (int it = lt; it < 6 * a.r3max; it += 4 * S) {
         const int c = it / a.r3max, q = it - c * a.r3max;
-        const CompMeta<T>& m = a.meta[c];
+        const CompMeta<float>& m = a.meta[c];
         C acc = czero<C>();
         if (q < m.r3) {
           const C* sl = m.slab + (long long)k1 * a.r2max * a.r3max + q;
@@ -353,10 +357,10 @@ __global__ void __launch_bounds__(FusedPlan<R1, R2, R3>::threads, fused_blocks<T
       const float4* src = reinterpret_cast<const float4*>(
           a.octant + ((long long)(k1 - a.oct_k1a) * a.H2 + k2) * 6 * H3);
       float4* dst = reinterpret_cast<float4*>(G);
-      for (int it = lt; it < 6 * H3 * (int)sizeof(C) / 16; it += 4 * S) dst[it] = src[it];
+      for (int it = lt; it < 3 * H3; it += 4 * S) dst[it] = src[it];
     }
   }
-  const T sx = ix ? (T)-1 : (T)1, sy = iy ? (T)-1 : (T)1;
+  const float sx = ix ? -1.f : 1.f, sy = iy ? -1.f : 1.f;
   __syncthreads();                                     // tables and half fibres
   for (bool first = true; b < a.B; b = next_active(b + 1), first = false) {   // block-uniform
     if (!first) load(b);
@@ -411,7 +415,7 @@ __global__ void __launch_bounds__(FusedPlan<R1, R2, R3>::threads, fused_blocks<T
         const int f = sl + P::TL * h;
         const bool zm = 2 * f > N;
         const C* gf = G + (zm ? N - f : f);
-        const T sz = zm ? (T)-1 : (T)1;
+        const float sz = zm ? -1.f : 1.f;
         const C gxx = gf[0], gyy = gf[3 * H3], gzz = gf[5 * H3];
         const C gxy = (sx * sy) * gf[H3], gxz = (sx * sz) * gf[2 * H3], gyz = (sy * sz) * gf[4 * H3];
         const C jx = s[0][h], jy = s[1][h], jz = s[2][h];
@@ -473,25 +477,25 @@ __global__ void __launch_bounds__(FusedPlan<R1, R2, R3>::threads, fused_blocks<T
   }
 }
 
-template <typename T, int R1, int R2, int R3>
+template <int R1, int R2, int R3>
 constexpr size_t fused_smem_fixed() {
-  return (size_t)FusedPlan<R1, R2, R3>::fixed * sizeof(cx<T>);
+  return (size_t)FusedPlan<R1, R2, R3>::fixed * sizeof(float2);
 }
 
 // groups k1 in [k10, k10 + nk1), every k2
-template <typename T, int R1, int R2, int R3>
-void launch_plan_fused(const FusedArgs<T>& a, int k10, int nk1, cudaStream_t s) {
+template <int R1, int R2, int R3>
+void launch_plan_fused(const FusedArgs<float>& a, int k10, int nk1, cudaStream_t s) {
   using P = FusedPlan<R1, R2, R3>;
-  size_t smem = fused_smem_fixed<T, R1, R2, R3>();
-  if (a.spec == nullptr && a.octant == nullptr) smem += (size_t)P::GP * 6 * a.r3max * sizeof(cx<T>);
-  launch_pdl(plan_fused_kernel<T, R1, R2, R3>, dim3((unsigned)((a.H2 + P::GP - 1) / P::GP), (unsigned)nk1),
+  size_t smem = fused_smem_fixed<R1, R2, R3>();
+  if (a.spec == nullptr && a.octant == nullptr) smem += (size_t)P::GP * 6 * a.r3max * sizeof(float2);
+  launch_pdl(plan_fused_kernel<R1, R2, R3>, dim3((unsigned)((a.H2 + P::GP - 1) / P::GP), (unsigned)nk1),
              dim3(P::threads), smem, s, a, k10);
 }
 
 constexpr size_t kFusedSmemMax = 200 * 1024;
 
-template <typename T, int R1, int R2, int R3> cudaError_t prepare_plan_fused() {
-  return cudaFuncSetAttribute(plan_fused_kernel<T, R1, R2, R3>,
+template <int R1, int R2, int R3> cudaError_t prepare_plan_fused(float) {
+  return cudaFuncSetAttribute(plan_fused_kernel<R1, R2, R3>,
                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFusedSmemMax);
 }
 
