@@ -141,7 +141,11 @@ typedef struct vie_op_info_t {
                                     scratch, 2 tensor cores through warp-level
                                     mma.sync (3xTF32) into it, 3 tensor cores
                                     through tcgen05.mma with TMEM accumulators
-                                    (3xTF32) into it                          */
+                                    (3xTF32) into it.  Matvecs of small grids
+                                    (y and z edges up to 24) whose planes are
+                                    all resident at once rebuild inside their
+                                    plane kernel instead, unless a rebuild was
+                                    chosen by flag                            */
     int cp_rank;                 /* terms R of the Tucker+CP model (0: none)   */
     double cp_rel_err[6];        /* ||core - CP|| / ||core|| per component;
                                     the factors U^q are orthonormal, so this
@@ -439,7 +443,7 @@ int vie_profile_stop(vie_profile_entry* out, int max_entries, int* count);
 
 /*
  * Self-test of the bounded device waits (no counterpart in the paper).  The
- * TMA-fed kernels wait on shared-memory barriers for their copies with a
+ * tcgen05 rebuild waits on shared-memory barriers for its matrix products with a
  * limit of one second of the device's global timer; a wait that runs out sets
  * a device word that the next vie_solve synchronisation reports as
  * VIE_ERR_TIMEOUT, and the kernel returns.  This call runs that wait alone in

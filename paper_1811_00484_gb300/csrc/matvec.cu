@@ -9,9 +9,11 @@
 //     -- inverse x-FFT, cropped P1 -> n1, scaled
 //        by 1/(P1 P2 P3), optional epilogue -->    Y [B][3][n1][n2][n3]
 //
+// On a small grid the middle three stages are one launch (plane.cu), T1 in place.
+//
 // Lines that are entirely zero padding are never transformed: the x stage
 // runs n2 n3 lines, the y stage P1 n3 lines.
-#include "vie_internal.cuh"
+#include "stages.cuh"
 
 template <typename T>
 int launch_fused(const vie_op* op, cx<T>* data, int B, bool stored, const int* active,
@@ -193,6 +195,15 @@ int matvec_run(const vie_op* op, void* ws, const cx<T>* in, cx<T>* out, int B, i
   const bool cp = (path == VIE_PATH_TUCKER_CP);
   const LineStages<T> st = make_line_stages<T>(op, ws, in, out, B, pro_flags, epi_flags, chi,
                                                addend, active, rscale, rscale_stride);
+  // a small grid: the y and z stages and the rebuild in one launch
+  if (!cp && !(mv_flags & MV_SEPARATE) && vie::plane_eligible<T>(op, B)) {
+    launch_line_fft<T>(st.s[0], s);
+    vie::launch_plane<T>(op, st.s[0].out, B, stored, active, s);
+    launch_line_fft<T>(st.s[3], s);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return cuda_status(e, "matvec launch");
+    return VIE_OK;
+  }
   C* T2 = const_cast<C*>(st.s[1].out);
   // FP32 Tucker path on the register kernels: the first k1 chunk of the rebuild
   // does not read J, so it runs on the operator's side stream beside the x and

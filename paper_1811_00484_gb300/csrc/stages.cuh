@@ -722,14 +722,17 @@ __device__ __forceinline__ void fused_fs_group(const FusedArgs<float>& a, int g,
   }
 }
 
-// Length-512 kernels (tp512.cu): x / y line stages and the fused z stage
-bool launch_line_tp(LineArgs<float> a, cudaStream_t s);
+// Length-512 kernels (tp512.cu): FP64 x / y line stages and the fused z stage
 bool launch_line_tp64(LineArgs<double> a, cudaStream_t s);
 bool fused_tp_supported(const FusedArgs<float>& a);
 void launch_fused_tp(const FusedArgs<float>& a, int groups, cudaStream_t s);
 // every edge with a factor plan (plan.cu): false when the launch is not one of theirs
 bool plan_exists(int N);
 template <typename T> bool launch_plan_line(const LineArgs<T>& a, cudaStream_t s);
+// y and z stages of a small grid's planes in one launch, T1 in place (plane.cu)
+template <typename T> bool plane_eligible(const vie_op* op, int B);
+template <typename T>
+void launch_plane(const vie_op* op, cx<T>* T1, int B, bool stored, const int* active, cudaStream_t s);
 template <typename T> bool launch_plan_fused(const FusedArgs<T>& a, int k10, int nk1, cudaStream_t s);
 
 }  // namespace vie

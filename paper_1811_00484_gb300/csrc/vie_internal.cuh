@@ -285,7 +285,10 @@ double wavenumber(double freq_hz);
 // matvec_impl / matvec_run option: after the fused kernel, start rebuilding the
 // half fibres for the next FP32 Tucker matvec on the operator's side stream (the
 // next matvec joins it); the caller must make another Tucker matvec follow
-enum { MV_PREFETCH_REBUILD = 1 };
+// MV_SEPARATE: no plane kernel (inside a captured graph launches cost the host
+// nothing, and the separate stages run on more SMs: 24^3, 57 us against 48 us per
+// Arnoldi step)
+enum { MV_PREFETCH_REBUILD = 1, MV_SEPARATE = 2 };
 // start that rebuild now (after the work already on s); the next matvec joins it
 int prefetch_rebuild(const vie_op* op, cudaStream_t s, bool cp = false);
 template <typename T>
@@ -353,6 +356,7 @@ int build_operator(const vie_grid* grid, double tol, int rank_rule, int flags, c
 int assemble_spectrum(const vie_op* op, int c, double2* out, cudaStream_t s);
 // padded z edges 32 R that the tcgen05 rebuild and the Tucker+CP model accept
 bool lane_fft_edge(int P3);
+int plane_init_attributes();
 int plan_prepare(int N);     // kernel attributes of padded edge N (plan.cu)
 int op_tables(vie_op* op);   // FFT plans and root tables of op->P
 int line_fft_init_attributes();

@@ -60,3 +60,29 @@ def test_ranks_beyond_the_rebuild_kernels(n):
     J = _field(n, 2, 3, np.complex64)
     assert _rel(op.matvec(J), matvec.matvec_fft(G, J.cpu().numpy().astype(np.complex128))) <= 1e-5
     op.close()
+
+
+@pytest.mark.parametrize("n", [(8, 8, 8), (7, 9, 10), (16, 12, 24), (5, 24, 18), (20, 21, 15), (3, 14, 16), (10, 24, 24)])
+def test_plane_kernel_equals_the_separate_stages(n):
+    """Small grids take the y and z stages in one launch; an operator whose rebuild is
+    chosen by flag takes them one by one.  Same FP32 rebuild, different radix orders."""
+    op, ref = vie.Operator(n, H, F, TOL_SVD, store_uncompressed=True), \
+        vie.Operator(n, H, F, TOL_SVD, store_uncompressed=True, rebuild="simt")
+    rng = np.random.default_rng(1)
+    chi = torch.from_numpy(rng.standard_normal(n) + 1j * rng.standard_normal(n)).cuda()
+    for dtype, tol in ((np.complex64, 2e-6), (np.complex128, 2e-14)):   # rounding of two FFT orders
+        J = _field(n, 3, 5, dtype)
+        c = chi.to(J.dtype)
+        for path in ("tucker", "uncompressed"):
+            pairs = [(o.matvec(J, path=path), o.apply_system(c, J, path=path),
+                      o.apply_system(c, J, adjoint=True, path=path)) for o in (op, ref)]
+            for a, b in zip(*pairs):
+                assert float(torch.linalg.vector_norm(a - b) / torch.linalg.vector_norm(b)) <= tol, (path, dtype)
+    # a batch whose right-hand sides converge at different steps
+    rhs = torch.cat([_field(n, 1, 8, np.complex64), 0 * _field(n, 1, 8, np.complex64)])
+    w, info = op.solve((0.1 * chi).to(torch.complex64), rhs, tol=1e-6)
+    w2, info2 = ref.solve((0.1 * chi).to(torch.complex64), rhs, tol=1e-6)
+    assert info["converged"] and info2["converged"]
+    assert float(torch.linalg.vector_norm(w - w2) / torch.linalg.vector_norm(w2)) <= 1e-4
+    op.close()
+    ref.close()
