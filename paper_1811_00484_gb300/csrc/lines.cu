@@ -90,11 +90,7 @@ static void launch_tw(LineArgs<T> a, size_t smem, cudaStream_t s) {
 // ping-pong buffers and root table fit in 227 KB of shared memory.
 template <typename T>
 void launch_line_fft(const LineArgs<T>& a, cudaStream_t s) {
-  if constexpr (sizeof(T) == 4) {
-    // length 512: the persistent TMA-fed kernel (x + y + their inverses of eight
-    // 256^3 right-hand sides 12.4 ms; 32 x 16 of the planned kernel 14.8 ms)
-    if (a.plan.N == 512 && launch_line_tp(a, s)) return;
-  } else {
+  if constexpr (sizeof(T) == 8) {
     if (a.plan.N == 512 && launch_line_tp64(a, s)) return;
   }
   if (launch_plan_line(a, s)) return;

@@ -1,7 +1,10 @@
 // Length-512 transforms of the matvec (Section V.B) for 256-voxel grid edges
-// (P = 512): the x and y line stages and the fused z stage (zero-padded
-// forward z-FFT, voxel-wise product with the rebuilt or stored spectra,
-// cropped inverse z-FFT).
+// (P = 512): the fused z stage (zero-padded forward z-FFT, voxel-wise product
+// with the rebuilt or stored spectra, cropped inverse z-FFT) and the FP64 x and y
+// line stages.  The FP32 line stages are the planned 32 x 16 kernels: with eight
+// 256^3 right-hand sides x 2.0, y 3.9, inverse y 3.5 and inverse x 2.6 ms with its
+// epilogue, against 2.4, 4.2, 3.9 and 4.1 ms for persistent three-pass kernels
+// fed by TMA tiles, which one exchange and one barrier per line beat.
 //
 // Three radix-8 passes, 64 threads per line, 8 values per thread.  With
 // n = a + 64 b (a < 64, b < 8), a = e + 8 f and k = c + 8 g + 64 h,
@@ -24,7 +27,7 @@
 #include <algorithm>
 
 #include "stages.cuh"
-#include "tma.cuh"
+#include "mbar.cuh"
 
 namespace vie {
 
@@ -76,48 +79,12 @@ __device__ __forceinline__ void pass1(C (&v)[8], int a, const C* roots, C* x1, i
   for (int c = 0; c < 8; ++c) x1[c * la + a] = v[c];
 }
 
-// pass 2 in thread (c, e): X1[c][e + 8f]  ->  X2[c][g][e]
-template <bool INV, typename C>
-__device__ __forceinline__ void pass2(int c, int e, const C* x1, int la, C* x2, const C* roots) {
-  C u[8];
-#pragma unroll
-  for (int f = 0; f < 8; ++f) u[f] = x1[c * la + e + 8 * f];
-  dft8<C, typename RealOf<C>::type>(u, INV);
-#pragma unroll
-  for (int g = 1; g < 8; ++g) u[g] = u[g] * root(roots, 8 * e * g, INV);
-#pragma unroll
-  for (int g = 0; g < 8; ++g) x2[c * 72 + 9 * g + e] = u[g];
-}
-
 // pass 3 in thread (c, g): X2[c][g][e]  ->  w[h] = X[c + 8 g + 64 h]
 template <bool INV, typename C>
 __device__ __forceinline__ void pass3(int c, int g, const C* x2, C (&w)[8]) {
 #pragma unroll
   for (int e = 0; e < 8; ++e) w[e] = x2[c * 72 + 9 * g + e];
   dft8<C, typename RealOf<C>::type>(w, INV);
-}
-
-// inverse of pass 3 in thread (c, g): w[h] = Y[c + 8g + 64h]  ->  X2[c][g][e]
-__device__ __forceinline__ void ipass3(int c, int g, float2 (&w)[8], float2* x2, const float2* roots) {
-  dft8<float2, float>(w, true);
-#pragma unroll
-  for (int e = 1; e < 8; ++e) w[e] = w[e] * root(roots, 8 * e * g, true);
-#pragma unroll
-  for (int e = 0; e < 8; ++e) x2[c * 72 + 9 * g + e] = w[e];
-}
-
-// inverse of pass 2 in thread (c, e): X2[c][g][e]  ->  X1[c][e + 8f]
-__device__ __forceinline__ void ipass2(int c, int e, const float2* x2, float2* x1, int la,
-                                       const float2* roots) {
-  float2 u[8];
-#pragma unroll
-  for (int g = 0; g < 8; ++g) u[g] = x2[c * 72 + 9 * g + e];
-  dft8<float2, float>(u, true);
-#pragma unroll
-  for (int f = 0; f < 8; ++f) {
-    const int a = e + 8 * f;
-    x1[c * la + a] = (c == 0) ? u[f] : u[f] * root(roots, a * c, true);
-  }
 }
 
 // inverse of pass 1 in thread a: X1[c][a]  ->  v[b] = 512 x[a + 64 b]
@@ -188,282 +155,6 @@ __device__ __forceinline__ void ipass2t(int t, const float2* x2, float2* x1, int
   dft8<float2, float>(u, true);
 #pragma unroll
   for (int f = 0; f < 8; ++f) x1[c * la + e + 8 * f] = u[f] * twv(tw, 14 + f, t, true);
-}
-
-// ---------------------------------------------------------------------------
-// x / y line stage: 8 adjacent columns per CTA, 64 threads per column.
-// Thread tid: column col = tid & 7, slot t = tid >> 3.  A warp's global
-// accesses are 4 rows x 64 contiguous bytes.  X1 column stride 514, X2 578
-// (both 2 mod 16 in float2 units).
-// ---------------------------------------------------------------------------
-constexpr int kLineCols = 8;
-constexpr int kCS1 = 514, kCS2 = 578;
-constexpr size_t kLineSmem = (size_t)kLineCols * (kCS1 + kCS2) * sizeof(float2);
-
-// INV: inverse transform (conjugate roots); HALF: forward from x[n < 256]
-// (the rest zero padding) or inverse cropped to outputs n < 256
-template <bool INV, bool HALF>
-__global__ void __launch_bounds__(512, 3) line_tp_kernel(const LineArgs<float> a) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  float2* sm = reinterpret_cast<float2*>(smem_raw);
-  const int tid = threadIdx.x, col = tid & 7, t = tid >> 3;
-  float2* x1 = sm + col * kCS1;
-  float2* x2 = sm + kLineCols * kCS1 + col * kCS2;
-  const int c0 = blockIdx.x * kLineCols, o = blockIdx.y, bb = blockIdx.z;
-  pdl_trigger();
-  pdl_wait();
-  if (a.active != nullptr && a.active[bb / a.batch_per_rhs] == 0) return;   // block-uniform
-  if (a.prof != nullptr && blockIdx.x == 0 && o == 0 && tid == 0) atomicAdd(a.prof, a.prof_batch_bytes);
-  const bool col_ok = c0 + col < a.ncol;
-  const float rs = (a.flags & (PRO_RSCALE | EPI_RSCALE))
-                       ? (float)a.rscale[(long long)(bb / a.batch_per_rhs) * a.rscale_stride]
-                       : 1.f;
-  const float2* in = a.in + bb * a.in_bs + o * a.in_os + (long long)(c0 + col);
-  float2 v[8];
-#pragma unroll
-  for (int b = 0; b < 8; ++b) {
-    const int p = t + kM * b;
-    float2 x = make_float2(0.f, 0.f);
-    if ((INV || !HALF || b < 4) && col_ok && p < a.lin) {
-      x = in[(long long)p * a.in_ls];
-      if (!INV) {
-        if (a.flags & PRO_RSCALE) x = rs * x;
-        if (a.flags & PRO_CONJ) x = conjg(x);
-        if (a.flags & PRO_CHI) x = a.chi[o * a.chi_os + (long long)p * a.chi_ls + (long long)(c0 + col)] * x;
-      }
-    }
-    v[b] = x;
-  }
-  pass1<INV, !INV && HALF>(v, t, a.roots, x1, 64);
-  __syncthreads();
-  pass2<INV>(t >> 3, t & 7, x1, 64, x2, a.roots);
-  __syncthreads();
-  const int c = t >> 3, g = t & 7;
-  pass3<INV>(c, g, x2, v);
-  float2* out = a.out + bb * a.out_bs + o * a.out_os + (long long)(c0 + col);
-  if (!col_ok) return;
-#pragma unroll
-  for (int h = 0; h < 8; ++h) {
-    if (INV && HALF && h >= 4) continue;
-    const int p = c + 8 * g + kM * h;
-    if (p >= a.lout) continue;
-    float2 x = v[h];
-    if (INV) {
-      x = a.scale * x;
-      if (a.flags & EPI_CONJ) x = conjg(x);
-      if (a.flags & (EPI_SUB | EPI_ADD)) {
-        if (a.flags & EPI_CHI) x = a.chi[o * a.chi_os + (long long)p * a.chi_ls + (long long)(c0 + col)] * x;
-        float2 w = a.addend[bb * a.out_bs + o * a.out_os + (long long)(c0 + col) + (long long)p * a.out_ls];
-        if (a.flags & EPI_RSCALE) w = rs * w;
-        x = (a.flags & EPI_SUB) ? (w - x) : (w + x);
-      }
-    }
-    out[(long long)p * a.out_ls] = x;
-  }
-}
-
-// ---------------------------------------------------------------------------
-// The same line stage as a persistent kernel whose input tiles arrive by TMA:
-// each CTA walks its tiles (8 columns x one line position range) through a
-// ring of `nstage` input buffers, so that the next tiles' copies are in
-// flight while the current one is transformed; one exchange buffer serves
-// as X1 and then as X2.  A tile is one or two boxes of 256 rows x 8 columns,
-// stored [row][column].
-// ---------------------------------------------------------------------------
-constexpr size_t kPipeX = (size_t)kLineCols * kCS2 * sizeof(float2);   // X1 / X2 (37 KB)
-constexpr size_t kTwBytes = (size_t)kTwRows * kM * sizeof(float2);       // 11 KB
-constexpr unsigned long long kWaitNs = 1000000000ull;     // 1 s per bounded wait
-constexpr int kMaxStages = 4;
-
-struct PipeTiles {
-  int ncg;              // column groups
-  int ntiles;           // ncg * nother * nbatch
-  int rows;             // input rows per tile (256 or 512)
-  int p_dim;            // tensor-map dimension of the line position (1 or 2; the other is `o`)
-  int nstage;           // ring depth (2 .. kMaxStages)
-};
-
-__host__ __device__ constexpr size_t pipe_stage_bytes(int rows) {
-  return (size_t)rows * kLineCols * sizeof(float2);
-}
-__host__ __device__ constexpr size_t pipe_smem(int rows, int nstage) {
-  return (size_t)nstage * pipe_stage_bytes(rows) + kPipeX + kTwBytes + kMaxStages * sizeof(uint64_t) +
-         1024;
-}
-
-// Position of a tile (column group, other index, batch index) of the CTA's
-// sequence blockIdx.x, blockIdx.x + G, ...: stepped by G with carries, no
-// divisions.
-struct TilePos {
-  int cg, o, bb;
-};
-struct TileStep {
-  int cg, o, bb;        // G split into the three digits (cg fastest)
-};
-
-template <bool INV, bool HALF, bool FLAGS>
-__global__ void __launch_bounds__(512, 2) line_tpp_kernel(const LineArgs<float> a,
-                                                        const __grid_constant__ CUtensorMap map,
-                                                        const PipeTiles pt) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  unsigned char* base = reinterpret_cast<unsigned char*>(
-      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  const int sbytes = (int)pipe_stage_bytes(pt.rows);
-  const int NS = pt.nstage;
-  auto stage = [&](int s) { return reinterpret_cast<float2*>(base + s * sbytes); };
-  float2* xb = reinterpret_cast<float2*>(base + NS * sbytes);
-  float2* tw = reinterpret_cast<float2*>(base + NS * sbytes + kPipeX);
-  uint64_t* bar = reinterpret_cast<uint64_t*>(base + NS * sbytes + kPipeX + kTwBytes);
-  const int tid = threadIdx.x, col = tid & 7, t = tid >> 3;
-  if (tid == 0) {
-    for (int q = 0; q < NS; ++q) mbar_init(&bar[q], 1);
-    mbar_fence_init();
-  }
-  fill_twiddles(tw, a.roots, tid, blockDim.x);
-  __syncthreads();
-  pdl_trigger();
-  pdl_wait();
-  const int ncg = pt.ncg, nother = a.nother, nbatch = a.nbatch;
-  TileStep st;
-  {
-    const int G = gridDim.x;
-    st.cg = G % ncg;
-    const int r = G / ncg;
-    st.o = r % nother;
-    st.bb = r / nother;
-  }
-  auto advance = [&](TilePos& q) {
-    q.cg += st.cg;
-    int carry = q.cg >= ncg;
-    if (carry) q.cg -= ncg;
-    q.o += st.o + carry;
-    carry = q.o >= nother;
-    if (carry) q.o -= nother;
-    q.bb += st.bb + carry;
-  };
-  // the next tile at or after q (in steps of G) whose right-hand side is active
-  auto settle = [&](TilePos& q) {
-    if (a.active == nullptr) return;
-    while (q.bb < nbatch && a.active[q.bb / 3] == 0) advance(q);
-  };
-  const int box_rows = pt.rows < 256 ? pt.rows : 256;
-  auto issue = [&](const TilePos& q, int s) {
-    mbar_arrive_expect_tx(&bar[s], (unsigned)sbytes);
-    for (int p0 = 0; p0 < pt.rows; p0 += box_rows) {
-      const int c1 = pt.p_dim == 1 ? p0 : q.o, c2 = pt.p_dim == 1 ? q.o : p0;
-      tma_load_4d(stage(s) + p0 * kLineCols, &map, q.cg * kLineCols, c1, c2, q.bb, &bar[s]);
-    }
-  };
-  TilePos cur;
-  {
-    const int b0 = blockIdx.x;
-    cur.cg = b0 % ncg;
-    const int r = b0 / ncg;
-    cur.o = r % nother;
-    cur.bb = r / nother;
-  }
-  settle(cur);
-  // the ring holds the tile cur and the next NS - 1 ones (ahead is the newest)
-  TilePos ahead = cur;
-  if (tid == 0 && cur.bb < nbatch) issue(cur, 0);
-  for (int q = 1; q < NS; ++q) {
-    if (ahead.bb < nbatch) {
-      advance(ahead);
-      settle(ahead);
-    }
-    if (tid == 0 && ahead.bb < nbatch) issue(ahead, q);
-  }
-  if (a.prof != nullptr && blockIdx.x == 0 && tid == 0) {
-    unsigned long long nb = 0;
-    for (int bb = 0; bb < nbatch; ++bb) nb += (a.active == nullptr || a.active[bb / 3]) ? 1 : 0;
-    atomicAdd(a.prof, nb * a.prof_batch_bytes);
-  }
-  const int c = t >> 3, g = t & 7;
-  const long long out_step = (long long)kM * a.out_ls;
-  int s = 0;
-  unsigned phase_bits = 0;                        // bit q: parity of the next wait on stage q
-  while (cur.bb < nbatch) {
-    const bool ok = mbar_wait_bounded(&bar[s], (phase_bits >> s) & 1u, kWaitNs);
-    if (__syncthreads_or(!ok)) {
-      if (tid == 0 && a.err != nullptr) atomicExch(a.err, VIE_ERR_TIMEOUT);
-      for (int q = 0; q < NS; ++q) mbar_wait_bounded(&bar[q], (phase_bits >> q) & 1u, kWaitNs);
-      return;
-    }
-    phase_bits ^= 1u << s;
-    const int o = cur.o, bb = cur.bb;
-    const int c0 = cur.cg * kLineCols;
-    const bool col_ok = c0 + col < a.ncol;
-    float rs = 1.f;
-    if (FLAGS && (a.flags & (PRO_RSCALE | EPI_RSCALE)))
-      rs = (float)a.rscale[(long long)(bb / 3) * a.rscale_stride];
-    const float2* S = stage(s) + col;
-    float2 v[8];
-#pragma unroll
-    for (int b = 0; b < 8; ++b) {
-      const int p = t + kM * b;
-      float2 x = make_float2(0.f, 0.f);
-      if (INV || !HALF || b < 4) {
-        x = S[p * kLineCols];
-        if (FLAGS && !INV) {
-          if (a.flags & PRO_RSCALE) x = rs * x;
-          if (a.flags & PRO_CONJ) x = conjg(x);
-          if ((a.flags & PRO_CHI) && col_ok)
-            x = a.chi[o * a.chi_os + (long long)p * a.chi_ls + (long long)(c0 + col)] * x;
-        }
-      }
-      v[b] = x;
-    }
-    __syncthreads();                       // stage s read; the exchange buffer is free
-    if (ahead.bb < nbatch) {
-      advance(ahead);
-      settle(ahead);
-    }
-    if (tid == 0 && ahead.bb < nbatch) {
-      fence_proxy_async_smem();
-      issue(ahead, s);
-    }
-    float2* x1 = xb + col * kCS1;
-    float2* x2 = xb + col * kCS2;
-    pass1t<INV, !INV && HALF>(v, t, tw, x1, 64);
-    __syncthreads();
-    {
-      float2 u[8];
-      pass2t_load<INV>(u, t, x1, 64, tw);
-      __syncthreads();                     // X1 read: X2 overwrites the same buffer
-#pragma unroll
-      for (int q = 0; q < 8; ++q) x2[c * 72 + 9 * q + g] = u[q];
-    }
-    __syncthreads();
-    pass3<INV>(c, g, x2, v);
-    if (col_ok) {
-      float2* out = a.out + bb * a.out_bs + o * a.out_os + (long long)(c0 + col) +
-                    (long long)(c + 8 * g) * a.out_ls;
-#pragma unroll
-      for (int h = 0; h < 8; ++h) {
-        if (INV && HALF && h >= 4) continue;
-        float2 x = v[h];
-        if (INV) {
-          x = a.scale * x;
-          if (FLAGS) {
-            const int p = c + 8 * g + kM * h;
-            if (a.flags & EPI_CONJ) x = conjg(x);
-            if (a.flags & (EPI_SUB | EPI_ADD)) {
-              if (a.flags & EPI_CHI)
-                x = a.chi[o * a.chi_os + (long long)p * a.chi_ls + (long long)(c0 + col)] * x;
-              float2 w = a.addend[bb * a.out_bs + o * a.out_os + (long long)(c0 + col) +
-                                  (long long)p * a.out_ls];
-              if (a.flags & EPI_RSCALE) w = rs * w;
-              x = (a.flags & EPI_SUB) ? (w - x) : (w + x);
-            }
-          }
-        }
-        out[h * out_step] = x;
-      }
-    }
-    s = (s + 1 == NS) ? 0 : s + 1;
-    advance(cur);
-    settle(cur);
-  }
 }
 
 // ---------------------------------------------------------------------------
@@ -598,6 +289,9 @@ __global__ void __launch_bounds__(256, 3) fused_tp_kernel(const FusedArgs<float>
   const float sx = ix ? -1.f : 1.f, sy = iy ? -1.f : 1.f;
   const int c = t >> 3, g = t & 7;
   __syncthreads();
+  // a line's 64 threads (two warps) exchange values only among themselves: a named
+  // barrier per line instead of the CTA's
+  auto line_sync = [&]() { asm volatile("bar.sync %0, 64;" ::"r"(1 + l) : "memory"); };
   for (int b = 0; b < a.B; ++b) {
     if (a.active != nullptr && a.active[b] == 0) continue;   // block-uniform
     float2 s[3][8];
@@ -611,14 +305,14 @@ __global__ void __launch_bounds__(256, 3) fused_tp_kernel(const FusedArgs<float>
         v[m] = (m < 4 && valid && p < n3) ? line[p] : make_float2(0.f, 0.f);
       }
       pass1t<false, true>(v, t, tw, x1, kLA);
-      __syncthreads();
+      line_sync();
       {
         float2 u[8];
         pass2t_load<false>(u, t, x1, kLA, tw);
 #pragma unroll
         for (int q = 0; q < 8; ++q) x2[c * 72 + 9 * q + (t & 7)] = u[q];
       }
-      __syncthreads();
+      line_sync();
       pass3<false>(c, g, x2, s[comp]);
     }
     // Y = D G D J at f = c + 8 g + 64 h
@@ -647,9 +341,9 @@ __global__ void __launch_bounds__(256, 3) fused_tp_kernel(const FusedArgs<float>
     for (int comp = 0; comp < 3; ++comp) {
       float2* line = a.data + (long long)(b * 3 + comp) * a.comp_stride + line_off;
       ipass3t(t, s[comp], x1, tw);
-      __syncthreads();
+      line_sync();
       ipass2t(t, x1, x2, kLA, tw);
-      __syncthreads();
+      line_sync();
       float2 v[8];
       ipass1(t, x2, kLA, v);
 #pragma unroll
@@ -664,73 +358,6 @@ __global__ void __launch_bounds__(256, 3) fused_tp_kernel(const FusedArgs<float>
 }
 
 }  // namespace tp
-
-static int g_sms = 0;
-
-// the TMA-pipelined persistent form: input rows 256 or 512, strides of 16-byte
-// multiples, 16-byte aligned input
-static bool launch_line_tpp(LineArgs<float> a, bool half, cudaStream_t s) {
-  const int rows = a.lin;
-  if (rows != 256 && rows != 512) return false;
-  // every tile's rows are loaded and, inverse and halved, its first 256 outputs
-  // stored: the kernel relies on lin = N (inverse) or N / 2 (forward halved)
-  // and lout = N / 2 (inverse halved) or N (forward)
-  if (a.inverse ? (rows != 512 || a.lout != (half ? 256 : 512)) : (a.lout != 512 || rows != (half ? 256 : 512)))
-    return false;
-  if (a.batch_per_rhs != 3) return false;
-  if (((uintptr_t)a.in & 15u) != 0 || a.in_os % 2 || a.in_ls % 2 || a.in_bs % 2) return false;
-  tp::PipeTiles pt;
-  pt.ncg = (a.ncol + tp::kLineCols - 1) / tp::kLineCols;
-  if ((long long)pt.ncg * a.nother * a.nbatch >= (1LL << 31)) return false;
-  pt.ntiles = pt.ncg * a.nother * a.nbatch;
-  pt.rows = rows;
-  pt.p_dim = a.in_ls < a.in_os ? 1 : 2;
-  const unsigned long long dp = (unsigned long long)rows, doth = (unsigned long long)a.nother;
-  const unsigned long long dims[4] = {(unsigned long long)a.ncol, pt.p_dim == 1 ? dp : doth,
-                                      pt.p_dim == 1 ? doth : dp, (unsigned long long)a.nbatch};
-  const unsigned long long strides[3] = {(unsigned long long)(pt.p_dim == 1 ? a.in_ls : a.in_os),
-                                         (unsigned long long)(pt.p_dim == 1 ? a.in_os : a.in_ls),
-                                         (unsigned long long)a.in_bs};
-  pt.nstage = rows == 256 ? 4 : 2;
-  const unsigned box_rows = rows < 256 ? rows : 256;
-  const unsigned box[4] = {(unsigned)tp::kLineCols, pt.p_dim == 1 ? box_rows : 1u,
-                           pt.p_dim == 1 ? 1u : box_rows, 1u};
-  CUtensorMap map;
-  if (encode_tensor_map_c64(&map, a.in, 4, dims, strides, box) != VIE_OK) return false;
-  if (g_sms == 0) g_sms = device_sms();
-  const long long grid = std::min<long long>(pt.ntiles, 2LL * g_sms);
-  a.prof = prof_bytes(a.prof_family);
-  ProfScope ps(a.prof_family, s);
-  const size_t smem = tp::pipe_smem(rows, pt.nstage);
-  using K = void (*)(LineArgs<float>, CUtensorMap, tp::PipeTiles);
-  static const K kernels[2][2][2] = {
-      {{tp::line_tpp_kernel<false, false, false>, tp::line_tpp_kernel<false, false, true>},
-       {tp::line_tpp_kernel<false, true, false>, tp::line_tpp_kernel<false, true, true>}},
-      {{tp::line_tpp_kernel<true, false, false>, tp::line_tpp_kernel<true, false, true>},
-       {tp::line_tpp_kernel<true, true, false>, tp::line_tpp_kernel<true, true, true>}}};
-  const K k = kernels[a.inverse ? 1 : 0][half ? 1 : 0][a.flags != 0 ? 1 : 0];
-  launch_pdl(k, dim3((unsigned)grid), dim3(512), smem, s, a, map, pt);
-  return true;
-}
-
-// x / y stage of a length-512 line (columns contiguous in memory)
-bool launch_line_tp(LineArgs<float> a, cudaStream_t s) {
-  if (a.plan.N != tp::kN || a.in_cs != 1 || a.out_cs != 1) return false;
-  if ((a.flags & (PRO_CHI | EPI_CHI)) && a.chi_cs != 1) return false;
-  if (a.nother > 65535 || a.nbatch > 65535) return false;
-  const bool half = a.inverse ? (2 * a.lout == tp::kN) : (2 * a.lin == tp::kN);
-  if (launch_line_tpp(a, half, s)) return true;
-  dim3 grid((a.ncol + tp::kLineCols - 1) / tp::kLineCols, a.nother, a.nbatch);
-  a.prof = prof_bytes(a.prof_family);
-  ProfScope ps(a.prof_family, s);
-  if (a.inverse)
-    launch_pdl(half ? tp::line_tp_kernel<true, true> : tp::line_tp_kernel<true, false>, grid,
-               dim3(512), tp::kLineSmem, s, a);
-  else
-    launch_pdl(half ? tp::line_tp_kernel<false, true> : tp::line_tp_kernel<false, false>, grid,
-               dim3(512), tp::kLineSmem, s, a);
-  return true;
-}
 
 // FP64 x / y stage of a length-512 line (columns contiguous in memory)
 bool launch_line_tp64(LineArgs<double> a, cudaStream_t s) {
@@ -763,55 +390,9 @@ void launch_fused_tp(const FusedArgs<float>& a, int groups, cudaStream_t s) {
 
 int tp_init_attributes() {
   cudaError_t e = cudaSuccess;
-  const int ls = (int)vie::tp::kLineSmem, fs = (int)vie::tp::kFusedSmem;
-  e = e != cudaSuccess ? e : cudaFuncSetAttribute(vie::tp::line_tp_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, ls);
-  e = e != cudaSuccess ? e : cudaFuncSetAttribute(vie::tp::line_tp_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ls);
-  e = e != cudaSuccess ? e : cudaFuncSetAttribute(vie::tp::line_tp_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, ls);
-  e = e != cudaSuccess ? e : cudaFuncSetAttribute(vie::tp::line_tp_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ls);
-  const int ps = (int)std::max(vie::tp::pipe_smem(256, 4), vie::tp::pipe_smem(512, 2));
-#define VIE_TPP_ATTR(I, H, F) \
-  e = e != cudaSuccess ? e : cudaFuncSetAttribute(vie::tp::line_tpp_kernel<I, H, F>, cudaFuncAttributeMaxDynamicSharedMemorySize, ps)
-  VIE_TPP_ATTR(false, false, false); VIE_TPP_ATTR(false, false, true);
-  VIE_TPP_ATTR(false, true, false); VIE_TPP_ATTR(false, true, true);
-  VIE_TPP_ATTR(true, false, false); VIE_TPP_ATTR(true, false, true);
-  VIE_TPP_ATTR(true, true, false); VIE_TPP_ATTR(true, true, true);
-#undef VIE_TPP_ATTR
+  const int fs = (int)vie::tp::kFusedSmem;
   e = e != cudaSuccess ? e : cudaFuncSetAttribute(vie::tp::fused_tp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, fs);
   return e == cudaSuccess ? VIE_OK : cuda_status(e, "length-512 kernel attributes");
-}
-
-// Host: tiled tensor map of 8-byte elements through the driver entry point
-// (looked up once; the library links only the runtime).
-int encode_tensor_map_c64(CUtensorMap* map, const void* base, int rank, const unsigned long long* dims,
-                          const unsigned long long* strides, const unsigned* box) {
-  using Encode = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                              const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                              CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-  static Encode fn = nullptr;
-  static bool looked = false;
-  if (!looked) {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-            cudaSuccess && q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<Encode>(p);
-    else
-      cudaGetLastError();
-    looked = true;
-  }
-  if (fn == nullptr || rank < 1 || rank > 5) return VIE_ERR_ARG;
-  cuuint64_t gd[5], gs[4];
-  cuuint32_t bd[5], es[5];
-  for (int i = 0; i < rank; ++i) {
-    gd[i] = dims[i];
-    bd[i] = box[i];
-    es[i] = 1;
-    if (i > 0) gs[i - 1] = strides[i - 1] * 8ull;
-  }
-  const CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, (cuuint32_t)rank, const_cast<void*>(base), gd,
-                        gs, bd, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                        CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? VIE_OK : VIE_ERR_ARG;
 }
 
 // ---------------------------------------------------------------------------

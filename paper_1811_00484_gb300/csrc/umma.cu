@@ -37,7 +37,7 @@
 // descriptor starts 256 bytes after the previous one.
 #include <algorithm>
 
-#include "tma.cuh"
+#include "mbar.cuh"
 
 namespace vie {
 
