@@ -83,9 +83,8 @@ __device__ __forceinline__ float2 wsum32(float2 v) {
   return v;
 }
 
-// dots: a tile is kDotThreads x kDotPacks packs; basis vectors kDotBlock at a time
+// dots: a tile is kDotThreads x 1, 2 or 4 packs (dot_packs); basis vectors kDotBlock at a time
 constexpr int kDotThreads = 128;
-constexpr int kDotPacks = 4;
 constexpr int kDotBlock = 4;
 constexpr int kMaxDotCtas = 4096;             // per right-hand side (bounds the partials)
 // update: one pack per thread, basis vectors kUpdBlock at a time
@@ -96,7 +95,7 @@ constexpr int kUpdBlock = 4;
 // Products and warp sums in FP32 (the data are FP32); sums across tiles, warps
 // and CTAs in FP64 (GB300's FP64 rate is far below its FP32 rate, so FP64
 // stays out of per-element work).
-template <int W>
+template <int W, int kDotPacks>
 __global__ void __launch_bounds__(kDotThreads) dots_kernel(const float2* __restrict__ V,
                                                            const float2* __restrict__ w, int k, int B,
                                                            long long N, int G, int ps, double2* partial,
@@ -214,12 +213,16 @@ __global__ void __launch_bounds__(kUpdThreads) update_kernel(const float2* __res
                                                              int k, int m, int B, long long N, int G,
                                                              double* nrm_partial, int* ticket,
                                                              int mode, double* nrm_out, int* again,
-                                                             const int* mask,
+                                                             const int* mask, const int* active,
+                                                             int* mv_active,
                                                              unsigned long long* prof,
                                                              unsigned long long prof_bytes) {
   const int b = blockIdx.y, cta = blockIdx.x;
   pdl_trigger();
   pdl_wait();
+  // the next matvec's copy of the active flags, taken before the Givens step of
+  // this column can change them (see arnoldi_step)
+  if (cta == 0 && threadIdx.x == 0) mv_active[b] = active[b];
   if (!mask[b]) return;
   if (prof != nullptr && cta == 0 && threadIdx.x == 0) atomicAdd(prof, prof_bytes);
   __shared__ float2 c[129];
@@ -313,11 +316,16 @@ __global__ void __launch_bounds__(kUpdThreads) update_kernel(const float2* __res
 
 // One Givens step per right-hand side (one warp each): finish column k
 // (h_{k+1,k} = nrm), apply the k earlier rotations, form the new one, update
-// g and test convergence.  The column and the rotations are staged in shared
-// memory so the sequential rotation chain does not wait on global memory.  It
-// runs beside the next matvec (which needs only sig[b][k+1]); its FP64 chain,
-// a few microseconds on a part with GB300's FP64 latency, is then off the
-// critical path.
+// g and test convergence.  It runs beside the next matvec (which needs only
+// sig[b][k+1]) and has to finish before that does.
+//
+// Rotation i takes (x_i, h_{i+1}) to t_i = c_i x_i + s_i h_{i+1} and x_{i+1} =
+// conj(c_i) h_{i+1} - s_i x_i (s_i is real): the x_i are a linear recurrence, so 32
+// rotations at a time are composed by a scan of the maps x -> a x + b over the
+// lanes.  A warp's FP64 instruction occupies its SM quarter for 64 clocks whether
+// one lane or 32 are active; one lane applying the rotations in turn took 0.69 us
+// each (10 us at column 5, 35 us at column 41, longer than the matvec of a 40^3
+// grid beside it).
 __global__ void __launch_bounds__(128) givens_kernel(double2* H, double2* cs, double2* sn, double2* g,
                                                      const double* nrm, int k, int m, int B,
                                                      int* active, int* again, int* iters,
@@ -335,26 +343,46 @@ __global__ void __launch_bounds__(128) givens_kernel(double2* H, double2* cs, do
     ss[warp][i] = s[i];
   }
   __syncwarp();
+  double2* hh = sh[warp];
+  double2 x0 = hh[0];
+  for (int i0 = 0; i0 < k; i0 += 32) {
+    const int i = i0 + lane;
+    const bool on = i < k;
+    const double2 ci = on ? sc[warp][i] : make_double2(1.0, 0.0);
+    const double si = on ? ss[warp][i].x : 0.0;
+    const double2 hn = on ? hh[i + 1] : make_double2(0.0, 0.0);
+    // inclusive scan: x_{i+1} = A x_{i0} + Bv
+    double A = on ? -si : 1.0;
+    double2 Bv = conjg(ci) * hn;
+    for (int d = 1; d < 32; d <<= 1) {
+      const double Ap = __shfl_up_sync(0xffffffffu, A, d);
+      const double bx = __shfl_up_sync(0xffffffffu, Bv.x, d), by = __shfl_up_sync(0xffffffffu, Bv.y, d);
+      if (lane >= d) {
+        Bv.x = fma(A, bx, Bv.x);
+        Bv.y = fma(A, by, Bv.y);
+        A *= Ap;
+      }
+    }
+    const double2 xn = make_double2(fma(A, x0.x, Bv.x), fma(A, x0.y, Bv.y));
+    double2 xi = make_double2(__shfl_up_sync(0xffffffffu, xn.x, 1), __shfl_up_sync(0xffffffffu, xn.y, 1));
+    if (lane == 0) xi = x0;
+    if (on) hh[i] = cmadd(ci, xi, si * hn);      // lane i has read hh[i + 1] of the old column
+    x0 = make_double2(__shfl_sync(0xffffffffu, xn.x, 31), __shfl_sync(0xffffffffu, xn.y, 31));
+    __syncwarp();
+  }
   if (lane == 0) {
     count[b] += 1;
-    double2* hh = sh[warp];
     const double hk1 = nrm[b];
-    hh[k + 1] = make_double2(hk1, 0.0);
-    for (int i = 0; i < k; ++i) {
-      const double2 ci = sc[warp][i], si = ss[warp][i];
-      const double2 t = ci * hh[i] + si * hh[i + 1];
-      hh[i + 1] = (-1.0) * (conjg(si) * hh[i]) + conjg(ci) * hh[i + 1];
-      hh[i] = t;
-    }
-    const double2 x = hh[k], y = hh[k + 1];
+    const double2 x = x0, y = make_double2(hk1, 0.0);
     const double den = sqrt(abs2(x) + abs2(y));
     double2 ck, sk;
     if (den == 0.0) {
       ck = make_double2(1.0, 0.0);
       sk = make_double2(0.0, 0.0);
     } else {
-      ck = (1.0 / den) * conjg(x);
-      sk = (1.0 / den) * conjg(y);
+      const double rden = 1.0 / den;
+      ck = rden * conjg(x);
+      sk = rden * conjg(y);
     }
     c[k] = ck;
     s[k] = sk;
@@ -648,6 +676,7 @@ struct SolverState {
   int nchunk = 0;
   int G = 0, Gu = 0;                // CTAs per RHS of the dots and update kernels
   int wide = 0;                     // 16-byte loads in dots / update (N even)
+  int dot_packs = 4;                // packs per thread of the dots kernel
   size_t bytes = 0;
   char* base = nullptr;
   float2 *V, *W, *d, *r32;
@@ -739,6 +768,12 @@ static size_t carve_bytes(int B, int m, long long N, int nchunk, int G, int Gu) 
   return (size_t)(p - (char*)nullptr);
 }
 
+// Packs per thread of the dots kernel: four where that still gives every SM a few
+// CTAs (64^3 voxels: 768), fewer on small grids, whose vectors would otherwise
+// occupy a fraction of the SMs (Arnoldi step at 24^3: 39.9 us with four packs, 35.7
+// us with one; at 50^3: 92.6 us with four, 86.8 us with two, 93.2 us with one).
+static int dot_packs(long long N) { return N < 131072 ? 1 : (N < 589824 ? 2 : 4); }
+
 static int get_state(vie_op* op, int B, int m, SolverState** out) {
   SolverState* st = static_cast<SolverState*>(op->solver);
   const long long N = 3LL * op->n[0] * op->n[1] * op->n[2];
@@ -748,7 +783,8 @@ static int get_state(vie_op* op, int B, int m, SolverState** out) {
   }
   const int wide = (N % 2 == 0) ? 1 : 0;
   const int W = wide ? 2 : 1;
-  const long long dtile = (long long)kDotThreads * kDotPacks * W;
+  const int packs = dot_packs(N);
+  const long long dtile = (long long)kDotThreads * packs * W;
   // tiles per CTA: as few as the cap on CTAs allows, and the same for every CTA
   const long long ntile = (N + dtile - 1) / dtile;
   const long long per = (ntile + kMaxDotCtas - 1) / kMaxDotCtas;
@@ -765,6 +801,7 @@ static int get_state(vie_op* op, int B, int m, SolverState** out) {
   st->G = G;
   st->Gu = Gu;
   st->wide = wide;
+  st->dot_packs = packs;
   st->bytes = carve_bytes(B, m, N, st->nchunk, st->G, st->Gu);
   cudaError_t e = cudaMalloc(&st->base, st->bytes);
   if (e != cudaSuccess) {
@@ -830,6 +867,12 @@ static int get_state(vie_op* op, int B, int m, SolverState** out) {
   return VIE_OK;
 }
 
+using DotsFn = void (*)(const float2*, const float2*, int, int, long long, int, int, double2*, const int*,
+                        unsigned long long*, unsigned long long);
+static DotsFn dots_variant(int wide, int packs) {
+  if (wide) return packs == 1 ? dots_kernel<2, 1> : packs == 2 ? dots_kernel<2, 2> : dots_kernel<2, 4>;
+  return packs == 1 ? dots_kernel<1, 1> : packs == 2 ? dots_kernel<1, 2> : dots_kernel<1, 4>;
+}
 // Wait on stream s for the Givens step running on the side stream.
 static int join_givens(SolverState* st, cudaStream_t s) {
   if (!st->givens_pending) return VIE_OK;
@@ -863,10 +906,10 @@ static int arnoldi_step(const vie_op* op, SolverState* st, const float2* chi, in
   // the cycle tail's) starts beside this step's Gram-Schmidt work
   if (!adjoint)
     VIE_TRY(matvec_impl<float>(op, vk, w, B, path, 0, EPI_SUB | EPI_CHI, chi, vk, st->mv_active, s,
-                               st->sig + k, m + 1));
+                               st->sig + k, m + 1, MV_SEPARATE));
   else
     VIE_TRY(matvec_impl<float>(op, vk, w, B, path, PRO_CONJ | PRO_CHI, EPI_CONJ | EPI_SUB, chi, vk,
-                               st->mv_active, s, st->sig + k, m + 1));
+                               st->mv_active, s, st->sig + k, m + 1, MV_SEPARATE));
   VIE_TRY(join_givens(st, s));
   const unsigned long long vec = (unsigned long long)N * sizeof(float2);
   for (int pass = 0; pass < passes; ++pass) {
@@ -874,7 +917,7 @@ static int arnoldi_step(const vie_op* op, SolverState* st, const float2* chi, in
     const int mode = (pass == 0 && passes > 1) ? UPD_DGKS : UPD_FINAL;
     {
       ProfScope ps(PF_DOTS, s);
-      launch_pdl(st->wide ? dots_kernel<2> : dots_kernel<1>, dim3(G, B), dim3(kDotThreads), 0, s,
+      launch_pdl(dots_variant(st->wide, st->dot_packs), dim3(G, B), dim3(kDotThreads), 0, s,
                  (const float2*)st->V, (const float2*)w, k, B, N, G, m + 1, st->partial, mask,
                  prof_bytes(PF_DOTS), (k + 2) * vec);
     }
@@ -891,13 +934,12 @@ static int arnoldi_step(const vie_op* op, SolverState* st, const float2* chi, in
       ProfScope ps(PF_UPDATE, s);
       launch_pdl(st->wide ? update_kernel<2> : update_kernel<1>, dim3(Gu, B), dim3(kUpdThreads), 0,
                  s, (const float2*)st->V, w, (const double2*)st->coef, st->sig, k, m, B, N, Gu,
-                 st->nrm_partial, st->ticket, mode, st->nrm, st->again, mask,
-                 prof_bytes(PF_UPDATE), (k + 3) * vec);
+                 st->nrm_partial, st->ticket, mode, st->nrm, st->again, mask, (const int*)st->active,
+                 st->mv_active, prof_bytes(PF_UPDATE), (k + 3) * vec);
     }
   }
-  // the Givens step beside the next matvec (which reads the flags as they are now)
-  if (k + 1 < m)
-    VIE_CUDA(cudaMemcpyAsync(st->mv_active, st->active, flag_bytes, cudaMemcpyDeviceToDevice, s));
+  // the Givens step beside the next matvec (which reads the update kernel's copy of
+  // the flags)
   VIE_CUDA(cudaEventRecord(st->ev_fork, s));
   VIE_CUDA(cudaStreamWaitEvent(st->aux, st->ev_fork, 0));
   {
@@ -927,10 +969,11 @@ static int cycle_tail(const vie_op* op, SolverState* st, const float2* chi, int 
   }
   // W = A d for the RHS still wanted
   if (!adjoint)
-    VIE_TRY(matvec_impl<float>(op, st->d, st->W, B, path, 0, EPI_SUB | EPI_CHI, chi, st->d, st->want, s));
+    VIE_TRY(matvec_impl<float>(op, st->d, st->W, B, path, 0, EPI_SUB | EPI_CHI, chi, st->d, st->want, s,
+                               nullptr, 0, MV_SEPARATE));
   else
     VIE_TRY(matvec_impl<float>(op, st->d, st->W, B, path, PRO_CONJ | PRO_CHI, EPI_CONJ | EPI_SUB, chi,
-                               st->d, st->want, s));
+                               st->d, st->want, s, nullptr, 0, MV_SEPARATE));
   {
     ProfScope ps(PF_SMALL, s);
     residual32_kernel<<<grid, kThreads, 0, s>>>(st->r32, st->W, st->V, N, nc, st->nrm_partial,
