@@ -205,15 +205,14 @@ template <int Q1, int Q2> cudaError_t prepare_plan_line(float) {
 // fused z stage
 // ---------------------------------------------------------------------------
 // Threads per line: one per slot of the widest pass, or, where that makes a group
-// one warp (eight butterflies a line) or the first
-// radix is so large that registers limit the threads anyway, only the M1
-// butterflies of the first pass, later passes looping over their slots (N = 128
-// with 8 right-hand sides: 16 threads 171 us, 8 threads 165 us; N = 112: 37 and
-// 30 us; N = 216: 357 and 295 us; but N = 160: 97 and 122 us, N = 40: 9.7 and
-// 13.2 us).
+// one warp (eight butterflies a line, radix 12 and up) or the first radix is so
+// large that registers limit the threads anyway, only the M1 butterflies of the
+// first pass, later passes looping over their slots (N = 128 with 8 right-hand
+// sides: 16 threads 171 us, 8 threads 165 us; N = 112: 37 and 30 us; N = 216: 357
+// and 295 us; but N = 160: 97 and 122 us, N = 80: 8.4 and 11.5 us).
 __host__ __device__ constexpr int fused_slots(int R1, int R2, int R3) {
   const int M1 = R2 * R3, wide = imax(imax(M1, R1 * R3), R3 > 1 ? R1 * R2 : R1);
-  return R3 == 1 && (M1 == 8 || R1 >= 18) ? M1 : wide;
+  return R3 == 1 && ((M1 == 8 && R1 >= 12) || R1 >= 18) ? M1 : wide;
 }
 
 template <int R1, int R2, int R3> struct FusedPlan {
