@@ -286,17 +286,21 @@ constexpr int kJacobiMaxPairs = 257;
 
 // Parallel cyclic Jacobi (round-robin pairing, all disjoint rotations of a step
 // applied at once), one cluster of eight CTAs per matrix, every matrix of the
-// operator in one launch.  A pair (p, q) is rotated when |a_pq| > tol
-// sqrt(|a_pp a_qq|); the sweep loop stops after a sweep without rotations or
-// after max_sweeps (status -1).
+// operator in one launch.  A pair (p, q) is rotated when |a_pq|^2 > tol^2
+// |a_pp a_qq|; the sweep loop stops after a sweep without rotations or after
+// max_sweeps (status -1).
 //
-// A step is bound by FP64 arithmetic (2 fused multiply-adds per clock and SM), so
-// it is spread over SMs and the Hermitian half is not computed: the rotations are
-// formed by the CTAs in turn and written into every CTA's shared memory
-// (distributed shared memory), then each 2 x 2 block (pair i, pair j >= i) of A is
-// rotated from both sides by one thread, which also writes its mirror image, and
-// each row of V by pairs.  Two cluster barriers a step.  A and V change hands
-// between SMs through L2.
+// A step is bound by FP64 issue (a warp instruction occupies its SM quarter for 64
+// clocks, with one lane or 32), so it is spread over the cluster's 32 quarters, warp
+// by warp, with full warps:
+//   1. the first warp of every CTA forms the rotations of its pairs and writes them
+//      into every CTA's shared memory, while the warps of the other quarters apply
+//      the previous step's rotations to V;
+//   2. each 2 x 2 block (pair i, pair j > i) of A is rotated from both sides by one
+//      thread, which also writes its mirror image.
+// One cluster barrier after each.  A and V change hands between SMs through L2.
+// 65 x 65 matrices: 14.3 ms a pass with the rotations' square roots and divisions
+// taken one by one, V in a third phase and half-empty warps.
 __global__ void __launch_bounds__(kJacobiThreads) jacobi_kernel(const JacobiJob* jobs, int max_sweeps,
                                                                 double tol, int* rotated, int* status) {
   namespace cg = cooperative_groups;
@@ -307,64 +311,98 @@ __global__ void __launch_bounds__(kJacobiThreads) jacobi_kernel(const JacobiJob*
   const int m = job.m, mm = m + (m & 1), M = mm - 1, npair = mm / 2;
   double2* A = job.A;
   double2* V = job.V;
-  __shared__ JacobiRot rot[kJacobiMaxPairs];
-  const int gt = rank * kJacobiThreads + threadIdx.x, gn = kJacobiCtas * kJacobiThreads;
+  __shared__ JacobiRot rots[2][kJacobiMaxPairs];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  constexpr int kWarps = kJacobiThreads / 32;
+  const int gt = (warp * kJacobiCtas + rank) * 32 + lane, gn = kJacobiCtas * kJacobiThreads;
+  // V's warps: those off the first quarter (warps 0 and 4 share it)
+  const int vwarp = warp < 4 ? warp - 1 : warp - 2, vn = (kWarps - 2) * kJacobiCtas * 32;
+  const bool on_v = (warp & 3) != 0;
+  const int nblk = npair * (npair - 1) / 2;
+  const double tol2 = tol * tol;
   for (int e = gt; e < m * m; e += gn) V[e] = make_double2((e / m) == (e % m) ? 1.0 : 0.0, 0.0);
   cluster.sync();
-  int sweep = 0;
-  bool done = (m <= 1);
+  auto update_v = [&](const JacobiRot* rot) {            // V <- V J
+    if (!on_v) return;
+    for (int it = (vwarp * kJacobiCtas + rank) * 32 + lane; it < npair * m; it += vn) {
+      const int k = it / npair, bj = it - k * npair;
+      const JacobiRot& rj = rot[bj];
+      if (rj.q < 0 || (rj.s.x == 0.0 && rj.s.y == 0.0)) continue;
+      const double2 vp = __ldcg(&V[k * m + rj.p]), vq = __ldcg(&V[k * m + rj.q]);
+      V[k * m + rj.p] = conj_madd(make_double2(-rj.s.x, -rj.s.y), vq, rj.c * vp);
+      V[k * m + rj.q] = cmadd(rj.s, vp, rj.c * vq);
+    }
+  };
+  int sweep = 0, buf = 0;
+  bool done = (m <= 1), pending = false;
   for (; sweep < max_sweeps && !done; ++sweep) {
     int* flag = rotated + jobid * max_sweeps + sweep;
-    for (int step = 0; step < M; ++step) {
-      // this CTA's pairs: rank, rank + 8, ...
-      const int i = rank + kJacobiCtas * (int)threadIdx.x;
-      if (i < npair) {
-        int p, q;
-        if (i == 0) { p = 0; q = 1 + step; }
-        else { p = 1 + (step + i) % M; q = 1 + (step - i + M) % M; }
-        if (p > q) { int t = p; p = q; q = t; }
-        JacobiRot r;
-        r.c = 1.0;
-        r.np = r.nq = 0.0;
-        r.s = make_double2(0.0, 0.0);
-        r.p = p;
-        r.q = q < m ? q : -1;
-        if (q < m) {
-          const double app = __ldcg(&A[p * m + p]).x, aqq = __ldcg(&A[q * m + q]).x;
-          const double2 apq = __ldcg(&A[p * m + q]);
-          const double mag = sqrt(abs2(apq));
-          if (mag > tol * sqrt(fabs(app * aqq)) && mag > 0.0) {
-            const double th = (aqq - app) / (2.0 * mag);
-            const double t = (th >= 0.0 ? 1.0 : -1.0) / (fabs(th) + sqrt(th * th + 1.0));
-            r.c = 1.0 / sqrt(t * t + 1.0);
-            const double sm = t * r.c / mag;
-            r.s = make_double2(sm * apq.x, sm * apq.y);          // s e^{i phi}
-            r.np = app - t * mag;                                 // rotated diagonal
-            r.nq = aqq + t * mag;
-            *flag = 1;
+    for (int step = 0; step < M; ++step, buf ^= 1) {
+      JacobiRot* rot = rots[buf];
+      if (warp == 0) {
+        // this CTA's pairs: rank, rank + 8, ...
+        for (int i = rank + kJacobiCtas * lane; i < npair; i += 32 * kJacobiCtas) {
+          int p, q;
+          if (i == 0) { p = 0; q = 1 + step; }
+          else { p = 1 + (step + i) % M; q = 1 + (step - i + M) % M; }
+          if (p > q) { int t = p; p = q; q = t; }
+          JacobiRot r;
+          r.c = 1.0;
+          r.np = r.nq = 0.0;
+          r.s = make_double2(0.0, 0.0);
+          r.p = p;
+          r.q = q < m ? q : -1;
+          if (q < m) {
+            const double app = __ldcg(&A[p * m + p]).x, aqq = __ldcg(&A[q * m + q]).x;
+            const double2 apq = __ldcg(&A[p * m + q]);
+            const double a2 = abs2(apq);
+            if (a2 > tol2 * fabs(app * aqq) && a2 > 0.0) {
+              const double rmag = rsqrt(a2), mag = a2 * rmag;
+              const double th = 0.5 * (aqq - app) * rmag, ath = fabs(th);
+              const double u = fma(th, th, 1.0);
+              // t = sign(th) / (|th| + sqrt(th^2 + 1))
+              const double t = copysign(1.0 / (ath + (ath > 1e9 ? ath : u * rsqrt(u))), th);
+              r.c = rsqrt(fma(t, t, 1.0));
+              const double sm = t * r.c * rmag;
+              r.s = make_double2(sm * apq.x, sm * apq.y);          // s e^{i phi}
+              r.np = fma(-t, mag, app);                             // rotated diagonal
+              r.nq = fma(t, mag, aqq);
+              *flag = 1;
+            }
           }
+          for (int k = 0; k < kJacobiCtas; ++k) cluster.map_shared_rank(rot, k)[i] = r;
         }
-        for (int k = 0; k < kJacobiCtas; ++k) cluster.map_shared_rank(rot, k)[i] = r;
+      } else if (pending) {
+        update_v(rots[buf ^ 1]);
       }
+      pending = true;
       cluster.sync();
-      // A <- J^* A J, the blocks (i, j >= i) and their mirror images
-      for (int it = gt; it < npair * npair; it += gn) {
-        const int bi = it / npair, bj = it - bi * npair;
-        if (bj < bi) continue;
-        const JacobiRot& ri = rot[bi];
-        const JacobiRot& rj = rot[bj];
-        const bool zi = ri.s.x == 0.0 && ri.s.y == 0.0, zj = rj.s.x == 0.0 && rj.s.y == 0.0;
-        if (zi && zj) continue;
-        if (bi == bj) {
+      // A <- J^* A J: the diagonal blocks, then the blocks (i, j > i) and their mirror
+      // images (the index runs along the rows of the strict upper triangle)
+      for (int it = gt; it < nblk + npair; it += gn) {
+        if (it >= nblk) {
           // the rotation annihilates a_pq exactly and moves t|a_pq| between a_pp and
           // a_qq; writing those values (instead of the rounded updates) lets the
           // relative stopping test be met on graded matrices
+          const JacobiRot& ri = rot[it - nblk];
+          if (ri.s.x == 0.0 && ri.s.y == 0.0) continue;
           A[ri.p * m + ri.p] = make_double2(ri.np, 0.0);
           A[ri.q * m + ri.q] = make_double2(ri.nq, 0.0);
           A[ri.p * m + ri.q] = make_double2(0.0, 0.0);
           A[ri.q * m + ri.p] = make_double2(0.0, 0.0);
           continue;
         }
+        // row bi starts at bi (2 npair - bi - 1) / 2
+        const float w = 2 * npair - 1;
+        int bi = (int)(0.5f * (w - sqrtf(w * w - 8.f * it)));
+        bi = max(0, min(bi, npair - 2));
+        while (bi > 0 && bi * (2 * npair - bi - 1) / 2 > it) --bi;
+        while (bi < npair - 2 && (bi + 1) * (2 * npair - bi - 2) / 2 <= it) ++bi;
+        const int bj = it - bi * (2 * npair - bi - 1) / 2 + bi + 1;
+        const JacobiRot& ri = rot[bi];
+        const JacobiRot& rj = rot[bj];
+        const bool zi = ri.s.x == 0.0 && ri.s.y == 0.0, zj = rj.s.x == 0.0 && rj.s.y == 0.0;
+        if (zi && zj) continue;
         const double2 z = make_double2(0.0, 0.0);
         const bool hi = ri.q >= 0, hj = rj.q >= 0;
         double2 pp = __ldcg(&A[ri.p * m + rj.p]), pq = hj ? __ldcg(&A[ri.p * m + rj.q]) : z;
@@ -396,19 +434,11 @@ __global__ void __launch_bounds__(kJacobiThreads) jacobi_kernel(const JacobiJob*
           A[rj.q * m + ri.q] = conjg(qq);
         }
       }
-      // V <- V J
-      for (int it = gt; it < npair * m; it += gn) {
-        const int k = it / npair, bj = it - k * npair;
-        const JacobiRot& rj = rot[bj];
-        if (rj.q < 0 || (rj.s.x == 0.0 && rj.s.y == 0.0)) continue;
-        const double2 vp = __ldcg(&V[k * m + rj.p]), vq = __ldcg(&V[k * m + rj.q]);
-        V[k * m + rj.p] = conj_madd(make_double2(-rj.s.x, -rj.s.y), vq, rj.c * vp);
-        V[k * m + rj.q] = cmadd(rj.s, vp, rj.c * vq);
-      }
       cluster.sync();
     }
     done = __ldcg(flag) == 0;            // the same for every CTA: set before the last barrier
   }
+  if (pending) update_v(rots[buf ^ 1]);
   if (rank == 0 && threadIdx.x == 0) status[jobid] = done ? sweep : -1;
 }
 
