@@ -10,14 +10,15 @@
 // coordinate), and so are the HOSVD factors of its unfoldings.  Only the half
 // fibres k3 <= P3/2 of the octant k1 <= P1/2, k2 <= P2/2 are rebuilt, and
 // each serves, with signs, the up-to-four z-lines (k1 | P1-k1, k2 | P2-k2)
-// of every right-hand side.  On the register path the half fibres of a chunk
+// of every right-hand side.  In FP32 the half fibres of a chunk
 // of k1 are rebuilt into an FP32 scratch (one k1 chunk at a time, so the
 // scratch stays a small fraction of the uncompressed spectra) by
 // octant_tc_kernel on the tensor cores (or octant_kernel with FP32 FMAs, or,
 // for the Tucker+CP model of eq. (17), octant_cp_kernel), and one CTA per
-// (k1, k2) mirror group copies its 6 x (P3/2 + 1) values to shared memory;
-// the multi-grid and shared-memory variants rebuild the fibre in the CTA.
-// The stored (uncompressed) variant reads the six spectra from memory instead.
+// (k1, k2) mirror group copies its 6 x (P3/2 + 1) values to shared memory (z
+// stages of the planned edges: planfft.cuh, planfft64.cuh, tp512.cu, plane.cu).
+// The general kernel here (edges without a plan) rebuilds the fibre in the CTA,
+// or reads the six stored spectra.
 #include <algorithm>
 
 #include "stages.cuh"

@@ -1,6 +1,7 @@
 // Strided line FFTs: the x- and y-axis stages of the zero-padded forward
 // FFT and of the cropped inverse FFT of the matvec (Section V.B), and the
-// full 3-D FFT of the FP64 spectrum assembly (Section V.A).
+// full 3-D FFT of the FP64 spectrum assembly (Section V.A): dispatch, and the
+// general kernel.
 //
 // One CTA transforms TW lines that sit next to each other in memory (a tile
 // of TW consecutive columns), so that every global load and store of a

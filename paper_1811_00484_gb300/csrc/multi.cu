@@ -97,21 +97,21 @@ __device__ __forceinline__ void multi_fused_body(const MultiFused& mf, long long
   const FusedArgs<float>& a = mf.a[p];
   if (mf.fs[p]) {
     switch (mf.R[p]) {
-      case 2: fused_fs_group<8, false>(a, g, smem); break;
-      case 4: fused_fs_group<16, false>(a, g, smem); break;
-      case 6: if constexpr (RMAX >= 6) fused_fs_group<24, false>(a, g, smem); break;
+      case 2: fused_fs_group<8>(a, g, smem); break;
+      case 4: fused_fs_group<16>(a, g, smem); break;
+      case 6: if constexpr (RMAX >= 6) fused_fs_group<24>(a, g, smem); break;
       default: break;
     }
     return;
   }
   switch (mf.R[p]) {
-    case 1: fused_warp_group<1, false>(a, g, smem); break;
-    case 2: fused_warp_group<2, false>(a, g, smem); break;
-    case 3: fused_warp_group<3, false>(a, g, smem); break;
-    case 4: fused_warp_group<4, false>(a, g, smem); break;
-    case 5: if constexpr (RMAX >= 5) fused_warp_group<5, false>(a, g, smem); break;
-    case 6: if constexpr (RMAX >= 6) fused_warp_group<6, false>(a, g, smem); break;
-    case 8: if constexpr (RMAX >= 8) fused_warp_group<8, false>(a, g, smem); break;
+    case 1: fused_warp_group<1>(a, g, smem); break;
+    case 2: fused_warp_group<2>(a, g, smem); break;
+    case 3: fused_warp_group<3>(a, g, smem); break;
+    case 4: fused_warp_group<4>(a, g, smem); break;
+    case 5: if constexpr (RMAX >= 5) fused_warp_group<5>(a, g, smem); break;
+    case 6: if constexpr (RMAX >= 6) fused_warp_group<6>(a, g, smem); break;
+    case 8: if constexpr (RMAX >= 8) fused_warp_group<8>(a, g, smem); break;
     default: break;
   }
 }

@@ -1,8 +1,15 @@
 // Matvec stages for every padded edge N = 2n with a factor plan: x / y line
 // stages (zero-padded forward, cropped inverse) and the fused z stage (forward
-// transform, voxel-wise product, inverse transform), in FP32 (planfft64.cuh: FP64).  All
-// lengths, strides in shared memory and radices are compile-time constants, so
-// the only index arithmetic left is one multiply-add per access.
+// transform, voxel-wise product, inverse transform), in FP32 (planfft64.cuh:
+// FP64).  All lengths, strides in shared memory and radices are compile-time
+// constants, so the only index arithmetic left is one multiply-add per access.
+//
+// What bounds them: the line stages the memory (96^3, 16 right-hand sides: x 192,
+// y 371, inverse y 319 and inverse x 168 us, 5.3 to 6.4 TB/s of their bytes; 363,
+// 701, 501 and 260 us with radices as uneven as 24 x 8), on small grids the latency of
+// one load, exchange and store; the z stage shared-memory wavefronts (60 to 70 % of
+// the peak) and issue (60 %) together (96^3, 16 right-hand sides: 983 us against
+// 1421 us for a four-step transform of one component per warp).
 //
 // Line stage, N = Q1 Q2, thread (col, t): columns are adjacent in memory.
 // With n = a + Q2 b, k = c + Q1 h,
@@ -51,9 +58,13 @@ __host__ __device__ constexpr int imin(int a, int b) { return a < b ? a : b; }
 // ---------------------------------------------------------------------------
 // Threads per column: the smaller radix when it divides the larger (every thread
 // then has the same work in both passes; with 16 threads for 16 x 8 half of them
-// waited at the barrier through pass 1), else the larger.
-__host__ __device__ constexpr int line_slots(int Q1, int Q2) {
-  return imax(Q1, Q2) % (Q1 + Q2 - imax(Q1, Q2)) == 0 ? Q1 + Q2 - imax(Q1, Q2) : imax(Q1, Q2);
+// waited at the barrier through pass 1), else the larger.  An inverse stage waits
+// for its loads, twice the forward one's: one thread per first-pass butterfly up
+// to radix 16 (N = 128, 8 right-hand sides: 58 us with 8 threads, 52 us with 16; N
+// = 512, 32 x 16: 921 us with 16 threads, 1096 us with 32).
+__host__ __device__ constexpr int line_slots(int Q1, int Q2, bool inv) {
+  const int big = imax(Q1, Q2), small = imin(Q1, Q2);
+  return inv && Q2 >= Q1 && Q2 <= 16 ? Q2 : (big % small == 0 ? small : big);
 }
 // columns per CTA: 128 bytes of a row, fewer when a line needs more than 16 threads
 __host__ __device__ constexpr int line_cols(int S) { return S <= 16 ? 16 : 8; }
@@ -64,17 +75,17 @@ __host__ __device__ constexpr int line_cols(int S) { return S <= 16 ? 16 : 8; }
 __host__ __device__ constexpr int line_regs(int R, int S) {
   return R <= 8 ? 48 : R <= 10 ? 56 : R <= 16 ? (S >= 12 ? 64 : 80) : R <= 21 ? 96 : 128;
 }
-__host__ __device__ constexpr int line_blocks(int Q1, int Q2) {
-  const int S = line_slots(Q1, Q2), th = line_cols(S) * S;
+__host__ __device__ constexpr int line_blocks(int Q1, int Q2, bool inv) {
+  const int S = line_slots(Q1, Q2, inv), th = line_cols(S) * S;
   const int b = 65536 / (line_regs(imax(Q1, Q2), S) * ((th + 31) / 32 * 32));
   return b < 1 ? 1 : (b > 24 ? 24 : b);
 }
 
 template <int Q1, int Q2, bool INV>
-__global__ void __launch_bounds__(line_cols(line_slots(Q1, Q2)) * line_slots(Q1, Q2), line_blocks(Q1, Q2))
+__global__ void __launch_bounds__(line_cols(line_slots(Q1, Q2, INV)) * line_slots(Q1, Q2, INV), line_blocks(Q1, Q2, INV))
     plan_line_kernel(const LineArgs<float> a) {
   using C = float2;
-  constexpr int S = line_slots(Q1, Q2);
+  constexpr int S = line_slots(Q1, Q2, INV);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* X = reinterpret_cast<C*>(smem_raw);               // [Q1][Q2][CW]
   const int CW = blockDim.x, col = threadIdx.x, t0 = threadIdx.y;
@@ -167,10 +178,9 @@ __global__ void __launch_bounds__(line_cols(line_slots(Q1, Q2)) * line_slots(Q1,
   }
 }
 
-// Q1 is even: forward Q1 x Q2, inverse Q2 x Q1 (the even radix where the half is)
-template <int Q1, int Q2> void launch_plan_line(LineArgs<float> a, cudaStream_t s) {
-  static_assert(Q1 % 2 == 0, "the pruned radix is even");
-  constexpr int S = line_slots(Q1, Q2), CMAX = line_cols(S);
+// kernel of the pass order Q1, Q2 (forward: Q1 even; inverse: Q2 even)
+template <int Q1, int Q2, bool INV> void launch_plan_line_order(LineArgs<float> a, cudaStream_t s) {
+  constexpr int S = line_slots(Q1, Q2, INV), CMAX = line_cols(S);
   // lines whose columns are adjacent across `o` too (the x stages) form one run
   if (a.in_os == a.ncol && a.out_os == a.ncol && (a.chi == nullptr || a.chi_os == a.ncol) &&
       (long long)a.ncol * a.nother < (1LL << 30)) {
@@ -178,18 +188,25 @@ template <int Q1, int Q2> void launch_plan_line(LineArgs<float> a, cudaStream_t 
     a.nother = 1;
   }
   // equal column groups: 50 columns are 4 groups of 13, not 3 of 16 and one of 2
-  const int tiles = (a.ncol + CMAX - 1) / CMAX;
+  // (vie_autotune may have chosen smaller CTAs than the default)
+  const int cmax = a.threads > 0 ? imin(CMAX, imax(4, a.threads / S)) : CMAX;
+  const int tiles = (a.ncol + cmax - 1) / cmax;
   const int cw = (a.ncol + tiles - 1) / tiles;
   a.prof = prof_bytes(a.prof_family);
   ProfScope ps(a.prof_family, s);
   const dim3 grid((unsigned)tiles, (unsigned)a.nother, (unsigned)a.nbatch), block((unsigned)cw, S);
-  const size_t smem = (size_t)Q1 * Q2 * cw * sizeof(float2);
-  if (a.inverse) launch_pdl(plan_line_kernel<Q2, Q1, true>, grid, block, smem, s, a);
-  else launch_pdl(plan_line_kernel<Q1, Q2, false>, grid, block, smem, s, a);
+  launch_pdl(plan_line_kernel<Q1, Q2, INV>, grid, block, (size_t)Q1 * Q2 * cw * sizeof(float2), s, a);
+}
+
+// Q1 is even: forward Q1 x Q2, inverse Q2 x Q1 (the even radix where the half is)
+template <int Q1, int Q2> void launch_plan_line(const LineArgs<float>& a, cudaStream_t s) {
+  static_assert(Q1 % 2 == 0, "the pruned radix is even");
+  if (a.inverse) launch_plan_line_order<Q2, Q1, true>(a, s);
+  else launch_plan_line_order<Q1, Q2, false>(a, s);
 }
 
 template <int Q1, int Q2> cudaError_t prepare_plan_line(float) {
-  constexpr size_t smem = (size_t)Q1 * Q2 * line_cols(line_slots(Q1, Q2)) * sizeof(float2);
+  constexpr size_t smem = (size_t)Q1 * Q2 * 16 * sizeof(float2);       // at most 16 columns
   if constexpr (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(plan_line_kernel<Q1, Q2, false>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

@@ -299,8 +299,9 @@ constexpr int kJacobiMaxPairs = 257;
 //   2. each 2 x 2 block (pair i, pair j > i) of A is rotated from both sides by one
 //      thread, which also writes its mirror image.
 // One cluster barrier after each.  A and V change hands between SMs through L2.
-// 65 x 65 matrices: 14.3 ms a pass with the rotations' square roots and divisions
-// taken one by one, V in a third phase and half-empty warps.
+// Eighteen 65 x 65 matrices: about 8 ms a pass (14.3 ms with the rotations' square
+// roots and divisions taken one by one, V in a third phase and half-empty warps; 20
+// ms for three of them with one CTA each).
 __global__ void __launch_bounds__(kJacobiThreads) jacobi_kernel(const JacobiJob* jobs, int max_sweeps,
                                                                 double tol, int* rotated, int* status) {
   namespace cg = cooperative_groups;

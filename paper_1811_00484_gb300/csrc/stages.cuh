@@ -1,6 +1,6 @@
-// Device bodies of the register-path (N = 32 R) matvec stages, shared by the
-// per-operator kernels (lines.cu, fused.cu) and the multi-grid kernels
-// (multi.cu): one x/y line tile, one fused z-line group, one slab-core block.
+// Arguments of the matvec's stages, and the device bodies of the multi-grid
+// kernels (multi.cu, edges N = 32 R): one x/y line tile, one fused z-line group;
+// one slab-core block.
 #pragma once
 
 #include "warpfft.cuh"
@@ -428,7 +428,7 @@ __host__ __device__ constexpr size_t fused_warp_smem(int R, int H3, int r2max, i
 // FFT, the voxel-wise product with the rebuilt (or stored) components in the
 // bit-reversed lane layout, and the inverse lane FFT.  The rebuild of the
 // half fibre (k3 <= P3/2) is shared by the CTA.  Every thread must call it.
-template <int R, bool STORED>
+template <int R>
 __device__ __forceinline__ void fused_warp_group(const FusedArgs<float>& a, int g, float2* smem) {
   using C = float2;
   constexpr int P3 = 32 * R;
@@ -451,7 +451,7 @@ __device__ __forceinline__ void fused_warp_group(const FusedArgs<float>& a, int 
   C* wv = ghalf + 6 * GS;              // [6][r3max]
   // prologue: tables and factors only (no earlier kernel writes them)
   for (int m = tid; m < P3; m += nth) roots[m] = a.roots[m];
-  const bool rebuild_here = !STORED && a.octant == nullptr;
+  const bool rebuild_here = a.octant == nullptr;
   if (rebuild_here) {
     for (int it = tid; it < 6 * a.r3max; it += nth) {
       const int c = it / a.r3max, gm = it % a.r3max;
@@ -502,7 +502,7 @@ __device__ __forceinline__ void fused_warp_group(const FusedArgs<float>& a, int 
     }
   };
   if (has_line && b0 < a.B) load_lines(b0);
-  if (!STORED && !rebuild_here) {
+  if (!rebuild_here) {
     // the group's half fibres, rebuilt for this matvec into the scratch
     const C* src = a.octant + ((long long)(k1 - a.oct_k1a) * a.H2 + k2) * 6 * H3;
     for (int it = tid; it < 6 * H3; it += nth) {
@@ -530,35 +530,22 @@ __device__ __forceinline__ void fused_warp_group(const FusedArgs<float>& a, int 
       const int kk = q + R * br;                       // z-frequency held in register q
       C gc[6];
       C jx = v[0][q], jy = v[1][q], jz = v[2][q];
-      float sz = 1.f;
-      if (STORED) {
-        const long long off = ((long long)kx * a.P2 + ky) * P3 + kk;
+      const bool zm = 2 * kk > P3;
+      const int fold = zm ? P3 - kk : kk;
+      const float sz = zm ? -1.f : 1.f;
+      const C* gp = ghalf + ghalf_slot(fold);
 #pragma unroll
-        for (int c = 0; c < 6; ++c) gc[c] = a.spec[c * a.spec_stride + off];
-      } else {
-        const bool zm = 2 * kk > P3;
-        const int fold = zm ? P3 - kk : kk;
-        sz = zm ? -1.f : 1.f;
-        const C* gp = ghalf + ghalf_slot(fold);
-#pragma unroll
-        for (int c = 0; c < 6; ++c) gc[c] = gp[c * GS];
-        jx = sx * jx;
-        jy = sy * jy;
-        jz = sz * jz;
-      }
+      for (int c = 0; c < 6; ++c) gc[c] = gp[c * GS];
+      jx = sx * jx;
+      jy = sy * jy;
+      jz = sz * jz;
       // Y_a = sum_b G_ab J_b with G symmetric: xx xy xz / xy yy yz / xz yz zz
       const C yx = gc[0] * jx + gc[1] * jy + gc[2] * jz;
       const C yy = gc[1] * jx + gc[3] * jy + gc[4] * jz;
       const C yz = gc[2] * jx + gc[4] * jy + gc[5] * jz;
-      if (STORED) {
-        v[0][q] = yx;
-        v[1][q] = yy;
-        v[2][q] = yz;
-      } else {
-        v[0][q] = sx * yx;
-        v[1][q] = sy * yy;
-        v[2][q] = sz * yz;
-      }
+      v[0][q] = sx * yx;
+      v[1][q] = sy * yy;
+      v[2][q] = sz * yz;
     }
 #pragma unroll
     for (int comp = 0; comp < 3; ++comp) {
@@ -590,7 +577,7 @@ __host__ __device__ constexpr size_t fused_fs_smem(int V, int H3) {
          sizeof(float2);
 }
 
-template <int V, bool STORED>
+template <int V>
 __device__ __forceinline__ void fused_fs_group(const FusedArgs<float>& a, int g, float2* smem) {
   using C = float2;
   constexpr int N = 8 * V;                     // P3
@@ -620,7 +607,7 @@ __device__ __forceinline__ void fused_fs_group(const FusedArgs<float>& a, int g,
     for (int b = 0; b < a.B; ++b) nb += (a.active == nullptr || a.active[b]) ? 1 : 0;
     atomicAdd(a.prof, nb * a.prof_rhs_bytes + a.prof_launch_bytes);
   }
-  if (!STORED) {
+  {
     // the group's half fibres, rebuilt for this matvec into the scratch
     const C* src = a.octant + ((long long)(k1 - a.oct_k1a) * a.H2 + k2) * 6 * H3;
     for (int it = tid; it < 6 * H3; it += nth) {
@@ -674,26 +661,13 @@ __device__ __forceinline__ void fused_fs_group(const FusedArgs<float>& a, int g,
 #pragma unroll
       for (int m = 0; m < V; ++m) {
         const int f = j + 8 * m;
-        C G0, G1, G2;
-        float sz = 1.f;
-        if (STORED) {
-          const long long off = ((long long)kx * a.P2 + ky) * N + f;
-          G0 = a.spec[g0 * a.spec_stride + off];
-          G1 = a.spec[g1 * a.spec_stride + off];
-          G2 = a.spec[g2 * a.spec_stride + off];
-        } else {
-          const bool zm = 2 * f > N;
-          const int fold = zm ? N - f : f;
-          sz = zm ? -1.f : 1.f;
-          const C* gp = ghalf + ghalf_slot(fold);
-          G0 = gp[g0 * GS];
-          G1 = gp[g1 * GS];
-          G2 = gp[g2 * GS];
-        }
-        // stored spectra are complete: no mirror signs
-        const float ex = STORED ? 1.f : sx, ey = STORED ? 1.f : sy;
-        C y = G0 * (ex * s0[f]) + G1 * (ey * s1[f]) + G2 * (sz * s2[f]);
-        if (!STORED) y = (comp == 2 ? sz : sc) * y;
+        const bool zm = 2 * f > N;
+        const int fold = zm ? N - f : f;
+        const float sz = zm ? -1.f : 1.f;
+        const C* gp = ghalf + ghalf_slot(fold);
+        const C G0 = gp[g0 * GS], G1 = gp[g1 * GS], G2 = gp[g2 * GS];
+        C y = G0 * (sx * s0[f]) + G1 * (sy * s1[f]) + G2 * (sz * s2[f]);
+        y = (comp == 2 ? sz : sc) * y;
         v[m] = y;
       }
       // inverse pass 1 (exchange buffer free: pass 2 read it before the barrier)

@@ -178,20 +178,6 @@ __device__ __forceinline__ void warp_fft_inv(C* v, int lane, const LaneConsts<C,
   (void)HALF;
 }
 
-// the original forms (per-call constants), kept for the FP64 and non-template users
-template <typename C, typename T, int R>
-__device__ __forceinline__ void warp_fft_fwd(C* v, int lane, const C* roots, int N) {
-  LaneConsts<C, T, R> lc;
-  lc.init(lane, roots, N);
-  warp_fft_fwd<C, T, R, false>(v, lc, roots, N);
-}
-template <typename C, typename T, int R>
-__device__ __forceinline__ void warp_fft_inv(C* v, int lane, const C* roots, int N) {
-  LaneConsts<C, T, R> lc;
-  lc.init(lane, roots, N);
-  warp_fft_inv<C, T, R, false>(v, lane, lc, roots, N);
-}
-
 // radices handled by the register path (N = 32 R <= 512)
 __host__ __device__ constexpr bool warp_fft_supported(int R) {
   return R == 1 || R == 2 || R == 3 || R == 4 || R == 5 || R == 6 || R == 8 || R == 10 || R == 12 ||
