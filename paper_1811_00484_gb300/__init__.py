@@ -144,14 +144,25 @@ def _check(status, where):
         raise VieError(status, where, detail)
 
 
+_torch_module = None
+
+
 def _torch():
-    import torch
-    return torch
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _torch_module = torch
+    return _torch_module
 
 
 def _stream():
+    """The current stream's handle (an int; the C functions take it as a pointer)."""
     torch = _torch()
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    if torch.cuda.is_initialized():
+        # without the Stream object that current_stream() makes (products of small
+        # grids are bound by the host: 16^3 takes three launches)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return torch.cuda.current_stream().cuda_stream
 
 
 def _precision(t):
@@ -169,9 +180,9 @@ def _dev(t, name, shape_tail=None):
         raise TypeError(f"{name} must be a CUDA tensor")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
-    if shape_tail is not None and tuple(t.shape[-len(shape_tail):]) != tuple(shape_tail):
+    if shape_tail is not None and t.shape[-len(shape_tail):] != shape_tail:
         raise ValueError(f"{name} has shape {tuple(t.shape)}, expected [..., {shape_tail}]")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _batch(t, n):
@@ -404,9 +415,9 @@ def solve_multi(ops, chis, rhss, incident=True, adjoint=False, tol=1e-6, restart
     opts = _solve_opts(tol, restart, max_outer, inner_tol, max_refine, path, use_graph, refine, orth)
     infs = (SolveInfo * count)()
     hs = (ctypes.c_void_p * count)(*[op._h.value for op in ops])
-    cp = (ctypes.c_void_p * count)(*[_dev(c, "chi", op.n).value for op, c in zip(ops, chis)])
-    rp = (ctypes.c_void_p * count)(*[_dev(r, "rhs", op.n).value for op, r in zip(ops, rhss)])
-    wp = (ctypes.c_void_p * count)(*[_dev(w, "w", op.n).value for op, w in zip(ops, ws)])
+    cp = (ctypes.c_void_p * count)(*[_dev(c, "chi", op.n) for op, c in zip(ops, chis)])
+    rp = (ctypes.c_void_p * count)(*[_dev(r, "rhs", op.n) for op, r in zip(ops, rhss)])
+    wp = (ctypes.c_void_p * count)(*[_dev(w, "w", op.n) for op, w in zip(ops, ws)])
     bs = (ctypes.c_int * count)(*[_batch(r, op.n) for op, r in zip(ops, rhss)])
     st = lib.vie_solve_multi(hs, cp, rp, wp, bs, count, flags, _precision(rhss[0]),
                              ctypes.byref(opts), infs, _stream())
@@ -430,8 +441,8 @@ def matvec_multi(ops, Js, outs=None, mode="persistent"):
         if J.dtype != torch.complex64:
             raise TypeError("vie_matvec_multi takes complex64")
     hs = (ctypes.c_void_p * count)(*[op._h.value for op in ops])
-    jp = (ctypes.c_void_p * count)(*[_dev(J, "J", op.n).value for op, J in zip(ops, Js)])
-    yp = (ctypes.c_void_p * count)(*[_dev(Y, "out", op.n).value for op, Y in zip(ops, outs)])
+    jp = (ctypes.c_void_p * count)(*[_dev(J, "J", op.n) for op, J in zip(ops, Js)])
+    yp = (ctypes.c_void_p * count)(*[_dev(Y, "out", op.n) for op, Y in zip(ops, outs)])
     bs = (ctypes.c_int * count)(*[_batch(J, op.n) for op, J in zip(ops, Js)])
     _check(lib.vie_matvec_multi_ex(hs, jp, yp, bs, count, MULTI_MODES[mode], _stream()),
            "vie_matvec_multi_ex")
