@@ -67,7 +67,12 @@ static bool radices_ok(int q1, int q2) {
   return (q1 == 4 || q1 == 6 || q1 == 8) && q2 >= 3 && q2 <= 7;
 }
 
-template <typename T> __global__ void __launch_bounds__(kThreads) plane_kernel(const PlaneArgs<T> a) {
+// resident CTAs per SM that the registers are held to (FP32: 80; without the limit
+// 89 allowed two, and 14 x 20 x 16 with 16 right-hand sides took two waves)
+constexpr int kPerSm = 3;
+
+template <typename T>
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kPerSm : 1) plane_kernel(const PlaneArgs<T> a) {
   using C = cx<T>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int tid = threadIdx.x;
@@ -290,7 +295,7 @@ template <typename T> bool plane_eligible(const vie_op* op, int B) {
   if ((size_t)6 * op->H[1] * (op->rmax[2] + op->H[2]) > all) return false;
   const size_t smem = all * sizeof(cx<T>);
   if (smem > plane::kSmemMax) return false;
-  const long long per_sm = std::min<long long>(4, (227 * 1024) / (smem + 1024));
+  const long long per_sm = std::min<long long>(sizeof(T) == 4 ? plane::kPerSm : 1, (227 * 1024) / (smem + 1024));
   return (long long)op->P[0] * B <= per_sm * device_sms();
 }
 
