@@ -278,13 +278,16 @@ static bool radices(int N, int* q1, int* q2) {
 
 }  // namespace plane
 
-// Small enough for the planes: y and z edges up to 24 voxels (24^3: 24.9 us against
-// the separate stages' host-bound 29.1 us; 28^3: 31.4 and 30.0 us), the planes of
-// all right-hand sides resident at once (one wave; each CTA rebuilds its plane's
-// entries, so more waves only repeat that), and no rebuild kernel chosen by flag.
+// Small enough for the planes: y and z edges up to 24 voxels, no rebuild kernel
+// chosen by flag, and few enough planes (each CTA rebuilds its plane's entries, so
+// waves of CTAs repeat that).  Where three planes fit an SM two waves still win (16
+// x 10 x 16 with 16 right-hand sides 22 us against 42 us for the separate stages,
+// 16^3 36 against 44 us); where two do, one (20^3: 17 us against 24 us with one or
+// two right-hand sides, the same from four on); where one does, half a wave (24^3:
+// 24.8 and 24.6 us with one, 27.7 and 24.6 us with two).
 // FP64 arithmetic is so slow that few CTAs lose more than the launches cost: there
-// only up to 9 x 9 voxels (8^3: 24 us either way, 8 right-hand sides 29 us against
-// 84 us; 12^3: 45 us against 30 us).
+// only up to 9 x 9 voxels (8^3: 24 us against 20 us, 8 right-hand sides 29 us against
+// 42 us; 12^3: 45 us against 30 us).
 template <typename T> bool plane_eligible(const vie_op* op, int B) {
   int q, z1, z2;
   if (op->flags & (VIE_REBUILD_SIMT | VIE_REBUILD_TCGEN05)) return false;
@@ -296,7 +299,11 @@ template <typename T> bool plane_eligible(const vie_op* op, int B) {
   const size_t smem = all * sizeof(cx<T>);
   if (smem > plane::kSmemMax) return false;
   const long long per_sm = std::min<long long>(sizeof(T) == 4 ? plane::kPerSm : 1, (227 * 1024) / (smem + 1024));
-  return (long long)op->P[0] * B <= per_sm * device_sms();
+  const int planes = sizeof(T) == 8 ? device_sms()
+                     : per_sm >= 3  ? 6 * device_sms()
+                     : per_sm == 2  ? 2 * device_sms()
+                                    : device_sms() / 2;
+  return (long long)op->P[0] * B <= planes;
 }
 
 template <typename T>
