@@ -167,7 +167,10 @@ typedef struct vie_op_info_t {
                                     compressing (released before it returned):
                                     the FP64 P1 P2 P3 spectrum of one component
                                     (spectrum route, or stored spectra), the
-                                    weighted octant, Gram matrices and vectors  */
+                                    weighted octants, Gram matrices and vectors
+                                    of the components compressed together (all
+                                    six on small grids; never more than 128 MiB
+                                    above one component's)                      */
     int rebuild_tiles[2];        /* rebuild_kernel 3: k3 columns of a CTA's
                                     range and CTAs per (component, range)
                                     (vie_autotune's choice, else the default

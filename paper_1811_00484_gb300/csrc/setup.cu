@@ -285,8 +285,8 @@ constexpr int kJacobiThreads = 256;
 constexpr int kJacobiMaxPairs = 257;
 
 // Parallel cyclic Jacobi (round-robin pairing, all disjoint rotations of a step
-// applied at once), one cluster of eight CTAs per matrix, every matrix of the
-// operator in one launch.  A pair (p, q) is rotated when |a_pq|^2 > tol^2
+// applied at once), one cluster of eight CTAs per matrix, every matrix of a group
+// of components in one launch.  A pair (p, q) is rotated when |a_pq|^2 > tol^2
 // |a_pp a_qq|; the sweep loop stops after a sweep without rotations or after
 // max_sweeps (status -1).
 //
@@ -470,30 +470,56 @@ template <typename P> int dalloc(P** p, size_t bytes) {
   return VIE_OK;
 }
 
+// Scratch of a setup that compresses `comps` components at a time; the arrays [6]
+// are indexed by the component's place in its group.
 struct DeviceBuffers {
+  int comps = 0;
   double2* full = nullptr;       // P1 P2 P3
-  double2* aw[6] = {};           // H1 H2 H3: every component's weighted octant
+  double2* aw[6] = {};           // H1 H2 H3: the group's weighted octants
   double2* tmp = nullptr;        // H1 H2 H3
   double2* gram[6][3] = {};      // Hq x Hq
   double2* vec[6][3] = {};       // Hq x Hq
   double2* vec2[6][3] = {};      // Hq x Hq
   double2* ytr = nullptr;        // truncated Y, max Hq x Hq
-  double2* part = nullptr;       // partial Gram matrices
+  double2* part = nullptr;       // partial Gram matrices: in `full` where they fit, the
+  double2* part_own = nullptr;   // spectrum being out of use by then, else here
   size_t part_entries = 0;
   JacobiJob* jobs = nullptr;     // [18]
   int* jstatus = nullptr;        // [18], then the sweeps' rotation flags [18][kJacobiSweeps]
   unsigned long long* red = nullptr;   // [6][2]
-  ~DeviceBuffers() {
-    cudaFree(full); cudaFree(tmp); cudaFree(ytr); cudaFree(part);
-    for (int c = 0; c < 6; ++c) {
-      cudaFree(aw[c]);
-      for (int q = 0; q < 3; ++q) { cudaFree(gram[c][q]); cudaFree(vec[c][q]); cudaFree(vec2[c][q]); }
+  void release_group() {
+    for (int i = 0; i < 6; ++i) {
+      cudaFree(aw[i]);
+      aw[i] = nullptr;
+      for (int q = 0; q < 3; ++q) {
+        for (double2** p : {&gram[i][q], &vec[i][q], &vec2[i][q]}) {
+          cudaFree(*p);
+          *p = nullptr;
+        }
+      }
     }
+  }
+  ~DeviceBuffers() {
+    cudaFree(full); cudaFree(tmp); cudaFree(ytr); cudaFree(part_own);
+    release_group();
     cudaFree(jobs); cudaFree(jstatus); cudaFree(red);
   }
 };
 
 constexpr int kJacobiSweeps = 60;
+
+// Components compressed at a time.  All six together keep the eigen-solver's SMs
+// busy, but hold six octants and 54 matrices: at 256^3 2.2 s with 4.1 GB of scratch
+// (factor-wise route, which is there to do without the 2.1 GB spectrum: 1.9 s, 1.95
+// GB), one by one 3.9 s with 2.7 GB (3.5 s, 0.55 GB).  So a group may hold
+// kSetupExtra more than one component's scratch: six together up to about 100^3
+// (96^3: 88 ms), three at 128^3 (258 ms; six 217 ms), one from about 200^3.
+constexpr size_t kSetupExtra = 128u << 20;
+int setup_group(size_t comp_bytes) {
+  for (int g : {6, 3, 2})
+    if ((g - 1) * comp_bytes <= kSetupExtra) return g;
+  return 1;
+}
 
 // upper-triangle 16 x 16 tiles of a D x D Gram matrix, and its column ranges: enough
 // CTAs for about four per SM
@@ -596,16 +622,18 @@ static void launch_gram(DeviceBuffers& d, const double2* X, double2* G, int q, c
   gram_sum_kernel<<<grid_for((long long)D * D), 256, 0, s>>>(d.part, G, D, nz);
 }
 
-// Diagonalise the 18 Gram matrices (6 components x 3 modes) in one launch.
-static int run_jacobi(DeviceBuffers& d, double2* (&V)[6][3], const int* H, cudaStream_t s) {
-  constexpr int kJobs = 18;
-  JacobiJob jobs[kJobs];
-  for (int j = 0; j < kJobs; ++j) jobs[j] = JacobiJob{d.gram[j / 3][j % 3], V[j / 3][j % 3], H[j % 3]};
-  int* flags = d.jstatus + kJobs;
-  VIE_CUDA(cudaMemcpyAsync(d.jobs, jobs, sizeof(jobs), cudaMemcpyHostToDevice, s));
-  VIE_CUDA(cudaMemsetAsync(flags, 0, kJobs * kJacobiSweeps * sizeof(int), s));
+// Diagonalise the Gram matrices of the group's components (first: c0; 3 modes each)
+// in one launch.
+static int run_jacobi(DeviceBuffers& d, int c0, double2* (&V)[6][3], const int* H, cudaStream_t s) {
+  constexpr int kMaxJobs = 18;
+  const int njobs = 3 * d.comps;
+  JacobiJob jobs[kMaxJobs];
+  for (int j = 0; j < njobs; ++j) jobs[j] = JacobiJob{d.gram[j / 3][j % 3], V[j / 3][j % 3], H[j % 3]};
+  int* flags = d.jstatus + kMaxJobs;
+  VIE_CUDA(cudaMemcpyAsync(d.jobs, jobs, njobs * sizeof(JacobiJob), cudaMemcpyHostToDevice, s));
+  VIE_CUDA(cudaMemsetAsync(flags, 0, njobs * kJacobiSweeps * sizeof(int), s));
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(kJobs * kJacobiCtas);
+  cfg.gridDim = dim3(njobs * kJacobiCtas);
   cfg.blockDim = dim3(kJacobiThreads);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -616,12 +644,12 @@ static int run_jacobi(DeviceBuffers& d, double2* (&V)[6][3], const int* H, cudaS
   cfg.numAttrs = 1;
   VIE_CUDA(cudaLaunchKernelEx(&cfg, jacobi_kernel, (const JacobiJob*)d.jobs, (int)kJacobiSweeps, 1e-15, flags,
                               d.jstatus));
-  int st[kJobs];
-  VIE_CUDA(cudaMemcpyAsync(st, d.jstatus, sizeof(st), cudaMemcpyDeviceToHost, s));
+  int st[kMaxJobs];
+  VIE_CUDA(cudaMemcpyAsync(st, d.jstatus, njobs * sizeof(int), cudaMemcpyDeviceToHost, s));
   VIE_CUDA(cudaStreamSynchronize(s));
-  for (int j = 0; j < kJobs; ++j) {
+  for (int j = 0; j < njobs; ++j) {
     if (st[j] < 0) {
-      set_error("Jacobi eigen-solver did not converge (component %d, matrix %d, size %d)", j / 3, j % 3,
+      set_error("Jacobi eigen-solver did not converge (component %d, matrix %d, size %d)", c0 + j / 3, j % 3,
                 H[j % 3]);
       return VIE_ERR_NUMERIC;
     }
@@ -653,16 +681,16 @@ static size_t rank_from_sigma2(const std::vector<double>& s2, double tol, int ru
 // the Toeplitz defining tensor, then the embedding and DFT of each factor
 // column; F_q E_q / sqrt(P_q) is an isometry, so both routes give the same
 // ranks and the same truncated model (core scaled by sqrt(P1 P2 P3)).
-// The components go through each stage together, so that the eigen-solver, a
-// long chain on few SMs per matrix, runs once per pass on all 18 matrices.
+// The components of a group go through each stage together, so that the eigen-solver,
+// a long chain on few SMs per matrix, runs once per pass on all their matrices.
 
 // dimensions of the weighted octant the HOSVD runs on
 static void octant_dims(const vie_op* op, bool factorwise, int* H) {
   for (int q = 0; q < 3; ++q) H[q] = factorwise ? op->n[q] : op->H[q];
 }
 
-// weighted octant of component c into d.aw[c]; its parity check into d.red[2 c]
-static int component_octant(vie_op* op, int c, DeviceBuffers& d, cudaStream_t s, bool factorwise) {
+// weighted octant of component c into aw; its parity check into d.red[2 c]
+static int component_octant(vie_op* op, int c, double2* aw, DeviceBuffers& d, cudaStream_t s, bool factorwise) {
   const int P1 = op->P[0], P2 = op->P[1], P3 = op->P[2];
   int H[3];
   octant_dims(op, factorwise, H);
@@ -682,35 +710,35 @@ static int component_octant(vie_op* op, int c, DeviceBuffers& d, cudaStream_t s,
     }
   }
   if (!factorwise) {
-    octant_kernel<<<grid_for(oct), 256, 0, s>>>(d.full, d.aw[c], P1, P2, P3, H[0], H[1], H[2]);
+    octant_kernel<<<grid_for(oct), 256, 0, s>>>(d.full, aw, P1, P2, P3, H[0], H[1], H[2]);
   } else {
     int ca, cb;
     component_axes(c, &ca, &cb);
-    toeplitz_octant_kernel<<<grid_for(oct), 256, 0, s>>>(d.aw[c], ca, cb, H[0], H[1], H[2], op->grid.h,
+    toeplitz_octant_kernel<<<grid_for(oct), 256, 0, s>>>(aw, ca, cb, H[0], H[1], H[2], op->grid.h,
                                                           op->k0, self_term_value(op));
   }
   VIE_CUDA(cudaGetLastError());
   return VIE_OK;
 }
 
-// Both eigen-solver passes of every component: d.vec and d.vec2 hold the
-// eigenvectors Y and V2, the diagonals of d.gram the squared singular values.
-static int component_eigenvectors(vie_op* op, DeviceBuffers& d, cudaStream_t s, bool factorwise) {
+// Both eigen-solver passes of the components [c0, c0 + d.comps): d.vec and d.vec2
+// hold the eigenvectors Y and V2, the diagonals of d.gram the squared singular values.
+static int component_eigenvectors(vie_op* op, int c0, DeviceBuffers& d, cudaStream_t s, bool factorwise) {
   int H[3];
   octant_dims(op, factorwise, H);
   const long long oct = (long long)H[0] * H[1] * H[2];
   VIE_CUDA(cudaMemsetAsync(d.red, 0, 12 * sizeof(unsigned long long), s));
   // pass 1: Gram matrices of the three unfoldings and their eigenvectors Y
-  for (int c = 0; c < 6; ++c) {
-    VIE_TRY(component_octant(op, c, d, s, factorwise));
-    for (int q = 0; q < 3; ++q) launch_gram(d, d.aw[c], d.gram[c][q], q, H, s);
+  for (int i = 0; i < d.comps; ++i) {
+    VIE_TRY(component_octant(op, c0 + i, d.aw[i], d, s, factorwise));
+    for (int q = 0; q < 3; ++q) launch_gram(d, d.aw[i], d.gram[i][q], q, H, s);
   }
   VIE_CUDA(cudaGetLastError());
   if (!factorwise || op->spec64 != nullptr) {
     unsigned long long red[12];
     VIE_CUDA(cudaMemcpyAsync(red, d.red, sizeof(red), cudaMemcpyDeviceToHost, s));
     VIE_CUDA(cudaStreamSynchronize(s));
-    for (int c = 0; c < 6; ++c) {
+    for (int c = c0; c < c0 + d.comps; ++c) {
       double dev, mx;
       std::memcpy(&dev, &red[2 * c], 8);
       std::memcpy(&mx, &red[2 * c + 1], 8);
@@ -722,23 +750,23 @@ static int component_eigenvectors(vie_op* op, DeviceBuffers& d, cudaStream_t s, 
       }
     }
   }
-  VIE_TRY(run_jacobi(d, d.vec, H, s));
+  VIE_TRY(run_jacobi(d, c0, d.vec, H, s));
   // pass 2: Gram of Y^* A_w^(q), eigenvectors V2; final vectors Y V2
-  for (int c = 0; c < 6; ++c) {
+  for (int i = 0; i < d.comps; ++i) {
     for (int q = 0; q < 3; ++q) {
       const long long Dpre = q == 0 ? 1 : (q == 1 ? H[0] : (long long)H[0] * H[1]);
       const long long Dpost = q == 0 ? (long long)H[1] * H[2] : (q == 1 ? H[2] : 1);
-      mode_product_kernel<<<grid_for(oct), 256, 0, s>>>(d.aw[c], d.tmp, d.vec[c][q], H[q], 1, Dpre, H[q],
+      mode_product_kernel<<<grid_for(oct), 256, 0, s>>>(d.aw[i], d.tmp, d.vec[i][q], H[q], 1, Dpre, H[q],
                                                         Dpost, H[q]);
-      launch_gram(d, d.tmp, d.gram[c][q], q, H, s);
+      launch_gram(d, d.tmp, d.gram[i][q], q, H, s);
     }
   }
   VIE_CUDA(cudaGetLastError());
-  return run_jacobi(d, d.vec2, H, s);
+  return run_jacobi(d, c0, d.vec2, H, s);
 }
 
-// Ranks, core and stored factors of component c from its eigenvectors.
-static int compress_component(vie_op* op, int c, double tol, int rule, DeviceBuffers& d,
+// Ranks, core and stored factors of component c from its eigenvectors (place i).
+static int compress_component(vie_op* op, int c, int i, double tol, int rule, DeviceBuffers& d,
                               cudaStream_t s, bool factorwise) {
   const int P1 = op->P[0], P2 = op->P[1], P3 = op->P[2];
   int H[3];
@@ -751,10 +779,10 @@ static int compress_component(vie_op* op, int c, double tol, int rule, DeviceBuf
   for (int q = 0; q < 3; ++q) {
     const int h = H[q];
     std::vector<double2> G2(h), YV((size_t)h * h);             // G2: the diagonal
-    VIE_CUDA(cudaMemcpy2DAsync(G2.data(), sizeof(double2), d.gram[c][q], (h + 1) * sizeof(double2),
+    VIE_CUDA(cudaMemcpy2DAsync(G2.data(), sizeof(double2), d.gram[i][q], (h + 1) * sizeof(double2),
                                sizeof(double2), h, cudaMemcpyDeviceToHost, s));
     // Y V2: view Y as [h][h][1] and contract its second index with V2
-    mode_product_kernel<<<grid_for((long long)h * h), 256, 0, s>>>(d.vec[c][q], d.ytr, d.vec2[c][q], h,
+    mode_product_kernel<<<grid_for((long long)h * h), 256, 0, s>>>(d.vec[i][q], d.ytr, d.vec2[i][q], h,
                                                                    0, h, h, 1, h);
     VIE_CUDA(cudaGetLastError());
     VIE_CUDA(cudaMemcpyAsync(YV.data(), d.ytr, YV.size() * sizeof(double2), cudaMemcpyDeviceToHost,
@@ -790,14 +818,14 @@ static int compress_component(vie_op* op, int c, double tol, int rule, DeviceBuf
   // core = A_w x1 Y1^* x2 Y2^* x3 Y3^*  (the truncated Y's go to d.vec2)
   const int r1 = tc.r[0], r2 = tc.r[1], r3 = tc.r[2];
   for (int q = 0; q < 3; ++q)
-    VIE_CUDA(cudaMemcpy(d.vec2[c][q], Ytr[q].data(), Ytr[q].size() * sizeof(double2),
+    VIE_CUDA(cudaMemcpy(d.vec2[i][q], Ytr[q].data(), Ytr[q].size() * sizeof(double2),
                         cudaMemcpyHostToDevice));
   mode_product_kernel<<<grid_for((long long)r1 * H[1] * H[2]), 256, 0, s>>>(
-      d.aw[c], d.tmp, d.vec2[c][0], r1, 1, 1, H[0], (long long)H[1] * H[2], r1);
+      d.aw[i], d.tmp, d.vec2[i][0], r1, 1, 1, H[0], (long long)H[1] * H[2], r1);
   mode_product_kernel<<<grid_for((long long)r1 * r2 * H[2]), 256, 0, s>>>(
-      d.tmp, d.aw[c], d.vec2[c][1], r2, 1, r1, H[1], H[2], r2);
+      d.tmp, d.aw[i], d.vec2[i][1], r2, 1, r1, H[1], H[2], r2);
   mode_product_kernel<<<grid_for((long long)r1 * r2 * r3), 256, 0, s>>>(
-      d.aw[c], d.tmp, d.vec2[c][2], r3, 1, (long long)r1 * r2, H[2], 1, r3);
+      d.aw[i], d.tmp, d.vec2[i][2], r3, 1, (long long)r1 * r2, H[2], 1, r3);
   VIE_CUDA(cudaGetLastError());
   const size_t ncore = (size_t)r1 * r2 * r3;
   VIE_TRY(dalloc(&tc.core64, ncore * sizeof(double2)));
@@ -938,7 +966,6 @@ int build_operator(const vie_grid* grid, double tol, int rank_rule, int flags, c
   int st = init_tables(op);
   if (st != VIE_OK) { vie_destroy(op); return st; }
   const long long full = (long long)op->P[0] * op->P[1] * op->P[2];
-  const long long oct = (long long)op->H[0] * op->H[1] * op->H[2];
   if (flags & VIE_STORE_UNCOMPRESSED) {
     if ((st = dalloc(&op->spec64, 6 * full * sizeof(double2))) != VIE_OK ||
         (st = dalloc(&op->spec32, 6 * full * sizeof(float2))) != VIE_OK) {
@@ -954,35 +981,52 @@ int build_operator(const vie_grid* grid, double tol, int rank_rule, int flags, c
     const bool need_full = !factorwise || (flags & VIE_STORE_UNCOMPRESSED);
     int H[3];
     octant_dims(op, factorwise, H);
-    const long long aw = (long long)H[0] * H[1] * H[2];
-    for (int q = 0; q < 3; ++q)
+    const size_t aw = (size_t)H[0] * H[1] * H[2];
+    size_t mats = 0;                                   // Gram matrix, Y and V2 of every mode
+    for (int q = 0; q < 3; ++q) {
+      mats += 3 * (size_t)H[q] * H[q];
       d.part_entries = std::max(d.part_entries, (size_t)gram_ranges(H[q], aw / H[q]) * H[q] * H[q]);
-    const size_t tmp = (size_t)std::max(oct, (long long)hmax * hmax);
-    op->setup_scratch_bytes = ((need_full ? (size_t)full : 0) + 6 * (size_t)aw + tmp + (size_t)hmax * hmax +
-                               d.part_entries) * sizeof(double2);
+    }
+    const size_t tmp = std::max(aw, (size_t)hmax * hmax);
+    const bool part_in_full = need_full && (size_t)full >= d.part_entries;
+    const size_t fixed = (need_full ? (size_t)full : 0) + tmp + (size_t)hmax * hmax +
+                         (part_in_full ? 0 : d.part_entries);
     if ((need_full && (st = dalloc(&d.full, full * sizeof(double2))) != VIE_OK) ||
         (st = dalloc(&d.tmp, tmp * sizeof(double2))) != VIE_OK ||
         (st = dalloc(&d.ytr, (size_t)hmax * hmax * sizeof(double2))) != VIE_OK ||
-        (st = dalloc(&d.part, d.part_entries * sizeof(double2))) != VIE_OK ||
+        (!part_in_full && (st = dalloc(&d.part_own, d.part_entries * sizeof(double2))) != VIE_OK) ||
         (st = dalloc(&d.jobs, 18 * sizeof(JacobiJob))) != VIE_OK ||
         (st = dalloc(&d.jstatus, 18 * (1 + kJacobiSweeps) * sizeof(int))) != VIE_OK ||
         (st = dalloc(&d.red, 12 * sizeof(unsigned long long))) != VIE_OK) {
       vie_destroy(op);
       return st;
     }
-    for (int c = 0; c < 6 && st == VIE_OK; ++c) {
-      st = dalloc(&d.aw[c], aw * sizeof(double2));
-      for (int q = 0; q < 3 && st == VIE_OK; ++q) {
-        const size_t hh = (size_t)H[q] * H[q] * sizeof(double2);
-        if ((st = dalloc(&d.gram[c][q], hh)) != VIE_OK || (st = dalloc(&d.vec[c][q], hh)) != VIE_OK ||
-            (st = dalloc(&d.vec2[c][q], hh)) != VIE_OK)
-          break;
-        op->setup_scratch_bytes += 3 * hh;
+    d.part = part_in_full ? d.full : d.part_own;
+    auto alloc_group = [&](int g) {
+      d.comps = g;
+      for (int i = 0; i < g; ++i) {
+        VIE_TRY(dalloc(&d.aw[i], aw * sizeof(double2)));
+        for (int q = 0; q < 3; ++q) {
+          const size_t hh = (size_t)H[q] * H[q] * sizeof(double2);
+          VIE_TRY(dalloc(&d.gram[i][q], hh));
+          VIE_TRY(dalloc(&d.vec[i][q], hh));
+          VIE_TRY(dalloc(&d.vec2[i][q], hh));
+        }
       }
+      return (int)VIE_OK;
+    };
+    st = alloc_group(setup_group((aw + mats) * sizeof(double2)));
+    if (st == VIE_ERR_OOM && d.comps > 1) {            // one component at a time may still fit
+      d.release_group();
+      clear_error();
+      st = alloc_group(1);
     }
-    if (st == VIE_OK) st = component_eigenvectors(op, d, s, factorwise);
-    for (int c = 0; c < 6 && st == VIE_OK; ++c)
-      st = compress_component(op, c, tol, rank_rule, d, s, factorwise);
+    op->setup_scratch_bytes = (fixed + d.comps * (aw + mats)) * sizeof(double2);
+    for (int c0 = 0; c0 < 6 && st == VIE_OK; c0 += d.comps) {
+      st = component_eigenvectors(op, c0, d, s, factorwise);
+      for (int i = 0; i < d.comps && st == VIE_OK; ++i)
+        st = compress_component(op, c0 + i, i, tol, rank_rule, d, s, factorwise);
+    }
     if (st == VIE_OK) {
       cudaError_t e = cudaStreamSynchronize(s);
       if (e != cudaSuccess) st = cuda_status(e, "compress");
