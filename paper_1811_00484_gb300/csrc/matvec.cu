@@ -153,6 +153,16 @@ LineStages<T> make_line_stages(const vie_op* op, void* ws, const cx<T>* in, cx<T
                          ((a.flags & (EPI_SUB | EPI_ADD)) ? (unsigned long long)(n1 * n2 * n3 * sizeof(C)) : 0ull) +
                          ((a.flags & EPI_CHI) ? (unsigned long long)(n1 * n2 * n3 * sizeof(C)) : 0ull);
   }
+  // CTAs of the next kernel that start early take the slots that happen to be free: a
+  // few SMs get most of them, and those SMs decide when that kernel ends, unless it
+  // has so many CTAs that they even out.  So the y stage lets the z stage start
+  // beside it from 20 mirror groups per SM on (FP64: 64^3, 4225 groups, 1176 us
+  // instead of 1188, but 50 x 48 x 45, 2499 groups, 600 instead of 583 and 32 x 8 x 32,
+  // 297 groups, 136 instead of 52; FP32, stored spectra: 64^3 90.5 instead of 91.2 for
+  // two right-hand sides, but 32 x 16 x 32, 561 groups, 59 instead of 34 for eight).
+  // Between the other stages it costs nothing in FP32 and never pays in FP64.
+  for (int i = 0; i < 4; ++i) st.s[i].early = sizeof(T) == 4;
+  st.s[1].early = (long long)op->H[0] * op->H[1] >= 20ll * device_sms();
   for (int i = 0; i < 4; ++i) {
     st.s[i].batch_per_rhs = 3;
     st.s[i].active = active;
@@ -193,10 +203,13 @@ int matvec_run(const vie_op* op, void* ws, const cx<T>* in, cx<T>* out, int B, i
   using C = cx<T>;
   const bool stored = (path == VIE_PATH_UNCOMPRESSED);
   const bool cp = (path == VIE_PATH_TUCKER_CP);
-  const LineStages<T> st = make_line_stages<T>(op, ws, in, out, B, pro_flags, epi_flags, chi,
-                                               addend, active, rscale, rscale_stride);
+  LineStages<T> st = make_line_stages<T>(op, ws, in, out, B, pro_flags, epi_flags, chi,
+                                         addend, active, rscale, rscale_stride);
   // a small grid: the y and z stages and the rebuild in one launch
   if (!cp && !(mv_flags & MV_SEPARATE) && vie::plane_eligible<T>(op, B)) {
+    // its CTAs have an SM each, and rebuild their planes meanwhile (8^3 in FP64: 24.5
+    // us, 34.5 us when they start after the x stage)
+    st.s[0].early = st.s[3].early = 1;
     launch_line_fft<T>(st.s[0], s);
     vie::launch_plane<T>(op, st.s[0].out, B, stored, active, s);
     launch_line_fft<T>(st.s[3], s);

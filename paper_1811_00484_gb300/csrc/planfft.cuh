@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(line_cols(line_slots(Q1, Q2, INV)) * line_slot
   C* X = reinterpret_cast<C*>(smem_raw);               // [Q1][Q2][CW]
   const int CW = blockDim.x, col = threadIdx.x, t0 = threadIdx.y;
   const int c0 = blockIdx.x * CW + col, o = blockIdx.y, bb = blockIdx.z;
-  pdl_trigger();
+  if (a.early) pdl_trigger();
   pdl_wait();
   if (a.active != nullptr && a.active[bb / a.batch_per_rhs] == 0) return;   // block-uniform
   if (a.prof != nullptr && blockIdx.x == 0 && o == 0 && col == 0 && t0 == 0)

@@ -8,7 +8,11 @@
 // and lines of mirror groups that do not exist are skipped.  With threads tied to a
 // line as in FP32, a 36-thread group or five butterflies for eight threads left up to
 // half of the issue slots to idle lanes: products of 20^3 143 -> 97 us, 36^3 with 8
-// right-hand sides 2537 -> 1515 us, 64^3 1281 -> 1173 us.
+// right-hand sides 2537 -> 1515 us, 64^3 1281 -> 1173 us (every kernel started early).
+//
+// For the same reason a kernel here does not let the next one start beside it (but
+// see make_line_stages and matvec_run): the SMs that get most of the early CTAs decide
+// when the next kernel ends.
 #pragma once
 
 #include "planfft.cuh"
@@ -29,7 +33,7 @@ __global__ void __launch_bounds__(kThreads64, blocks64<imax(Q1, Q2)>())
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* X = reinterpret_cast<C*>(smem_raw);               // [Q1][Q2][CW]
   const int c00 = blockIdx.x * CW, o = blockIdx.y, bb = blockIdx.z;
-  pdl_trigger();
+  if (a.early) pdl_trigger();
   pdl_wait();
   if (a.active != nullptr && a.active[bb / a.batch_per_rhs] == 0) return;   // block-uniform
   const int cw = min(CW, a.ncol - c00);
@@ -180,7 +184,6 @@ __global__ void __launch_bounds__(kThreads64, blocks64<imax(R1, imax(R2, R3))>()
       G[it] = src[c * a.spec_stride + kk];
     }
   }
-  pdl_trigger();
   pdl_wait();
   // line lc = 3 l + component
   auto line = [&](int b, int lc) {

@@ -174,7 +174,7 @@ __global__ void __launch_bounds__(256, 3) line_tp64_kernel(const LineArgs<double
   const int tid = threadIdx.x, col = tid & 3, t = tid >> 2;
   double2* x = reinterpret_cast<double2*>(smem_raw) + col * kX64;
   const int c0 = blockIdx.x * kCols64, o = blockIdx.y, bb = blockIdx.z;
-  pdl_trigger();
+  if (a.early) pdl_trigger();
   pdl_wait();
   if (a.active != nullptr && a.active[bb / a.batch_per_rhs] == 0) return;   // block-uniform
   const bool col_ok = c0 + col < a.ncol;

@@ -148,6 +148,7 @@ template <typename T> struct LineArgs {
   int chi_vec, addend_vec;             // chi / addend rows allow 16-byte accesses
   int batch_per_rhs;                   // batches per RHS (3 components) for `active`
   const int* active;                   // per-RHS flag (nullptr = all active)
+  int early;                           // the next kernel may start beside this one
   int threads;                         // CTA size of the planned FP32 kernel at most (0 = its default)
   int prof_family;                     // profiler family of this launch
   unsigned long long* prof;            // profiler byte counter (nullptr = off)

@@ -86,3 +86,36 @@ def test_plane_kernel_equals_the_separate_stages(n):
     assert float(torch.linalg.vector_norm(w - w2) / torch.linalg.vector_norm(w2)) <= 1e-4
     op.close()
     ref.close()
+
+
+def _time(op, J, path="tucker"):
+    """Best of eight runs of 20 products, ms."""
+    best, (a, b) = float("inf"), (torch.cuda.Event(enable_timing=True) for _ in range(2))
+    for _ in range(8):
+        op.matvec(J, path=path)
+        a.record()
+        for _ in range(20):
+            op.matvec(J, path=path)
+        b.record()
+        torch.cuda.synchronize()
+        best = min(best, a.elapsed_time(b))
+    return best
+
+
+@pytest.mark.parametrize("n", [(32, 8, 32), (16, 24, 24), (20, 20, 20)])
+def test_fp64_product_costs_less_than_two(n):
+    """The stages spread evenly over the SMs: one right-hand side takes less time than
+    two (it took more where CTAs of the next kernel crowded on a few SMs)."""
+    op = vie.Operator(n, H, F, 1e-6)
+    one, two = (_time(op, _field(n, B, 2, np.complex128)) for B in (1, 2))
+    assert one < 0.9 * two, (one, two)
+    op.close()
+
+
+def test_stored_product_costs_no_more_than_the_rebuilt_one():
+    """The same in FP32: here the stored path has the same stages and no rebuild."""
+    op = vie.Operator((32, 16, 32), H, F, 1e-6, store_uncompressed=True)
+    J = _field((32, 16, 32), 8, 2, np.complex64)
+    stored, rebuilt = _time(op, J, "uncompressed"), _time(op, J)
+    assert stored < rebuilt, (stored, rebuilt)
+    op.close()
