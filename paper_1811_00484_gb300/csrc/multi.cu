@@ -509,7 +509,8 @@ static int tune_rebuild_tiles(vie_op* op, cudaStream_t s, cudaEvent_t e0, cudaEv
 }
 
 // Time the FP32 Tucker matvec at batch B with each candidate CTA size of each
-// line stage (the other stages at their current choice) and keep the fastest;
+// line stage (the other stages at their current choice) and keep the fastest, with
+// the stages launched one by one (the plane kernel has no y and inverse y stage);
 // then the tile shape of the tcgen05 rebuild.
 extern "C" int vie_autotune(vie_op* op, int B, void* stream) {
   if (!op || B < 1 || B > 4096) {
@@ -540,7 +541,8 @@ extern "C" int vie_autotune(vie_op* op, int B, void* stream) {
         float total = 0.f;
         for (int rep = 0; rep < 4 && rc == VIE_OK; ++rep) {   // rep 0 warms up
           cudaEventRecord(e0, s);
-          rc = matvec_impl<float>(op, J, Y, B, VIE_PATH_TUCKER, 0, 0, nullptr, nullptr, nullptr, s);
+          rc = matvec_impl<float>(op, J, Y, B, VIE_PATH_TUCKER, 0, 0, nullptr, nullptr, nullptr, s, nullptr,
+                                  0, MV_SEPARATE);
           cudaEventRecord(e1, s);
           cudaEventSynchronize(e1);
           float ms = 0.f;

@@ -119,3 +119,15 @@ def test_stored_product_costs_no_more_than_the_rebuilt_one():
     stored, rebuilt = _time(op, J, "uncompressed"), _time(op, J)
     assert stored < rebuilt, (stored, rebuilt)
     op.close()
+
+
+def test_autotune_times_every_stage_on_plane_grids():
+    """The solver runs the separate stages, also where products take the plane kernel:
+    the tuner launches each of them for each of its candidates (3 sizes, 4 products)."""
+    op = vie.Operator((16, 16, 16), H, F, 1e-6)
+    vie.profile_start()
+    op.autotune(1)
+    ran = vie.profile_stop()
+    for f in ("line_x", "line_y", "line_iy", "line_ix"):
+        assert ran.get(f, {"launches": 0})["launches"] >= 4 * 3 * 4, (f, ran)
+    op.close()
