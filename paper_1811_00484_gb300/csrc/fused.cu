@@ -663,7 +663,7 @@ template <typename T, bool STORED>
 static int launch_fused_impl(FusedArgs<T> a, cudaStream_t s) {
   if constexpr (sizeof(T) == 4) {
     if (launch_fused_fast(a, s)) return VIE_OK;
-  } else {
+  } else if (plan_exists(a.P3)) {
     ProfScope ps(PF_MATVEC64, s);
     a.prof = nullptr;
     if (launch_plan_fused(a, 0, a.H1, s)) return VIE_OK;

@@ -131,3 +131,15 @@ def test_autotune_times_every_stage_on_plane_grids():
     for f in ("line_x", "line_y", "line_iy", "line_ix"):
         assert ran.get(f, {"launches": 0})["launches"] >= 4 * 3 * 4, (f, ran)
     op.close()
+
+
+@pytest.mark.parametrize("n", [(12, 10, 7), (12, 30, 45)])
+def test_profiler_counts_each_fp64_stage_once(n):
+    """x, y, z, inverse y, inverse x, with and without a factor plan for the z edge."""
+    op = vie.Operator(n, H, F, 1e-6)
+    J = _field(n, 2, 6, np.complex128)
+    vie.profile_start(["matvec_fp64"])
+    op.matvec(J)
+    torch.cuda.synchronize()
+    assert vie.profile_stop()["matvec_fp64"]["launches"] == 5
+    op.close()
