@@ -142,10 +142,12 @@ typedef struct vie_op_info_t {
                                     mma.sync (3xTF32) into it, 3 tensor cores
                                     through tcgen05.mma with TMEM accumulators
                                     (3xTF32) into it.  Matvecs of small grids
-                                    (y and z edges up to 24) whose planes are
-                                    all resident at once rebuild inside their
-                                    plane kernel instead, unless a rebuild was
-                                    chosen by flag                            */
+                                    (y and z edges of 8 to 24 or 28 voxels, n2 n3
+                                    <= 576) whose n1 and batch are small too
+                                    (16^3: up to 28 right-hand sides) rebuild
+                                    with FP32 FMAs inside their plane kernel
+                                    instead, unless a rebuild was chosen by
+                                    flag; solves use the rebuild named here   */
     int cp_rank;                 /* terms R of the Tucker+CP model (0: none)   */
     double cp_rel_err[6];        /* ||core - CP|| / ||core|| per component;
                                     the factors U^q are orthonormal, so this

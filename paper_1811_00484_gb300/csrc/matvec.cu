@@ -205,13 +205,13 @@ int matvec_run(const vie_op* op, void* ws, const cx<T>* in, cx<T>* out, int B, i
   const bool cp = (path == VIE_PATH_TUCKER_CP);
   LineStages<T> st = make_line_stages<T>(op, ws, in, out, B, pro_flags, epi_flags, chi,
                                          addend, active, rscale, rscale_stride);
-  // a small grid: the y and z stages and the rebuild in one launch
-  if (!cp && !(mv_flags & MV_SEPARATE) && vie::plane_eligible<T>(op, B)) {
+  // a small grid: the y and z stages and the rebuild in one launch, for every right-hand side
+  if (!cp && active == nullptr && !(mv_flags & MV_SEPARATE) && vie::plane_eligible<T>(op, B)) {
     // its CTAs have an SM each, and rebuild their planes meanwhile (8^3 in FP64: 24.5
     // us, 34.5 us when they start after the x stage)
     st.s[0].early = st.s[3].early = 1;
     launch_line_fft<T>(st.s[0], s);
-    vie::launch_plane<T>(op, st.s[0].out, B, stored, active, s);
+    vie::launch_plane<T>(op, st.s[0].out, B, stored, s);
     launch_line_fft<T>(st.s[3], s);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_status(e, "matvec launch");

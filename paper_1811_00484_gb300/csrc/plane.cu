@@ -35,7 +35,6 @@ template <typename T> struct PlaneArgs {
   int r2max, r3max;
   const cx<T>* spec;                // stored spectra (nullptr: rebuild)
   long long spec_stride;
-  const int* active;
   unsigned long long* prof;
   unsigned long long prof_rhs_bytes;
 };
@@ -119,7 +118,6 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kPerSm : 1) plane_k
   }
   pdl_trigger();
   pdl_wait();
-  if (a.active != nullptr && a.active[b] == 0) return;   // block-uniform
   if (a.prof != nullptr && kx == 0 && tid == 0) atomicAdd(a.prof, a.prof_rhs_bytes);
   const long long cs = (long long)a.P1 * n2 * n3;
   C* plane0 = a.data + (long long)b * 3 * cs + (long long)kx * n2 * n3;
@@ -263,7 +261,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kPerSm : 1) plane_k
   });
 }
 
-// line radices of a planned edge this kernel has (padded edges 16 to 48)
+// line radices of a planned edge this kernel has (padded edges 16 to 48, and 56)
 static bool radices(int N, int* q1, int* q2) {
   switch (N) {
 #define VIE_X(N, Q1, Q2, ...) \
@@ -278,15 +276,17 @@ static bool radices(int N, int* q1, int* q2) {
 
 }  // namespace plane
 
-// Small enough for the planes: y and z edges up to 24 voxels, no rebuild kernel
-// chosen by flag, and few enough planes (each CTA rebuilds its plane's entries, so
-// waves of CTAs repeat that).  Where three planes fit an SM two waves still win (16
-// x 10 x 16 with 16 right-hand sides 22 us against 42 us for the separate stages,
-// 16^3 36 against 44 us); where two do, one (20^3: 17 us against 24 us with one or
-// two right-hand sides, the same from four on); where one does, half a wave (24^3:
-// 24.8 and 24.6 us with one, 27.7 and 24.6 us with two).
+// Small enough for the planes: y and z edges of 8 to 24 or 28 voxels with P2 P3 <= 48^2,
+// no rebuild kernel chosen by flag, and few enough planes (each CTA rebuilds its
+// plane's entries, so waves of CTAs repeat that).  Where three planes fit an SM two
+// waves still win (against the separate stages: 16 x 10 x 16 with 16 right-hand sides
+// 22 against 43 us, 16^3 35 against 44, 40 x 8 x 28 with 8 38 against 38); where two do,
+// one (20^3 17 against 24 us with one or two right-hand sides, 26 against 26 with four;
+// 8 x 28 x 20 22 against 25 with one to four, 35 against 48 with 16; but 20 x 28 x 20
+// with four 34 against 28); where one does, half a wave (24^3 25 against 23 us, 12 x 24
+// x 24 22 against 25; with stored spectra 14 against 19 and 15 against 20).
 // FP64 arithmetic is so slow that few CTAs lose more than the launches cost: there
-// only up to 9 x 9 voxels (8^3: 24 us against 20 us, 8 right-hand sides 29 us against
+// only up to 9 x 9 (or 8 x 10) voxels (8^3: 24 us against 20 us, 8 right-hand sides 29 us against
 // 42 us; 12^3: 45 us against 30 us).
 template <typename T> bool plane_eligible(const vie_op* op, int B) {
   int q, z1, z2;
@@ -307,7 +307,7 @@ template <typename T> bool plane_eligible(const vie_op* op, int B) {
 }
 
 template <typename T>
-void launch_plane(const vie_op* op, cx<T>* T1, int B, bool stored, const int* active, cudaStream_t s) {
+void launch_plane(const vie_op* op, cx<T>* T1, int B, bool stored, cudaStream_t s) {
   plane::PlaneArgs<T> a = {};
   a.data = T1;
   if constexpr (sizeof(T) == 4) {
@@ -333,7 +333,6 @@ void launch_plane(const vie_op* op, cx<T>* T1, int B, bool stored, const int* ac
   a.r2max = op->rmax[1];
   a.r3max = op->rmax[2];
   a.spec_stride = (long long)a.P1 * a.P2 * a.P3;
-  a.active = active;
   const int fam = sizeof(T) == 8 ? PF_MATVEC64 : (stored ? PF_FUSED_STORED : PF_FUSED_TUCKER);
   a.prof = sizeof(T) == 8 ? nullptr : prof_bytes(fam);
   a.prof_rhs_bytes = 12ull * a.P1 * a.P2 * a.n3 * sizeof(cx<T>);     // 48 B per padded voxel
@@ -344,8 +343,8 @@ void launch_plane(const vie_op* op, cx<T>* T1, int B, bool stored, const int* ac
 
 template bool plane_eligible<float>(const vie_op*, int);
 template bool plane_eligible<double>(const vie_op*, int);
-template void launch_plane<float>(const vie_op*, float2*, int, bool, const int*, cudaStream_t);
-template void launch_plane<double>(const vie_op*, double2*, int, bool, const int*, cudaStream_t);
+template void launch_plane<float>(const vie_op*, float2*, int, bool, cudaStream_t);
+template void launch_plane<double>(const vie_op*, double2*, int, bool, cudaStream_t);
 
 }  // namespace vie
 

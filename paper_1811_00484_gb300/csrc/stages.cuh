@@ -706,7 +706,7 @@ template <typename T> bool launch_plan_line(const LineArgs<T>& a, cudaStream_t s
 // y and z stages of a small grid's planes in one launch, T1 in place (plane.cu)
 template <typename T> bool plane_eligible(const vie_op* op, int B);
 template <typename T>
-void launch_plane(const vie_op* op, cx<T>* T1, int B, bool stored, const int* active, cudaStream_t s);
+void launch_plane(const vie_op* op, cx<T>* T1, int B, bool stored, cudaStream_t s);
 template <typename T> bool launch_plan_fused(const FusedArgs<T>& a, int k10, int nk1, cudaStream_t s);
 
 }  // namespace vie
