@@ -92,7 +92,7 @@ static void launch_tw(LineArgs<T> a, size_t smem, cudaStream_t s) {
 template <typename T>
 void launch_line_fft(const LineArgs<T>& a, cudaStream_t s) {
   if constexpr (sizeof(T) == 8) {
-    if (a.plan.N == 512 && launch_line_tp64(a, s)) return;
+    if (launch_line_tp64(a, s)) return;
   }
   if (launch_plan_line(a, s)) return;
   const int N = a.plan.N;

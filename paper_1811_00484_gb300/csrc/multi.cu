@@ -5,8 +5,8 @@
 //
 // Each multi-grid kernel gets a table of per-problem arguments as a kernel
 // parameter, with the prefix sums of the problems' work-item counts; a CTA
-// finds its problem from the item index and runs the device body the
-// per-operator kernels run for that problem's FFT length P = 32 R: for a line
+// finds its problem from the item index and runs the device body of that
+// problem's FFT length P = 32 R (stages.cuh): for a line
 // item (16 adjacent columns) each of the four warps transforms four columns
 // with the four-step body (R even) or the register lane FFT (R odd), or the
 // CTA runs the shared-memory tile (R = 8); a fused item is one mirror group,
@@ -71,7 +71,7 @@ __device__ __forceinline__ void multi_line_body(const MultiLine& ml, long long b
   const int bb = (int)(t / ((long long)ntc * a.nother));
   const int R = ml.R[p];
   if (R == 8) {
-    if constexpr (RMAX >= 8) line_warp_tile<8, true>(a, ct * kLineTile, o, bb, smem);
+    if constexpr (RMAX >= 8) line_warp_tile<8>(a, ct * kLineTile, o, bb, smem);
     return;
   }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -79,12 +79,12 @@ __device__ __forceinline__ void multi_line_body(const MultiLine& ml, long long b
   if (c0 >= a.ncol) return;                           // warp-uniform; no block barrier here
   float2* xs = smem + (size_t)warp * kRegCols * fs_col_stride(4 * R);
   switch (R) {
-    case 1: line_reg_group<1, true>(a, c0, o, bb, ml.vec[p] != 0, lane); break;
-    case 2: line_fs_group<8, true>(a, c0, o, bb, lane, xs); break;
-    case 3: line_reg_group<3, true>(a, c0, o, bb, ml.vec[p] != 0, lane); break;
-    case 4: line_fs_group<16, true>(a, c0, o, bb, lane, xs); break;
-    case 5: if constexpr (RMAX >= 5) line_reg_group<5, true>(a, c0, o, bb, ml.vec[p] != 0, lane); break;
-    case 6: if constexpr (RMAX >= 6) line_fs_group<24, true>(a, c0, o, bb, lane, xs); break;
+    case 1: line_reg_group<1>(a, c0, o, bb, ml.vec[p] != 0, lane); break;
+    case 2: line_fs_group<8>(a, c0, o, bb, lane, xs); break;
+    case 3: line_reg_group<3>(a, c0, o, bb, ml.vec[p] != 0, lane); break;
+    case 4: line_fs_group<16>(a, c0, o, bb, lane, xs); break;
+    case 5: if constexpr (RMAX >= 5) line_reg_group<5>(a, c0, o, bb, ml.vec[p] != 0, lane); break;
+    case 6: if constexpr (RMAX >= 6) line_fs_group<24>(a, c0, o, bb, lane, xs); break;
     default: break;
   }
 }

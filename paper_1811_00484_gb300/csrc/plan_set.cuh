@@ -6,10 +6,16 @@
 namespace vie {
 namespace plan {
 
+// FP64 lines of length 512 have a kernel of their own (tp512.cu: 256 x 100 x 100, 14.1
+// ms a product, 14.2 ms with the planned x stages; 100 x 256 x 100 13.9 and 14.4 ms)
+static constexpr bool has_line(int N) { return sizeof(VIE_SET_T) == 4 || N != 512; }
+
 template <> bool line_set<VIE_SET_T, VIE_SET>(const LineArgs<VIE_SET_T>& a, cudaStream_t s) {
   switch (a.plan.N) {
-#define VIE_X(N, Q1, Q2, R1, R2, R3) \
-  case N: launch_plan_line<Q1, Q2>(a, s); return true;
+#define VIE_X(N, Q1, Q2, R1, R2, R3)                           \
+  case N:                                                      \
+    if constexpr (has_line(N)) launch_plan_line<Q1, Q2>(a, s); \
+    return has_line(N);
     VIE_SET_SIZES(VIE_X)
 #undef VIE_X
     default: return false;
@@ -32,7 +38,7 @@ template <> cudaError_t prepare_set<VIE_SET_T, VIE_SET>(int N) {
   switch (N) {
 #define VIE_X(N, Q1, Q2, R1, R2, R3)                                                   \
   case N:                                                                              \
-    e = prepare_plan_line<Q1, Q2>(VIE_SET_T());                                        \
+    if constexpr (has_line(N)) e = prepare_plan_line<Q1, Q2>(VIE_SET_T());             \
     return e != cudaSuccess ? e : prepare_plan_fused<R1, R2, R3>(VIE_SET_T());
     VIE_SET_SIZES(VIE_X)
 #undef VIE_X

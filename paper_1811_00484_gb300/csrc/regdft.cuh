@@ -112,7 +112,6 @@ VIE_SPLIT(24, 8, 3, true);
 VIE_SPLIT(25, 5, 5, false);
 VIE_SPLIT(27, 3, 9, false);
 VIE_SPLIT(28, 4, 7, true);
-VIE_SPLIT(30, 2, 15, true);
 VIE_SPLIT(32, 4, 8, false);
 #undef VIE_SPLIT
 

@@ -86,10 +86,10 @@ __host__ __device__ constexpr size_t line_warp_smem(int R) {
 // batch index bb and outer index o.  The CTA stages the tile in shared
 // memory (coalesced rows), each warp pulls whole columns into registers,
 // transforms them with the lane FFT and writes them back; forward transforms
-// write the bit-reversed lane layout to natural rows, inverse transforms read
-// it from natural rows.  HALF: forward from N/2 loaded points, or inverse
-// cropped to N/2 stored points.  Every thread of the block must call it.
-template <int R, bool HALF>
+// (from N/2 loaded points) write the bit-reversed lane layout to natural rows,
+// inverse transforms (cropped to N/2 stored points) read it from natural rows.
+// Every thread of the block must call it.
+template <int R>
 __device__ __forceinline__ void line_warp_tile(const LineArgs<float>& a, int c0, int o, int bb,
                                                float2* smem) {
   using C = float2;
@@ -103,22 +103,12 @@ __device__ __forceinline__ void line_warp_tile(const LineArgs<float>& a, int c0,
   for (int m = tid; m < N; m += nth) roots[m] = a.roots[m];
   pdl_trigger();
   pdl_wait();
-  if (a.active != nullptr && a.active[bb / a.batch_per_rhs] == 0) return;   // block-uniform
   if (a.prof != nullptr && c0 == 0 && o == 0 && tid == 0) atomicAdd(a.prof, a.prof_batch_bytes);
   const int ncols = min(TW, a.ncol - c0);
-  const float rs = (a.flags & (PRO_RSCALE | EPI_RSCALE))
-                       ? (float)a.rscale[(long long)(bb / a.batch_per_rhs) * a.rscale_stride]
-                       : 1.f;
   const C* in = a.in + bb * a.in_bs + o * a.in_os + (long long)c0;
   for (int e = tid; e < a.lin * TW; e += nth) {
     const int c = e % TW, p = e / TW;
-    if (c < ncols) {
-      C v = in[p * a.in_ls + c];
-      if (a.flags & PRO_RSCALE) v = rs * v;
-      if (a.flags & PRO_CONJ) v = conjg(v);
-      if (a.flags & PRO_CHI) v = a.chi[o * a.chi_os + p * a.chi_ls + (long long)(c0 + c)] * v;
-      tile[tile_slot(p, c)] = v;
-    }
+    if (c < ncols) tile[tile_slot(p, c)] = in[p * a.in_ls + c];
   }
   __syncthreads();
 
@@ -129,11 +119,11 @@ __device__ __forceinline__ void line_warp_tile(const LineArgs<float>& a, int c0,
     C v[R];
     if (!a.inverse) {
 #pragma unroll
-      for (int j = 0; j < (HALF ? (R + 1) / 2 : R); ++j) {
+      for (int j = 0; j < (R + 1) / 2; ++j) {
         const int p = lane + 32 * j;
         v[j] = p < a.lin ? tile[tile_slot(p, c)] : make_float2(0.f, 0.f);
       }
-      warp_fft_fwd<C, float, R, HALF>(v, lc, roots, N);
+      warp_fft_fwd<C, float, R>(v, lc, roots, N);
 #pragma unroll
       for (int k1 = 0; k1 < R; ++k1) {
         const int p = k1 + R * br;
@@ -142,9 +132,9 @@ __device__ __forceinline__ void line_warp_tile(const LineArgs<float>& a, int c0,
     } else {
 #pragma unroll
       for (int k1 = 0; k1 < R; ++k1) v[k1] = tile[tile_slot(k1 + R * br, c)];
-      warp_fft_inv<C, float, R, HALF>(v, lane, lc, roots, N);
+      warp_fft_inv<C, float, R>(v, lane, lc, roots, N);
 #pragma unroll
-      for (int j = 0; j < (HALF ? (R + 1) / 2 : R); ++j) {
+      for (int j = 0; j < (R + 1) / 2; ++j) {
         const int p = lane + 32 * j;
         if (p < a.lout) tile[tile_slot(p, c)] = v[j];
       }
@@ -152,21 +142,10 @@ __device__ __forceinline__ void line_warp_tile(const LineArgs<float>& a, int c0,
   }
   __syncthreads();
 
-  const long long obase = bb * a.out_bs + o * a.out_os + (long long)c0;
-  C* out = a.out + obase;
+  C* out = a.out + bb * a.out_bs + o * a.out_os + (long long)c0;
   for (int e = tid; e < a.lout * TW; e += nth) {
     const int c = e % TW, p = e / TW;
-    if (c >= ncols) continue;
-    C v = a.scale * tile[tile_slot(p, c)];
-    if (a.flags & EPI_CONJ) v = conjg(v);
-    const long long oi = p * a.out_ls + c;
-    if (a.flags & (EPI_SUB | EPI_ADD)) {
-      if (a.flags & EPI_CHI) v = a.chi[o * a.chi_os + p * a.chi_ls + (long long)(c0 + c)] * v;
-      C w = a.addend[obase + oi];
-      if (a.flags & EPI_RSCALE) w = rs * w;
-      v = (a.flags & EPI_SUB) ? (w - v) : (w + v);
-    }
-    out[oi] = v;
+    if (c < ncols) out[p * a.out_ls + c] = a.scale * tile[tile_slot(p, c)];
   }
 }
 
@@ -180,27 +159,23 @@ constexpr int kRegCols = 4;
 // k1 + R brev5(l) (the lane FFT's bit-reversed order) on the frequency side.
 // Each row access moves the group's 32 contiguous bytes, two 16-byte accesses
 // when `vec` (the caller has checked that every row of the group starts on a
-// 16-byte boundary), one 8-byte access per column otherwise.  HALF: forward
-// from N/2 loaded points, or inverse cropped to N/2 stored points.
-template <int R, bool HALF>
+// 16-byte boundary), one 8-byte access per column otherwise.  Forward from N/2
+// loaded points, inverse cropped to N/2 stored points.
+template <int R>
 __device__ __forceinline__ void line_reg_group(const LineArgs<float>& a, int c0, int o, int bb,
                                                bool vec, int lane) {
   using C = float2;
   constexpr int N = 32 * R;
   constexpr int NC = kRegCols;
-  constexpr int NH = HALF ? (R + 1) / 2 : R;     // natural-order rows held per lane
+  constexpr int NH = (R + 1) / 2;                // natural-order rows held per lane
   // prologue (tables only), then the preceding kernel's results
   LaneConsts<C, float, R> lc;
   lc.init(lane, a.roots, N);
   pdl_trigger();
   pdl_wait();
-  if (a.active != nullptr && a.active[bb / a.batch_per_rhs] == 0) return;   // warp-uniform
   if (a.prof != nullptr && c0 == 0 && o == 0 && lane == 0) atomicAdd(a.prof, a.prof_batch_bytes);
   const int ncols = min(NC, a.ncol - c0);
   const bool v4 = vec && ncols == NC;
-  const float rs = (a.flags & (PRO_RSCALE | EPI_RSCALE))
-                       ? (float)a.rscale[(long long)(bb / a.batch_per_rhs) * a.rscale_stride]
-                       : 1.f;
   const int br = brev5(lane);
   C v[NC][R];
   const C* in = a.in + bb * a.in_bs + o * a.in_os + (long long)c0;
@@ -219,21 +194,6 @@ __device__ __forceinline__ void line_reg_group(const LineArgs<float>& a, int c0,
       for (int c = 0; c < NC; ++c) v[c][j] = c < ncols ? src[c] : make_float2(0.f, 0.f);
     }
   };
-  // kRegCols values of an array laid out like a row of the group (chi, addend)
-  auto load4 = [&](const C* src, bool wide, C* x) {
-    if (wide) {
-      const float4 x0 = *reinterpret_cast<const float4*>(src);
-      const float4 x1 = *reinterpret_cast<const float4*>(src + 2);
-      x[0] = make_float2(x0.x, x0.y);
-      x[1] = make_float2(x0.z, x0.w);
-      x[2] = make_float2(x1.x, x1.y);
-      x[3] = make_float2(x1.z, x1.w);
-    } else {
-#pragma unroll
-      for (int c = 0; c < NC; ++c) x[c] = c < ncols ? src[c] : make_float2(0.f, 0.f);
-    }
-  };
-  const bool chi4 = v4 && a.chi_vec;
   auto store_row = [&](int p, int j) {
     C* dst = out + (long long)p * a.out_ls;
     if (v4) {
@@ -251,25 +211,13 @@ __device__ __forceinline__ void line_reg_group(const LineArgs<float>& a, int c0,
       const int p = lane + 32 * j;
       if (p < a.lin) {
         load_row(p, j);
-        if (a.flags & (PRO_RSCALE | PRO_CONJ | PRO_CHI)) {
-          C ch[NC];
-          if (a.flags & PRO_CHI) load4(a.chi + o * a.chi_os + (long long)p * a.chi_ls + c0, chi4, ch);
-#pragma unroll
-          for (int c = 0; c < NC; ++c) {
-            C x = v[c][j];
-            if (a.flags & PRO_RSCALE) x = rs * x;
-            if (a.flags & PRO_CONJ) x = conjg(x);
-            if (a.flags & PRO_CHI) x = ch[c] * x;
-            v[c][j] = x;
-          }
-        }
       } else {
 #pragma unroll
         for (int c = 0; c < NC; ++c) v[c][j] = make_float2(0.f, 0.f);
       }
     }
 #pragma unroll
-    for (int c = 0; c < NC; ++c) warp_fft_fwd<C, float, R, HALF>(v[c], lc, a.roots, N);
+    for (int c = 0; c < NC; ++c) warp_fft_fwd<C, float, R>(v[c], lc, a.roots, N);
 #pragma unroll
     for (int k1 = 0; k1 < R; ++k1) {
       const int p = k1 + R * br;
@@ -279,34 +227,13 @@ __device__ __forceinline__ void line_reg_group(const LineArgs<float>& a, int c0,
 #pragma unroll
     for (int k1 = 0; k1 < R; ++k1) load_row(k1 + R * br, k1);
 #pragma unroll
-    for (int c = 0; c < NC; ++c) warp_fft_inv<C, float, R, HALF>(v[c], lane, lc, a.roots, N);
+    for (int c = 0; c < NC; ++c) warp_fft_inv<C, float, R>(v[c], lane, lc, a.roots, N);
 #pragma unroll
     for (int j = 0; j < NH; ++j) {
       const int p = lane + 32 * j;
       if (p < a.lout) {
-        if (a.flags & (EPI_CONJ | EPI_SUB | EPI_ADD)) {
-          C ch[NC], ad[NC];
-          if (a.flags & (EPI_SUB | EPI_ADD)) {
-            if (a.flags & EPI_CHI) load4(a.chi + o * a.chi_os + (long long)p * a.chi_ls + c0, chi4, ch);
-            load4(a.addend + bb * a.out_bs + o * a.out_os + (long long)c0 + (long long)p * a.out_ls,
-                  v4 && a.addend_vec, ad);
-          }
 #pragma unroll
-          for (int c = 0; c < NC; ++c) {
-            C x = a.scale * v[c][j];
-            if (a.flags & EPI_CONJ) x = conjg(x);
-            if (a.flags & (EPI_SUB | EPI_ADD)) {
-              if (a.flags & EPI_CHI) x = ch[c] * x;
-              C w = ad[c];
-              if (a.flags & EPI_RSCALE) w = rs * w;
-              x = (a.flags & EPI_SUB) ? (w - x) : (w + x);
-            }
-            v[c][j] = x;
-          }
-        } else {
-#pragma unroll
-          for (int c = 0; c < NC; ++c) v[c][j] = a.scale * v[c][j];
-        }
+        for (int c = 0; c < NC; ++c) v[c][j] = a.scale * v[c][j];
         store_row(p, j);
       }
     }
@@ -322,8 +249,8 @@ __device__ __forceinline__ void line_reg_group(const LineArgs<float>& a, int c0,
 //          X[k1 + V k2], k2 < 8.
 // The inverse runs the same steps with conjugate roots (unscaled).  For a
 // fixed register index the warp's 32 lanes touch 8 rows x 4 columns, i.e.
-// whole 32-byte sectors.  No shuffles.  HALF: forward from x[n < N/2] (m < V/2
-// nonzero), or inverse cropped to n < N/2 (k2 < 4).
+// whole 32-byte sectors.  No shuffles.  Forward from x[n < N/2] (m < V/2
+// nonzero), inverse cropped to n < N/2 (k2 < 4).
 // Exchange layout per warp: [c][j][k1], row stride V+1, column stride
 // 8(V+1)+4 (both passes conflict-free within each half-warp).
 __host__ __device__ constexpr int fs_col_stride(int V) { return 8 * (V + 1) + 4; }
@@ -331,7 +258,7 @@ __host__ __device__ constexpr size_t line_fs_smem(int V, int warps) {
   return (size_t)warps * kRegCols * fs_col_stride(V) * sizeof(float2);
 }
 
-template <int V, bool HALF>
+template <int V>
 __device__ __forceinline__ void line_fs_group(const LineArgs<float>& a, int c0, int o, int bb,
                                               int lane, float2* xs) {
   using C = float2;
@@ -341,30 +268,19 @@ __device__ __forceinline__ void line_fs_group(const LineArgs<float>& a, int c0, 
   C* xc = xs + c * S;
   pdl_trigger();
   pdl_wait();
-  if (a.active != nullptr && a.active[bb / a.batch_per_rhs] == 0) return;   // warp-uniform
   if (a.prof != nullptr && c0 == 0 && o == 0 && lane == 0) atomicAdd(a.prof, a.prof_batch_bytes);
   const bool col_ok = c0 + c < a.ncol;
-  const float rs = (a.flags & (PRO_RSCALE | EPI_RSCALE))
-                       ? (float)a.rscale[(long long)(bb / a.batch_per_rhs) * a.rscale_stride]
-                       : 1.f;
   const C* in = a.in + bb * a.in_bs + o * a.in_os + (long long)(c0 + c);
   C* out = a.out + bb * a.out_bs + o * a.out_os + (long long)(c0 + c);
   const bool inv = a.inverse != 0;
   C v[V];
   // pass 1: rows j + 8 m
-  constexpr int M1 = HALF ? V / 2 : V;         // forward: rows loaded (the rest is padding)
+  constexpr int M1 = V / 2;                    // forward: rows loaded (the rest is padding)
 #pragma unroll
   for (int m = 0; m < V; ++m) {
     const int p = j + 8 * m;
     C x = make_float2(0.f, 0.f);
-    if ((inv || m < M1) && col_ok && p < a.lin) {
-      x = in[(long long)p * a.in_ls];
-      if (!inv) {
-        if (a.flags & PRO_RSCALE) x = rs * x;
-        if (a.flags & PRO_CONJ) x = conjg(x);
-        if (a.flags & PRO_CHI) x = a.chi[o * a.chi_os + (long long)p * a.chi_ls + (long long)(c0 + c)] * x;
-      }
-    }
+    if ((inv || m < M1) && col_ok && p < a.lin) x = in[(long long)p * a.in_ls];
     v[m] = x;
   }
   if (!inv) {
@@ -382,7 +298,6 @@ __device__ __forceinline__ void line_fs_group(const LineArgs<float>& a, int c0, 
   for (int k1 = 0; k1 < V; ++k1) xc[j * (V + 1) + k1] = v[k1];
   __syncwarp();
   // pass 2: k1 = j + 8 t, DFT over the eight j
-  constexpr int K2 = (HALF ? 4 : 8);           // inverse: outputs kept (cropped to N/2)
 #pragma unroll
   for (int t = 0; t < V / 8; ++t) {
     const int k1 = j + 8 * t;
@@ -392,22 +307,10 @@ __device__ __forceinline__ void line_fs_group(const LineArgs<float>& a, int c0, 
     reg_dft<C, float, 8>(u, a.roots, N, inv);
 #pragma unroll
     for (int k2 = 0; k2 < 8; ++k2) {
-      if (inv && k2 >= K2) continue;
+      if (inv && k2 >= 4) continue;              // cropped to N/2
       const int p = k1 + V * k2;
       if (!col_ok || p >= a.lout) continue;
-      C x = u[k2];
-      if (inv) {
-        x = a.scale * x;
-        if (a.flags & EPI_CONJ) x = conjg(x);
-        if (a.flags & (EPI_SUB | EPI_ADD)) {
-          if (a.flags & EPI_CHI)
-            x = a.chi[o * a.chi_os + (long long)p * a.chi_ls + (long long)(c0 + c)] * x;
-          C w = a.addend[bb * a.out_bs + o * a.out_os + (long long)(c0 + c) + (long long)p * a.out_ls];
-          if (a.flags & EPI_RSCALE) w = rs * w;
-          x = (a.flags & EPI_SUB) ? (w - x) : (w + x);
-        }
-      }
-      out[(long long)p * a.out_ls] = x;
+      out[(long long)p * a.out_ls] = inv ? a.scale * u[k2] : u[k2];
     }
   }
 }
@@ -425,7 +328,7 @@ __host__ __device__ constexpr size_t fused_warp_smem(int R, int H3, int r2max, i
 // One (k1, k2) mirror group of the fused stage on the register path (P3 = 32 R):
 // the four warps of the CTA take one mirror z-line each, hold the three
 // components of every right-hand side in registers, and do the forward lane
-// FFT, the voxel-wise product with the rebuilt (or stored) components in the
+// FFT, the voxel-wise product with the rebuilt components in the
 // bit-reversed lane layout, and the inverse lane FFT.  The rebuild of the
 // half fibre (k3 <= P3/2) is shared by the CTA.  Every thread must call it.
 template <int R>
@@ -479,16 +382,9 @@ __device__ __forceinline__ void fused_warp_group(const FusedArgs<float>& a, int 
   pdl_trigger();
   pdl_wait();
 
-  if (a.prof != nullptr && g == 0 && tid == 0) {
-    unsigned long long nb = 0;
-    for (int b = 0; b < a.B; ++b) nb += (a.active == nullptr || a.active[b]) ? 1 : 0;
-    atomicAdd(a.prof, nb * a.prof_rhs_bytes + a.prof_launch_bytes);
-  }
-  // the first active right-hand side's lines are loaded before the half fibres
-  // are copied, so the two latencies overlap
-  int b0 = 0;
-  if (a.active != nullptr)
-    while (b0 < a.B && a.active[b0] == 0) ++b0;
+  if (a.prof != nullptr && g == 0 && tid == 0) atomicAdd(a.prof, a.B * a.prof_rhs_bytes + a.prof_launch_bytes);
+  // the first right-hand side's lines are loaded before the half fibres are copied,
+  // so the two latencies overlap
   C v[3][R];
   auto load_lines = [&](int b) {
 #pragma unroll
@@ -501,7 +397,7 @@ __device__ __forceinline__ void fused_warp_group(const FusedArgs<float>& a, int 
       }
     }
   };
-  if (has_line && b0 < a.B) load_lines(b0);
+  if (has_line) load_lines(0);
   if (!rebuild_here) {
     // the group's half fibres, rebuilt for this matvec into the scratch
     const C* src = a.octant + ((long long)(k1 - a.oct_k1a) * a.H2 + k2) * 6 * H3;
@@ -520,11 +416,10 @@ __device__ __forceinline__ void fused_warp_group(const FusedArgs<float>& a, int 
   // s_a s_b times its half-fibre value, s_q = -1 along each mirrored axis, so
   // Y = D G D J with D = diag(s_x, s_y, s_z)
   const float sx = ix ? -1.f : 1.f, sy = iy ? -1.f : 1.f;
-  for (int b = b0; b < a.B; ++b) {
-    if (a.active != nullptr && a.active[b] == 0) continue;   // warp-uniform
-    if (b != b0) load_lines(b);
+  for (int b = 0; b < a.B; ++b) {
+    if (b != 0) load_lines(b);
 #pragma unroll
-    for (int comp = 0; comp < 3; ++comp) warp_fft_fwd<C, float, R, true>(v[comp], lc, roots, P3);
+    for (int comp = 0; comp < 3; ++comp) warp_fft_fwd<C, float, R>(v[comp], lc, roots, P3);
 #pragma unroll
     for (int q = 0; q < R; ++q) {
       const int kk = q + R * br;                       // z-frequency held in register q
@@ -549,7 +444,7 @@ __device__ __forceinline__ void fused_warp_group(const FusedArgs<float>& a, int 
     }
 #pragma unroll
     for (int comp = 0; comp < 3; ++comp) {
-      warp_fft_inv<C, float, R, true>(v[comp], lane, lc, roots, P3);
+      warp_fft_inv<C, float, R>(v[comp], lane, lc, roots, P3);
       C* dst = a.data + (long long)(b * 3 + comp) * a.comp_stride + line_off;
 #pragma unroll
       for (int j = 0; j < NLOAD; ++j) {
@@ -566,8 +461,8 @@ __device__ __forceinline__ void fused_warp_group(const FusedArgs<float>& a, int 
 //   forward: pass 1 / exchange / pass 2 as in line_fs_group, then the
 //            component's spectrum goes to a shared buffer spec[comp][l][f];
 //   product: each lane forms Y_comp[l][f] = s_comp sum_b G_comp,b[fold f] s_b J_b[l][f]
-//            (D G D, with G the rebuilt half fibre, or the stored spectra) for
-//            the frequencies f = j + 8 m its inverse pass 1 needs;
+//            (D G D, with G the rebuilt half fibre) for the frequencies f = j + 8 m
+//            its inverse pass 1 needs;
 //   inverse: pass 1 / exchange / pass 2 cropped to n3 outputs, written in place.
 // Every thread must call it.
 __host__ __device__ constexpr int fused_fs_spec_stride(int V) { return 8 * V + 4; }
@@ -602,11 +497,7 @@ __device__ __forceinline__ void fused_fs_group(const FusedArgs<float>& a, int g,
   C* xc = xw + ln * XS;
   pdl_trigger();
   pdl_wait();
-  if (a.prof != nullptr && g == 0 && tid == 0) {
-    unsigned long long nb = 0;
-    for (int b = 0; b < a.B; ++b) nb += (a.active == nullptr || a.active[b]) ? 1 : 0;
-    atomicAdd(a.prof, nb * a.prof_rhs_bytes + a.prof_launch_bytes);
-  }
+  if (a.prof != nullptr && g == 0 && tid == 0) atomicAdd(a.prof, a.B * a.prof_rhs_bytes + a.prof_launch_bytes);
   {
     // the group's half fibres, rebuilt for this matvec into the scratch
     const C* src = a.octant + ((long long)(k1 - a.oct_k1a) * a.H2 + k2) * 6 * H3;
@@ -623,7 +514,6 @@ __device__ __forceinline__ void fused_fs_group(const FusedArgs<float>& a, int g,
   const float sc = comp == 0 ? sx : (comp == 1 ? sy : 1.f);
   __syncthreads();
   for (int b = 0; b < a.B; ++b) {
-    if (a.active != nullptr && a.active[b] == 0) continue;   // block-uniform
     C* line = a.data + (long long)(b * 3 + (act ? comp : 0)) * a.comp_stride + line_off;
     C v[V];
     if (act) {

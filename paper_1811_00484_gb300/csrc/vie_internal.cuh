@@ -145,7 +145,6 @@ template <typename T> struct LineArgs {
   long long in_bs, in_os, in_ls, in_cs;
   long long out_bs, out_os, out_ls, out_cs;
   long long chi_os, chi_ls, chi_cs;    // chi index = o*chi_os + p*chi_ls + c*chi_cs
-  int chi_vec, addend_vec;             // chi / addend rows allow 16-byte accesses
   int batch_per_rhs;                   // batches per RHS (3 components) for `active`
   const int* active;                   // per-RHS flag (nullptr = all active)
   int early;                           // the next kernel may start beside this one
@@ -153,7 +152,6 @@ template <typename T> struct LineArgs {
   int prof_family;                     // profiler family of this launch
   unsigned long long* prof;            // profiler byte counter (nullptr = off)
   unsigned long long prof_batch_bytes; // algorithmic bytes per active batch index
-  int* err;                            // device word set when a bounded wait gives up (or nullptr)
 };
 
 template <typename T> void launch_line_fft(const LineArgs<T>& a, cudaStream_t s);

@@ -84,13 +84,10 @@ template <typename C, typename T, int R1, int R2> struct RegDftSplit {
   }
 };
 template <typename C, typename T> struct RegDft<C, T, 6> : RegDftSplit<C, T, 2, 3> {};
-template <typename C, typename T> struct RegDft<C, T, 10> : RegDftSplit<C, T, 2, 5> {};
-template <typename C, typename T> struct RegDft<C, T, 12> : RegDftSplit<C, T, 4, 3> {};
 template <typename C, typename T> struct RegDft<C, T, 16> {
   static __device__ __forceinline__ void run(C* v, const C*, int, bool inv) { dft16<C, T>(v, inv); }
 };
 template <typename C, typename T> struct RegDft<C, T, 24> : RegDftSplit<C, T, 3, 8> {};
-template <typename C, typename T> struct RegDft<C, T, 32> : RegDftSplit<C, T, 4, 8> {};
 
 // Per-lane constants of the lane transforms, computed once per kernel:
 //   tw[k1]  = w_N^{lane k1}                       (twiddle between the stages)
@@ -124,16 +121,14 @@ template <typename C, typename T, int R> struct LaneConsts {
 };
 
 // forward: v[j] = x[lane + 32 j]  ->  v[k1] = X[k1 + R brev5(lane)].
-// HALF: only x[0 .. N/2) can be nonzero (zero-padded input): v[j] for
-// j >= (R+1)/2 (points lane + 32 j >= N/2 + 16) is set to zero here, so the
-// caller only loads j < (R+1)/2.
-template <typename C, typename T, int R, bool HALF = false>
+// Only x[0 .. N/2) can be nonzero (zero-padded input): v[j] for j >= (R+1)/2
+// (points lane + 32 j >= N/2 + 16) is set to zero here, so the caller only
+// loads j < (R+1)/2.
+template <typename C, typename T, int R>
 __device__ __forceinline__ void warp_fft_fwd(C* v, const LaneConsts<C, T, R>& lc, const C* roots,
                                              int N) {
-  if (HALF) {
 #pragma unroll
-    for (int j = (R + 1) / 2; j < R; ++j) v[j] = mk((T)0, (T)0);
-  }
+  for (int j = (R + 1) / 2; j < R; ++j) v[j] = mk((T)0, (T)0);
   reg_dft<C, T, R>(v, roots, N, false);
 #pragma unroll
   for (int k1 = 1; k1 < R; ++k1) v[k1] = v[k1] * lc.tw[k1];
@@ -153,9 +148,8 @@ __device__ __forceinline__ void warp_fft_fwd(C* v, const LaneConsts<C, T, R>& lc
 }
 
 // inverse (unscaled): v[k1] = X[k1 + R brev5(lane)]  ->  v[j] = N x[lane + 32 j].
-// HALF: only x[0 .. N/2) is wanted (cropped output): the caller stores only
-// j < (R+1)/2.
-template <typename C, typename T, int R, bool HALF = false>
+// Only x[0 .. N/2) is wanted (cropped output): the caller stores only j < (R+1)/2.
+template <typename C, typename T, int R>
 __device__ __forceinline__ void warp_fft_inv(C* v, int lane, const LaneConsts<C, T, R>& lc,
                                              const C* roots, int N) {
 #pragma unroll
@@ -175,7 +169,6 @@ __device__ __forceinline__ void warp_fft_inv(C* v, int lane, const LaneConsts<C,
 #pragma unroll
   for (int k1 = 1; k1 < R; ++k1) v[k1] = v[k1] * conjg(lc.tw[k1]);
   reg_dft<C, T, R>(v, roots, N, true);
-  (void)HALF;
 }
 
 // radices handled by the register path (N = 32 R <= 512)
