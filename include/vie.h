@@ -125,8 +125,11 @@ typedef struct vie_op_info_t {
                                     every matvec)                               */
     size_t rebuild_scratch_bytes;/* c64 scratch into which every Tucker matvec
                                     rebuilds the half fibres of a chunk of k1
-                                    (at most 64 MiB; 0 when the grid takes the
-                                    shared-memory path, which rebuilds on chip) */
+                                    (at most 64 MiB; held by every operator with
+                                    2 n3 from 16 to 512 but 490, 10 MiB at 50 x
+                                    72 x 60, unless its ranks are too large for
+                                    the rebuild kernels; otherwise 0, and the
+                                    z stage rebuilds on chip)                  */
     size_t uncompressed_bytes;   /* six c64 spectra, 6 P1 P2 P3 x 8 bytes       */
     size_t workspace_bytes;      /* scratch currently held                      */
     int has_uncompressed;        /* VIE_STORE_UNCOMPRESSED was given            */
@@ -335,9 +338,10 @@ int vie_matvec_multi(const vie_op* const* ops, const void* const* J,
                      void* const* Y, const int* B, int count, void* stream);
 
 /*
- * Pick the CTA size (64, 128 or 256 threads) of each register-path FFT
- * stage of `op` by timing FP32 Tucker matvecs at batch B on `stream`, and
- * keep the fastest; then, for the tcgen05 rebuild (rebuild_kernel 3), the
+ * Pick the CTA size (at most 64, 128 or 256 threads) of each line FFT stage of
+ * `op` by timing FP32 Tucker matvecs at batch B on `stream`, and keep the
+ * fastest (on grids whose products take the plane kernel: of the separate
+ * stages, which solves and larger batches run); then, for the tcgen05 rebuild (rebuild_kernel 3), the
  * tile shape of the rebuild of eq. (13) (k3 columns per CTA and CTAs per
  * component), timed over every k1 chunk of one matvec.  vie_op_info reports
  * the choices.  Allocates two temporary batches; synchronises `stream`.

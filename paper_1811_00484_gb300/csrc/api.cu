@@ -56,18 +56,6 @@ int device_sms() {
   return sms;
 }
 
-int persistent_grid(const void* kernel, int threads, size_t smem, long long work) {
-  const int sms = device_sms();
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem) != cudaSuccess ||
-      per_sm <= 0) {
-    cudaGetLastError();
-    per_sm = 1;
-  }
-  const long long g = (long long)per_sm * sms;
-  return (int)(work < g ? (work > 0 ? work : 1) : g);
-}
-
 int check_grid(const vie_grid* g) {
   if (!g) { set_error("grid is NULL"); return VIE_ERR_ARG; }
   const int n[3] = {g->n1, g->n2, g->n3};

@@ -896,9 +896,8 @@ static int arnoldi_step(const vie_op* op, SolverState* st, const float2* chi, in
   const size_t flag_bytes = (size_t)B * sizeof(int);
   // The matvec skips right-hand sides by a copy of the active flags taken
   // before the previous step's Givens step was forked: that step may retire a
-  // right-hand side while the matvec runs, and every thread of every stage
-  // (the producer and consumers of a persistent kernel alike) must take the
-  // same decision for it.  A right-hand side retired meanwhile is still
+  // right-hand side while the matvec runs, and every thread of every stage must
+  // take the same decision for it.  A right-hand side retired meanwhile is still
   // multiplied; its output is never read.
   if (k == 0)
     VIE_CUDA(cudaMemcpyAsync(st->mv_active, st->active, flag_bytes, cudaMemcpyDeviceToDevice, s));
@@ -1052,7 +1051,7 @@ static int check_device_error(const vie_op* op, cudaStream_t s) {
   VIE_CUDA(cudaStreamSynchronize(s));
   if (h != 0) {
     VIE_CUDA(cudaMemsetAsync(op->dev_err, 0, sizeof(int), s));
-    set_error("a bounded device wait gave up (an asynchronous copy did not complete)");
+    set_error("a bounded device wait gave up (the tcgen05 rebuild's or the multi-grid barrier's)");
     return VIE_ERR_TIMEOUT;
   }
   return VIE_OK;

@@ -359,10 +359,7 @@ int plane_init_attributes();
 int plan_prepare(int N);     // kernel attributes of padded edge N (plan.cu)
 int op_tables(vie_op* op);   // FFT plans and root tables of op->P
 int line_fft_init_attributes();
-// persistent grid size for `kernel` with `threads` threads and `smem` bytes of
-// dynamic shared memory: resident CTAs per SM x SMs, capped by `work`
 int device_sms();
-int persistent_grid(const void* kernel, int threads, size_t smem, long long work);
 int fused_init_attributes();
 int multi_init_attributes();
 int tp_init_attributes();
