@@ -926,7 +926,15 @@ static int finish_operator(vie_op* op) {
     constexpr size_t kOctBudget = 64u << 20;
     const size_t plane = (size_t)op->H[1] * 6 * op->H[2] * sizeof(float2);
     op->oct_k1 = (int)std::max<size_t>(1, std::min<size_t>(op->H[0], kOctBudget / plane));
-    VIE_TRY(dalloc(&op->oct32, (size_t)op->oct_k1 * plane));
+    const int st = dalloc(&op->oct32, (size_t)op->oct_k1 * plane);
+    if (st != VIE_OK && lane_fft_edge(op->P[2])) return st;
+    if (st != VIE_OK) {                    // the z stage of other edges does without
+      clear_error();
+      op->oct32 = nullptr;
+      op->oct_k1 = 0;
+    }
+  }
+  if (op->oct32 != nullptr) {
     VIE_CUDA(cudaStreamCreateWithFlags(&op->rb_stream, cudaStreamNonBlocking));
     VIE_CUDA(cudaEventCreateWithFlags(&op->rb_fork, cudaEventDisableTiming));
     VIE_CUDA(cudaEventCreateWithFlags(&op->rb_join, cudaEventDisableTiming));
