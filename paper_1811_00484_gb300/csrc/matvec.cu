@@ -216,6 +216,11 @@ int matvec_run(const vie_op* op, void* ws, const cx<T>* in, cx<T>* out, int B, i
     if (e != cudaSuccess) return cuda_status(e, "matvec launch");
     return VIE_OK;
   }
+  // in a solve's captured restart cycle the z stage starts early on every grid: there
+  // the smallest lose more without (an Arnoldi step of 20^3 33 us, 45 without; 16^3
+  // with four right-hand sides 42 and 52) than the next ones gain (24^3 with four 69
+  // and 56 with stored spectra, 60 and 60 with rebuilt ones)
+  if (sizeof(T) == 4 && (mv_flags & MV_SEPARATE)) st.s[1].early = 1;
   C* T2 = const_cast<C*>(st.s[1].out);
   // FP32 Tucker path on the register kernels: the first k1 chunk of the rebuild
   // does not read J, so it runs on the operator's side stream beside the x and

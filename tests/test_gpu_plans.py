@@ -1,6 +1,8 @@
 """The planned matvec stages (factor plans of the padded edges, plan_table.h) against
 the oracle's FFT matvec: every radix pair class, odd and even edges, columns that are
 no multiple of a tile, batches, masks of the mirror groups at thin edges."""
+import time
+
 import numpy as np
 import pytest
 import torch
@@ -143,3 +145,26 @@ def test_profiler_counts_each_fp64_stage_once(n):
     torch.cuda.synchronize()
     assert vie.profile_stop()["matvec_fp64"]["launches"] == 5
     op.close()
+
+
+def test_arnoldi_step_of_a_smaller_grid_costs_no_more():
+    """One right-hand side, 200 steps in captured cycles: 16^3 and 20^3 against 24^3."""
+    best = {}
+    for m in (16, 20, 24):
+        n = (m, m, m)
+        op = vie.Operator(n, H, F, 1e-6)
+        g = torch.Generator(device="cuda")
+        g.manual_seed(1)
+        chi = 5 * torch.randn(n, dtype=torch.complex64, device="cuda", generator=g)
+        rhs = torch.randn((1, 3) + n, dtype=torch.complex64, device="cuda", generator=g)
+        best[m] = float("inf")
+        for _ in range(6):
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            _, info = op.solve(chi, rhs, incident=False, tol=1e-13, max_outer=4, refine=False,
+                               raise_on_failure=False)
+            torch.cuda.synchronize()
+            best[m] = min(best[m], time.perf_counter() - t0)
+        assert info["iterations"] >= 200
+        op.close()
+    assert best[16] < 1.1 * best[24] and best[20] < 1.1 * best[24], best
